@@ -67,7 +67,7 @@ __device__ __forceinline__ Dual& operator-=(Dual& a, Dual b) {
   a = a - b;
   return a;
 }
-__device__ __forceinline__ Dual dexp(Dual a, const double* tab) {
+__device__ __forceinline__ Dual dexp(Dual a, const uint64_t* tab) {
   const double e = exp_fast(a.v, tab);
   return Dual{e, e * a.t};
 }
@@ -178,7 +178,7 @@ __device__ __forceinline__ void put(Dual& d, double a) { d.v = a; }
 __device__ __forceinline__ void put(Dual& d, Dual a) { d = a; }
 __device__ __forceinline__ double val(double a) { return a; }
 __device__ __forceinline__ double val(Dual a) { return a.v; }
-__device__ __forceinline__ double dexp(double a, const double* tab) { return exp_fast(a, tab); }
+__device__ __forceinline__ double dexp(double a, const uint64_t* tab) { return exp_fast(a, tab); }
 __device__ __forceinline__ double dlog(double a) { return log(a); }
 __device__ __forceinline__ double dlog10(double a) { return log10(a); }
 // the ln A gradient contribution: the value, or (tangent passes) the tangent

@@ -44,6 +44,7 @@
 #include <string>
 
 #include "exp2_table.h"
+#include "fx.cuh"
 #include "internal.h"
 #include "rok4e.h"
 
@@ -67,97 +68,54 @@ constexpr double BH1 = -0.217819895945721, BH2 = 1.03130847478467, BH3 = 0.18651
 constexpr double PI_ALPHA = 0.7 / 4.0, PI_BETA = 0.4 / 4.0;
 constexpr double FAC_MIN = 0.2, FAC_MAX = 5.0, SAFETY = 0.8, ERR_FLOOR = 1e-10;
 constexpr double BREAKDOWN_TOL = 1e-12, T_END_TOL = 1e-12, H_MIN_FRAC = 1e-12;
+#ifndef RK_UNROLL
+#define RK_UNROLL 2
+#endif
 constexpr int G_OVERFLOW_HI = 0x40654000;  // high word of 170.0
 constexpr int MAXM = RK_MAX_KRYLOV;
 // Threads per block of the per-cell kernels: 8 warps, so each thread may hold
 // up to 255 registers (one such block fills an SM's register file, which the
 // cells' shared-memory slots limit the SM to anyway).
 constexpr int MAX_BLOCK_THREADS = 256;
-constexpr int EXP_TAB_BYTES = RK_EXP2_TABLE_N * 8;  // leads the dynamic shared memory
+constexpr int EXP_TAB_BYTES = RK_FX_EXP2_N * 8;  // leads the dynamic shared memory
 
-static __constant__ double c_exp2_table[RK_EXP2_TABLE_N] = {RK_EXP2_TABLE_VALUES};
+static __constant__ uint64_t c_exp2_table[RK_FX_EXP2_N] = {RK_FX_EXP2_VALUES};
+static __constant__ uint64_t c_fx_inv_c[128] = {RK_FX_INV_C_VALUES};
+static __constant__ uint64_t c_fx_log2_c[128] = {RK_FX_LOG2_C_VALUES};
 static __constant__ double c_log_inv_c[RK_LOG_TABLE_N] = {RK_LOG_INV_C_VALUES};
 static __constant__ double c_log_ln_c[RK_LOG_TABLE_N] = {RK_LOG_LN_C_VALUES};
 
 // ------------------------------------------------- table-driven exponential
-// exp(x) by Tang's table-driven method (ACM TOMS 15(2), 1989) with a 256-entry
-// table of 2^(j/256): x = (256 m + j) ln2/256 + r with |r| <= ln2/512,
-// exp(x) = 2^m 2^(j/256) (1 + p(r)), p the degree-4 Taylor polynomial of
-// e^r - 1 (truncation < 4e-17 relative).  k = 256 m + j comes from adding a
-// 1.5 2^52 shifter, r from a two-part ln2/256, and the final scaling by 2^m is
-// an integer add to the exponent field, so the fast path costs 9 FP64
-// operations.  |x| >= 708, infinities and NaN take the library exp().
-constexpr double EXP_SHIFTER = 6755399441055744.0;  // 1.5 * 2^52
-constexpr int EXP_LOG2N = 8;                        // log2 of the table size
-
-__device__ __forceinline__ double exp_scale(double y, int e) {
-  return __hiloint2double(__double2hiint(y) + (e << 20), __double2loint(y));
-}
-
-__device__ __forceinline__ double exp_fast(double x, const double* __restrict__ tab) {
+// exp(x) by Tang's table-driven method (ACM TOMS 15(2), 1989) on the integer
+// pipes (fx::exp_double, 1.2 ulp): no FP64 instruction, where the same method
+// in FP64 was nine (576 cycles of the sub-partition's FP64 unit; the ~12
+// multiplies and ~30 adds and shifts here take ~100 of the integer pipes).
+// |x| >= 708, infinities and NaN take the library exp().
+__device__ __forceinline__ double exp_fast(double x, const uint64_t* __restrict__ tab) {
   if ((__double2hiint(x) & 0x7fffffff) >= 0x40862000) return exp(x);
-  const double kt = fma(x, RK_N_OVER_LN2, EXP_SHIFTER);
-  const int k = __double2loint(kt);
-  const double kd = kt - EXP_SHIFTER;
-  double r = fma(-kd, RK_LN2_OVER_N_HI, x);
-  r = fma(-kd, RK_LN2_OVER_N_LO, r);
-  double q = fma(r, 1.0 / 24.0, 1.0 / 6.0);
-  q = fma(q, r, 0.5);
-  const double p = fma(r * r, q, r);
-  const double t = tab[k & (RK_EXP2_TABLE_N - 1)];
-  return exp_scale(fma(t, p, t), k >> EXP_LOG2N);
+  return fx::exp_double(x, tab);
 }
 
-// Mixed-precision exp: the same argument reduction and reconstruction in FP64,
-// e^r - 1 = r + r^2 q(r) with the small term r^2 q(r) (|r| <= ln2/512, so at
-// most 9.2e-7) in FP32.  Relative error ~1e-13 for 6 FP64 operations instead
-// of 9.
-__device__ __forceinline__ double exp_mixed(double x, const double* __restrict__ tab) {
-  if ((__double2hiint(x) & 0x7fffffff) >= 0x40862000) return exp(x);
-  const double kt = fma(x, RK_N_OVER_LN2, EXP_SHIFTER);
-  const int k = __double2loint(kt);
-  const double kd = kt - EXP_SHIFTER;
-  double r = fma(-kd, RK_LN2_OVER_N_HI, x);
-  r = fma(-kd, RK_LN2_OVER_N_LO, r);
-  const float rf = __double2float_rn(r);
-  const float q = fmaf(fmaf(rf, 1.0f / 24.0f, 1.0f / 6.0f), rf, 0.5f);
-  const double p = r + (double)(rf * rf * q);
-  const double t = tab[k & (RK_EXP2_TABLE_N - 1)];
-  return exp_scale(fma(t, p, t), k >> EXP_LOG2N);
-}
-
-// (exp(x), exp(-x)) as exp_mixed, sharing the argument reduction.
-__device__ __forceinline__ void exp_pm_mixed(double x, const double* __restrict__ tab, double* ep, double* em) {
-  if ((__double2hiint(x) & 0x7fffffff) >= 0x40862000) {
-    *ep = exp(x);
-    *em = exp(-x);
-    return;
-  }
-  const double kt = fma(x, RK_N_OVER_LN2, EXP_SHIFTER);
-  const int k = __double2loint(kt);
-  const double kd = kt - EXP_SHIFTER;
-  double r = fma(-kd, RK_LN2_OVER_N_HI, x);
-  r = fma(-kd, RK_LN2_OVER_N_LO, r);
-  const float rf = __double2float_rn(r);
-  const float r2 = rf * rf;
-  const float qp = fmaf(fmaf(rf, 1.0f / 24.0f, 1.0f / 6.0f), rf, 0.5f);
-  const float qm = fmaf(fmaf(-rf, 1.0f / 24.0f, 1.0f / 6.0f), -rf, 0.5f);
-  const double pp = r + (double)(r2 * qp);
-  const double pm = (double)(r2 * qm) - r;
-  const double tp = tab[k & (RK_EXP2_TABLE_N - 1)];
-  const int km = -k;
-  const double tm = tab[km & (RK_EXP2_TABLE_N - 1)];
-  *ep = exp_scale(fma(tp, pp, tp), k >> EXP_LOG2N);
-  *em = exp_scale(fma(tm, pm, tm), km >> EXP_LOG2N);
+// a < b for doubles with b > 0 by their bits (an FP64 comparison takes the FP64
+// unit as long as a multiplication): false for NaN a of either sign, as a < b is.
+__device__ __forceinline__ bool below(double a, double b) {
+  return __double_as_longlong(a) < __double_as_longlong(b) && (__double2hiint(a) & 0x7ff00000) != 0x7ff00000;
 }
 
 // 1/x by Newton's iteration for the reciprocal, r <- r + r (1 - x r), from
 // an FP32 estimate: two steps square the estimate's relative error twice
-// ((1e-7)^4), leaving the last rounding.  Four FP64 operations instead of a
-// full-precision division; for positive normal x inside the FP32 range (the
-// temperature and the mixture sums of a cell).
+// ((2e-7)^4), leaving the last rounding.  Four FP64 operations instead of a
+// full-precision division; for normal x inside the FP32 range (the
+// temperature and the mixture sums of a cell).  The conversions to FP32
+// (truncated) and back are integer moves: a conversion instruction takes the FP64
+// unit as long as an FP64 operation.
 __device__ __forceinline__ double rcp_newton(double x) {
-  double r = (double)__frcp_rn(__double2float_rn(x));
+  const int hi = __double2hiint(x), sign = hi & (int)0x80000000;
+  const float f = __int_as_float((((hi & 0x7fffffff) - (896 << 20)) << 3) | (int)((unsigned)__double2loint(x) >> 29));
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(f));
+  const int b = __float_as_int(y);
+  double r = __hiloint2double(((b >> 3) + (896 << 20)) | sign, b << 29);
   double e = fma(-x, r, 1.0);
   r = fma(r, e, r);
   e = fma(-x, r, 1.0);
@@ -170,6 +128,29 @@ __device__ __forceinline__ double rcp_newton(double x) {
 __device__ __forceinline__ double rcp_any(double x) {
   const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
   return ex - 898u < 250u ? rcp_newton(x) : 1.0 / x;
+}
+
+// 1/sqrt(x) for positive, finite, normal x: FP32 estimate of the significand with
+// an even exponent (x = 4^k w, w in [1, 4)), one cubically convergent step
+// y += y e (1/2 + 3/8 e), e = 1 - w y^2 (|e| < 5e-7, so the rest is below 1e-19).
+__device__ __forceinline__ double rsqrt_newton(double x) {
+  const int hi = __double2hiint(x);
+  const int k = ((hi >> 20) - 1023) >> 1;
+  const double w = __hiloint2double(hi - (k << 21), __double2loint(x));
+  const int wh = __double2hiint(w);
+  float y0;
+  asm("rsqrt.approx.ftz.f32 %0, %1;"
+      : "=f"(y0)
+      : "f"(__int_as_float(((wh - (896 << 20)) << 3) | (int)((unsigned)__double2loint(w) >> 29))));
+  const int b = __float_as_int(y0);
+  const double y = __hiloint2double((b >> 3) + (896 << 20), b << 29);
+  const double e = fma(-(w * y), y, 1.0);
+  const double r = fma(y * e, fma(0.375, e, 0.5), y);
+  return __hiloint2double(__double2hiint(r) - (k << 20), __double2loint(r));
+}
+__device__ __forceinline__ double rsqrt_any(double x) {
+  const unsigned ex = (unsigned)__double2hiint(x) >> 20;  // sign and exponent
+  return ex - 1u < 2046u ? rsqrt_newton(x) : rsqrt(x);
 }
 
 // ------------------------------------------------- table-driven logarithm
@@ -235,34 +216,8 @@ __device__ __forceinline__ df2 df_scale(float c, df2 a) {  // c * a with the exa
   return df_norm(p, fmaf(c, a.l, e));
 }
 
-// (exp(x), exp(-x)) sharing one argument reduction.
-__device__ __forceinline__ void exp_pm(double x, const double* __restrict__ tab, double* ep, double* em) {
-  if ((__double2hiint(x) & 0x7fffffff) >= 0x40862000) {
-    *ep = exp(x);
-    *em = exp(-x);
-    return;
-  }
-  const double kt = fma(x, RK_N_OVER_LN2, EXP_SHIFTER);
-  const int k = __double2loint(kt);
-  const double kd = kt - EXP_SHIFTER;
-  double r = fma(-kd, RK_LN2_OVER_N_HI, x);
-  r = fma(-kd, RK_LN2_OVER_N_LO, r);
-  const double r2 = r * r;
-  double q = fma(r, 1.0 / 24.0, 1.0 / 6.0);
-  q = fma(q, r, 0.5);
-  const double pp = fma(r2, q, r);
-  double qm = fma(-r, 1.0 / 24.0, 1.0 / 6.0);
-  qm = fma(qm, -r, 0.5);
-  const double pm = fma(r2, qm, -r);
-  const double tp = tab[k & (RK_EXP2_TABLE_N - 1)];
-  const int km = -k;
-  const double tm = tab[km & (RK_EXP2_TABLE_N - 1)];
-  *ep = exp_scale(fma(tp, pp, tp), k >> EXP_LOG2N);
-  *em = exp_scale(fma(tm, pm, tm), km >> EXP_LOG2N);
-}
-
-__device__ inline void load_exp_table(double* dst) {
-  for (int i = threadIdx.x; i < RK_EXP2_TABLE_N; i += blockDim.x) dst[i] = c_exp2_table[i];
+__device__ inline void load_exp_table(uint64_t* dst) {
+  for (int i = threadIdx.x; i < RK_FX_EXP2_N; i += blockDim.x) dst[i] = c_exp2_table[i];
 }
 
 // --------------------------------------------------------------- error state
@@ -274,12 +229,19 @@ int cuda_error(cudaError_t e, const char* where);
 struct MechView {
   int ns, nr, ntb, ntroe;
   int nx;  // state components after T: 0, or 5 (rho, rho u, rho E) for the auxiliary-temperature system
-  const double* etab;  // 2^(j/256) table in shared memory
+  const uint64_t* etab;  // 2^(j/256) table in shared memory
   const double *W, *invW, *Tmid, *lo, *hi, *lnA, *bexp, *EaR, *eff, *fo, *csr_nu;
+  const uint64_t *fA, *fb, *fE;  // fixed-point Arrhenius coefficients (fx.cuh)
+  bool fx;                       // every coefficient fits that form
   const uint32_t* slots;
   const int32_t *meta, *csr_ptr, *csr_j;
+  const int32_t* gcsr_j;  // csr_j in global memory
   const int32_t *piece_ptr, *spec_piece;  // gather pieces of the species-major list
   int npiece;
+  const uint16_t* gidx;  // fixed-point gather: [glen][gnpp] reactions, pieces of each species
+  const int32_t* gspec;
+  int glen, gnpp, ghb;
+  bool gfix;  // gather in fixed point
   const float *Wf, *invWf, *bf, *EaRf, *efff, *csr_nuf;  // FP32 copies
   const int32_t* perm;  // input index of each packed reaction
   int nst, nrt;         // nu^T tiles (species, reactions) of the tensor-core gather
@@ -287,7 +249,12 @@ struct MechView {
   const int32_t *role_ptr, *role;  // species-major reaction slots (r << 2 | role)
 };
 
-__host__ __device__ inline MechView make_view(const unsigned char* base, const MechLayout& L) {
+// The view of a block that copied the buffer's first `prefix` bytes to base and,
+// with fxseg, the fixed-point segment after them; lnA, csr_ptr and csr_nu are read
+// from the whole buffer in global memory, gbase.
+__host__ __device__ inline MechView make_view(const unsigned char* base, const unsigned char* gbase,
+                                              const MechLayout& L, int64_t prefix, bool fxseg) {
+  const unsigned char* fbase = base + prefix - L.off_fA;  // the segment's arrays sit at fbase + their offset
   MechView m;
   m.ns = L.ns;
   m.nr = L.nr;
@@ -300,19 +267,30 @@ __host__ __device__ inline MechView make_view(const unsigned char* base, const M
   m.Tmid = reinterpret_cast<const double*>(base + L.off_Tmid);
   m.lo = reinterpret_cast<const double*>(base + L.off_lo);
   m.hi = reinterpret_cast<const double*>(base + L.off_hi);
-  m.lnA = reinterpret_cast<const double*>(base + L.off_lnA);
+  m.lnA = reinterpret_cast<const double*>(gbase + L.off_lnA);
+  m.fA = reinterpret_cast<const uint64_t*>(fbase + L.off_fA);
+  m.fb = reinterpret_cast<const uint64_t*>(fbase + L.off_fb);
+  m.fE = reinterpret_cast<const uint64_t*>(fbase + L.off_fE);
+  m.fx = fxseg && L.fx != 0;
+  m.gcsr_j = reinterpret_cast<const int32_t*>(gbase + L.off_csr_j);
   m.bexp = reinterpret_cast<const double*>(base + L.off_b);
   m.EaR = reinterpret_cast<const double*>(base + L.off_EaR);
   m.eff = reinterpret_cast<const double*>(base + L.off_eff);
   m.fo = reinterpret_cast<const double*>(base + L.off_fo);
-  m.csr_nu = reinterpret_cast<const double*>(base + L.off_csr_nu);
+  m.csr_nu = reinterpret_cast<const double*>(gbase + L.off_csr_nu);
   m.slots = reinterpret_cast<const uint32_t*>(base + L.off_slots);
   m.meta = reinterpret_cast<const int32_t*>(base + L.off_meta);
-  m.csr_ptr = reinterpret_cast<const int32_t*>(base + L.off_csr_ptr);
+  m.csr_ptr = reinterpret_cast<const int32_t*>(gbase + L.off_csr_ptr);
   m.csr_j = reinterpret_cast<const int32_t*>(base + L.off_csr_j);
   m.piece_ptr = reinterpret_cast<const int32_t*>(base + L.off_piece_ptr);
   m.spec_piece = reinterpret_cast<const int32_t*>(base + L.off_spec_piece);
   m.npiece = L.npiece;
+  m.gidx = reinterpret_cast<const uint16_t*>(fbase + L.off_gidx);
+  m.gspec = reinterpret_cast<const int32_t*>(fbase + L.off_gspec);
+  m.glen = L.glen;
+  m.gnpp = L.gnpp;
+  m.ghb = L.ghb;
+  m.gfix = L.gfix != 0;
   m.Wf = reinterpret_cast<const float*>(base + L.off_Wf);
   m.invWf = reinterpret_cast<const float*>(base + L.off_invWf);
   m.bf = reinterpret_cast<const float*>(base + L.off_bf);
@@ -384,19 +362,20 @@ inline SlotLayout make_slot(const MechLayout& L, int M, bool mixed = false, int 
   s.Einv = take(ns1);
   s.CE = take(ns1);
   s.om = take(ns1);
-  s.q = take(L.nr > 0 ? L.nr : 1);
-  s.kc = take(L.nr > 0 ? L.nr : 1);
-  s.krc = take(L.nr > 0 ? L.nr : 1);
-  s.qT = take(L.nr > 0 ? L.nr : 1);
-  // The stage vectors K live only inside an attempt; the J v caches kc, krc,
-  // qT (contiguous) only from the caching right-hand side to the end of the
+  // reactions, and entry nr: the zero rate that pads the gather's pieces
+  s.q = take(L.nr + 1);
+  s.kc = take(L.nr + 1);
+  s.qT = take(L.nr + 1);
+  s.krc = take(L.nr + 1);
+  // The stage vectors K live only inside an attempt; the J v caches kc, qT
+  // (contiguous) only from the caching right-hand side to the end of the
   // Arnoldi process that precedes the attempts.  K shares their storage when
-  // it fits there.
-  const int nr_even = ((L.nr > 0 ? L.nr : 1) + 1) & ~1;
-  s.K = (4 * Nq <= 3 * nr_even) ? s.kc : take(4 * Nq);
+  // it fits there (not krc's, which holds the low words of the gather's rates).
+  const int nr_even = (L.nr + 2) & ~1;
+  s.K = (4 * Nq <= 2 * nr_even) ? s.kc : take(4 * Nq);
   s.tb = take(4 * (L.ntb > 0 ? L.ntb : 1));
   s.tro = take(11 * (L.ntroe > 0 ? L.ntroe : 1));
-  s.part = take(L.npiece > 0 ? L.npiece : 1);
+  s.part = take(2 * L.gnpp > L.npiece ? 2 * L.gnpp : L.npiece);  // (hi, lo) words of the fixed-point gather
   s.C2 = df ? take(ns1) : -1;
   s.dC2 = df ? take(ns1) : -1;
   s.dig = tc ? take(2 * 16 * L.nrt) : -1;  // 8 x 16 nrt BF16 = 2 x 16 nrt doubles
@@ -461,6 +440,7 @@ struct Grp {
     return v;
   }
   __device__ __forceinline__ int imax(int v) const {
+    if constexpr (G == 32) return __reduce_max_sync(0xffffffffu, v);
 #pragma unroll
     for (int o = G / 2; o > 0; o >>= 1) v = ::max(v, __shfl_xor_sync(mask, v, o, G));
     return v;
@@ -528,12 +508,14 @@ __device__ __forceinline__ void sum_first(const Grp<G>& g, T (&v)[MAXM], int n) 
 // Jacobian-vector product needs (uniform across the group).
 struct CellScalars {
   double T, invT, lnT, S, invS, rho, invrho, cb, invcb, Sh;
+  double TSh, irc;  // T Sh, 1 / (rho cb)
   double pinv;  // 1 / p (constant pressure) or 1 / rho (constant volume): set by the caller
   int prec;     // precision level (3: mixed exp in the RHS, double-float J v core): set by the caller
   // auxiliary-temperature system: sum_k (cp_k/R - 1) F_k / W_k, the T row
   // without its own source, 1 / rho and the velocity
   double B, fT, irho_c, vel[3];
   bool cv;
+  bool zf;  // the caches are those of the scaled form (reactions_scaled), read by jvp_eval
 };
 
 struct SlotPtrs {
@@ -580,7 +562,7 @@ __device__ inline SlotPtrs slot_ptrs(double* b, const SlotLayout& s) {
   p.dC2 = s.dC2 >= 0 ? reinterpret_cast<df2*>(b + s.dC2) : nullptr;
   p.dig = s.dig >= 0 ? reinterpret_cast<uint16_t*>(b + s.dig) : nullptr;
   {
-    const int nr_even = ((s.nr > 0 ? s.nr : 1) + 1) & ~1, ns1 = s.ns + 1;
+    const int nr_even = (s.nr + 2) & ~1, ns1 = s.ns + 1;
     float* R = reinterpret_cast<float*>(b + s.kc);  // 3 nr_even doubles = 6 nr_even floats
     p.xk = R;
     p.xkr = R + nr_even;
@@ -619,32 +601,118 @@ __device__ inline SlotPtrs slot_ptrs(double* b, const SlotLayout& s) {
   return p;
 }
 
-// w = nu^T q, pass 1: the species-major list is cut into pieces of near-equal
-// length (chosen when the mechanism is packed); each lane sums whole pieces
-// into part[], so the warp's loop runs over the longest piece rather than the
-// longest species row.  Pass 2 (piece_sum) adds a species' pieces in order:
-// the result does not depend on the launch shape.
-template <int G, typename T>
-__device__ __forceinline__ void gather_pieces(const MechView& m, int lane, const T* __restrict__ nu,
-                                              const T* __restrict__ q, T* part) {
-  for (int p = lane; p < m.npiece; p += G) {
-    T acc = T(0);
-    const int e1 = m.piece_ptr[p + 1];
-    for (int e = m.piece_ptr[p]; e < e1; ++e) acc = fma(nu[e], q[m.csr_j[e]], acc);
-    part[p] = acc;
+// w = nu^T q by rows of the species-major list in FP64, into part[0..ns): cells in
+// the direct form, rates that are not finite (their rows alone become so).
+template <int G>
+__device__ __noinline__ void gather_rows(const MechView& m, const SlotPtrs& s) {
+  const Grp<G> g;
+  for (int k = g.lane; k < m.ns; k += G) {
+    double acc = 0.0;
+    for (int e = m.csr_ptr[k]; e < m.csr_ptr[k + 1]; ++e) acc = fma(m.csr_nu[e], s.q[m.gcsr_j[e]], acc);
+    s.part[k] = acc;
   }
+  g.sync();
 }
-template <typename T>
-__device__ __forceinline__ T piece_sum(const MechView& m, const T* part, int k) {
-  const int p1 = m.spec_piece[k + 1];
-  int p = m.spec_piece[k];
-  T acc = part[p];
-  for (++p; p < p1; ++p) acc += part[p];
-  return acc;
+// The gather in 128-bit fixed point (fx.cuh): the rates in s.q go onto one grid
+// below their largest (high words in place, low words in krc's storage), each lane
+// adds up whole pieces with integer adds, and a species adds and subtracts its
+// pieces and rounds once.  Exact sums, whatever the order, so the pieces' entries
+// are ordered to meet no shared-memory bank conflicts and no coefficient is
+// loaded or multiplied.  An FP64 term took 64 cycles of the FP64 unit, here ~20 of
+// the integer pipes and ~5 shared-memory wavefronts.  Returns the largest biased
+// exponent, or -1 with nothing done when a rate is infinite or NaN.
+// em: the largest (high word >> 20) & 0x7ff over the lane's rates.
+template <int G>
+__device__ __forceinline__ int gather_fixed(const MechView& m, const SlotPtrs& s, int em) {
+  const Grp<G> g;
+  em = g.imax(em);
+  if (em == 0x7ff) return -1;
+  uint64_t* qh = reinterpret_cast<uint64_t*>(s.q);
+  uint64_t* ql = reinterpret_cast<uint64_t*>(s.krc);
+  constexpr int U = 4;
+  for (int j0 = g.lane; j0 < m.nr; j0 += U * G) {
+    fx::Wide w[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) w[u] = fx::to_grid(s.q[min(j0 + u * G, m.nr - 1)], em, m.ghb);
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (j0 + u * G < m.nr) {
+        qh[j0 + u * G] = w[u].hi;
+        ql[j0 + u * G] = w[u].lo;
+      }
+  }
+  if (g.lane == 0) qh[m.nr] = ql[m.nr] = 0ull;
+  g.sync();
+  uint64_t* part = reinterpret_cast<uint64_t*>(s.part);
+  const uint4* ix = reinterpret_cast<const uint4*>(m.gidx);
+  const char* bh = reinterpret_cast<const char*>(qh);
+  const char* bl = reinterpret_cast<const char*>(ql);
+  for (int p = g.lane; p < m.gnpp; p += G) {
+    fx::Wide a = {0ull, 0ull};
+    for (int i = 0; i < m.glen; i += 8) {
+      const uint4 v = ix[(i >> 3) * m.gnpp + p];
+      const uint32_t o[8] = {v.x & 0xffffu, v.x >> 16, v.y & 0xffffu, v.y >> 16,
+                             v.z & 0xffffu, v.z >> 16, v.w & 0xffffu, v.w >> 16};
+      uint64_t h[8], l[8];
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        h[t] = *reinterpret_cast<const uint64_t*>(bh + o[t]);
+        l[t] = *reinterpret_cast<const uint64_t*>(bl + o[t]);
+      }
+#pragma unroll
+      for (int t = 0; t < 8; ++t) fx::add(a, h[t], l[t]);
+    }
+    part[p] = a.hi;
+    part[m.gnpp + p] = a.lo;
+  }
+  g.sync();
+  return em;
+}
+// The same pieces in FP64, for mechanisms of few entries (gfix false), where the
+// conversions to the grid and back would cost more than the additions they save.
+template <int G>
+__device__ __forceinline__ int gather_listed(const MechView& m, const SlotPtrs& s) {
+  const Grp<G> g;
+  if (g.lane == 0) s.q[m.nr] = 0.0;
+  g.sync();
+  const char* q = reinterpret_cast<const char*>(s.q);
+  for (int p = g.lane; p < m.gnpp; p += G) {
+    double a = 0.0;
+    for (int i = 0; i < m.glen; ++i) {
+      const double x = *reinterpret_cast<const double*>(q + m.gidx[((i >> 3) * m.gnpp + p) * 8 + (i & 7)]);
+      a = i == 0 ? x : a + x;
+    }
+    s.part[p] = a;
+  }
+  g.sync();
+  return -2;
+}
+// nu^T q of species k after gather_fixed (em >= 0), gather_listed (-2) or gather_rows (-1)
+__device__ __forceinline__ double gathered_row(const MechView& m, const SlotPtrs& s, int k, int em) {
+  if (em == -1) return s.part[k];
+  const int p1 = m.gspec[2 * k + 1], p2 = m.gspec[2 * k + 2];
+  int p = m.gspec[2 * k];
+  if (em < 0) {
+    double a = 0.0, b = 0.0;
+    if (p < p1) a = s.part[p++];
+    for (; p < p1; ++p) a += s.part[p];
+    if (p < p2) b = s.part[p++];
+    for (; p < p2; ++p) b += s.part[p];
+    return a - b;
+  }
+  const uint64_t* part = reinterpret_cast<const uint64_t*>(s.part);
+  fx::Wide a = {0ull, 0ull};
+#pragma unroll 2
+  for (; p < p1; ++p) fx::add(a, part[p], part[m.gnpp + p]);
+#pragma unroll 2
+  for (; p < p2; ++p) fx::sub(a, part[p], part[m.gnpp + p]);
+  return fx::from_grid(a, em, m.ghb);
 }
 
-// The same gather in double-float (FP32 pairs, ~44-bit significands, on the
-// FP32 pipe): the net coefficients are small integers, exact in FP32, so each
+// The gather in double-float (FP32 pairs, ~44-bit significands, on the FP32
+// pipe): the species-major list is cut into pieces of near-equal length (chosen
+// when the mechanism is packed), each lane sums whole pieces into part[] and
+// piece_sum_df adds a species' pieces in order.  The net coefficients are small integers, exact in FP32, so each
 // product nu_e q_j is formed with the pair's precision and summed by two-sums.
 template <int G>
 __device__ __forceinline__ void gather_pieces_df(const MechView& m, int lane, const df2* __restrict__ q,
@@ -691,7 +759,7 @@ __device__ __forceinline__ uint16_t bf16_of_small_int(int v) {
 // x * 2^e for a double x holding an integer of magnitude below 2^53 and an
 // exponent that keeps the result normal: an integer add to the exponent field.
 __device__ __forceinline__ double scale_pow2(double x, int e) {
-  return x == 0.0 ? 0.0 : exp_scale(x, e);
+  return x == 0.0 ? 0.0 : __hiloint2double(__double2hiint(x) + (e << 20), __double2loint(x));
 }
 
 // out[k] = sum_j nu_jk q_j for the cell (q: Nr doubles in shared memory).
@@ -755,6 +823,222 @@ __device__ bool gather_tc(const MechView& m, const SlotPtrs& s, const double* __
   return true;
 }
 
+// Cached values of a pressure-dependent reaction for the Jacobian-vector
+// product: [M], dk/d[M], d ln k/dT and 1/Kc (and their FP32 copies, MIXED).
+template <bool MIXED>
+__device__ __forceinline__ void cache_pressure(const SlotPtrs& s, int slot, double Mc, double dkdM, double dlnk,
+                                               double rfac) {
+  double* t = s.tb + 4 * slot;
+  t[0] = Mc;
+  t[1] = dkdM;
+  t[2] = dlnk;
+  t[3] = rfac;
+  if (MIXED) {
+    float* tf = s.ftb + 4 * slot;
+    tf[0] = __double2float_rn(Mc);
+    tf[1] = __double2float_rn(dkdM);
+    tf[2] = __double2float_rn(dlnk);
+    tf[3] = __double2float_rn(rfac);
+  }
+}
+template <int G>
+__device__ __forceinline__ double third_body_conc(const MechView& m, const SlotPtrs& s, int slot, bool coop_tb) {
+  if (coop_tb) return s.tb[4 * slot];
+  const double* e = m.eff + (size_t)slot * m.ns;
+  double Mc = 0.0;
+  for (int q = 0; q < m.ns; ++q) Mc = fma(e[q], s.C[q], Mc);
+  return Mc;
+}
+// The caches of one reaction that the selected Jacobian-vector product reads.
+template <bool MIXED>
+__device__ __forceinline__ void cache_reaction(const SlotPtrs& s, const CellScalars* cs, int j, double k, double kr,
+                                               double qT) {
+  if (cs->prec == 3) {  // double-float copies for the J v core, in the same storage
+    reinterpret_cast<df2*>(s.qT)[j] = df_from(qT);
+    reinterpret_cast<df2*>(s.kc)[j] = df_from(k);
+    reinterpret_cast<df2*>(s.krc)[j] = df_from(kr);
+  } else if (cs->prec == 6) {  // FP32 copies for the FP32 J v, in the same storage
+    s.xk[j] = __double2float_rn(k);
+    s.xkr[j] = __double2float_rn(kr);
+    s.xqT[j] = __double2float_rn(qT);
+  } else {
+    s.qT[j] = qT;
+    s.kc[j] = k;
+    s.krc[j] = kr;
+  }
+  if (MIXED) {
+    s.fkc[j] = __double2float_rn(k);
+    s.fkr[j] = __double2float_rn(kr);
+  }
+}
+
+// The reactions in the scaled form.  With E_s = e^{g_s/RT} (RT/p_ref) per species
+// (1/Kc = prod E'' / prod E') and z = C E,
+//   q = k prod C^nu' - k/Kc prod C^nu'' = kappa (z_ra z_rb - z_pa z_pb),
+//   ln kappa = ln k - ln E_ra - ln E_rb:
+// one exponential whose argument takes both Gibbs factors as additions.  The
+// argument is formed in fixed point from the mechanism's coefficients, the
+// exponential and the product with kappa stay on the integer pipes (fx.cuh),
+// and two FP64 instructions are left, the difference of the two products; the
+// form with k, E and 1/E in FP64 took sixteen (28 with the caches, now 11).
+// scaled_rate has no branch, so U reactions' chains interleave: one alone is
+// ~500 cycles of latency for ~150 of issue.
+struct ScaledRate {
+  uint64_t lg, ks;  // log2 kappa in fixed point; kappa = ks 2^(kn - 63)
+  int kn;
+  double D, zr, zs;  // z_ra z_rb - z_pa z_pb (its first product alone when irreversible), z_pa, z_pb
+};
+__device__ __forceinline__ ScaledRate scaled_rate(const MechView& m, const SlotPtrs& s, const fx::Temp& ft, int j,
+                                                  uint32_t sl, bool rev) {
+  const uint64_t* A = reinterpret_cast<const uint64_t*>(s.gRT);
+  const int ra = sl & 255, rb = (sl >> 8) & 255, pa = (sl >> 16) & 255, pb = sl >> 24;
+  ScaledRate r;
+  r.zr = s.CE[pa];
+  r.zs = s.CE[pb];
+  const double D0 = __dmul_rn(s.CE[ra], s.CE[rb]);
+  const double D1 = fma(-r.zr, r.zs, D0);
+  r.D = rev ? D1 : D0;
+  r.lg = fx::arrhenius(ft, m.fA[j], m.fb[j], m.fE[j]) - A[ra] - A[rb];
+  r.ks = fx::exp2_sig(r.lg, m.etab);
+  r.kn = fx::exponent(r.lg);
+  return r;
+}
+// What the caching right-hand side at u_n keeps of one reaction.
+template <bool MIXED>
+__device__ __forceinline__ void cache_scaled(const MechView& m, const SlotPtrs& s, double invT, CellScalars* cs, int j,
+                                             uint32_t sl, int kind, bool rev, int slot, double Mc, double mult,
+                                             const ScaledRate& r) {
+  const int ra = sl & 255, rb = (sl >> 8) & 255, pa = (sl >> 16) & 255, pb = sl >> 24;
+  const uint64_t* A = reinterpret_cast<const uint64_t*>(s.gRT);
+  const int nt = m.ntroe;
+  const double kap0 = fx::pack(r.ks, r.kn);
+  const double kap = kind == 2 ? kap0 * mult : kap0;
+  double dlnk = __dmul_rn(fma(m.EaR[j], invT, m.bexp[j]), invT);  // d ln k / dT
+  if (kind == 2) dlnk = s.tro[7 * nt + slot];
+  // d q_j / dT at fixed concentrations (without the third-body factor):
+  // d ln k/dT q + d ln Kc/dT k prod C^nu''/Kc, with d ln Kc/dT =
+  // (sum_products h/RT - sum_reactants h/RT - dnu) / T summed from the
+  // per-species (h/RT - 1)/T
+  const double t0 = __dmul_rn(dlnk, r.D);
+  const double dlnKc = __dsub_rn(__dadd_rn(s.dC[pa], s.dC[pb]), __dadd_rn(s.dC[ra], s.dC[rb]));
+  const double t1 = fma(dlnKc, __dmul_rn(r.zr, r.zs), t0);
+  const double qT = __dmul_rn(kap, rev ? t1 : t0);
+  if (!MIXED && cs->prec != 3 && cs->prec != 6) {
+    // the scaled Jacobian-vector product: kappa, d q/dT and the slot's d kappa/d[M]
+    if (kind != 0) cache_pressure<MIXED>(s, slot, Mc, kind == 2 ? kap0 * s.tro[8 * nt + slot] : 0.0, dlnk, 0.0);
+    s.kc[j] = kap;
+    s.qT[j] = qT;
+  } else {
+    const double Er = __dmul_rn(s.E[ra], s.E[rb]);
+    const double k = __dmul_rn(kap, Er);
+    const double kr = rev ? __dmul_rn(kap, __dmul_rn(s.E[pa], s.E[pb])) : 0.0;
+    if (kind != 0)
+      cache_pressure<MIXED>(s, slot, Mc, kind == 2 ? kap0 * Er * s.tro[8 * nt + slot] : 0.0, dlnk,
+                            rev ? fx::exp2_double(A[pa] + A[pb] - A[ra] - A[rb], m.etab) : 0.0);
+    cache_reaction<MIXED>(s, cs, j, k, kr, qT);
+  }
+}
+// Reactions j0 + lane + u G, u < U (indices past the last are computed as the last
+// and not stored).  PRESSURE: the first ones, some of them third-body or falloff.
+template <int G, bool MIXED, bool PRESSURE, int U>
+__device__ __forceinline__ void reactions_scaled(const MechView& m, const SlotPtrs& s, const fx::Temp& ft, double invT,
+                                                 bool coop_tb, bool cache, CellScalars* cs, int j0, int lane, int* qe) {
+  ScaledRate r[U];
+  uint32_t sl[U];
+  int meta[U];
+  double q[U];
+  double Mc = 0.0, mult = 1.0;
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int j = min(j0 + lane + u * G, m.nr - 1);
+    sl[u] = m.slots[j];
+    meta[u] = m.meta[j];
+    r[u] = scaled_rate(m, s, ft, j, sl[u], (meta[u] >> 2) & 1);
+    double Dm = r[u].D;  // with the third-body or falloff multiplier
+    if (PRESSURE && (meta[u] & 3) != 0) {
+      Mc = third_body_conc<G>(m, s, meta[u] >> 8, coop_tb);
+      mult = (meta[u] & 3) == 1 ? Mc : s.tro[6 * m.ntroe + (meta[u] >> 8)];
+      Dm = __dmul_rn(Dm, mult);
+    }
+    q[u] = fx::mul_sig(r[u].ks, r[u].kn, Dm);
+    *qe = max(*qe, (__double2hiint(q[u]) >> 20) & 0x7ff);
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int j = j0 + lane + u * G;
+    if (j < m.nr) {
+      if (MIXED) reinterpret_cast<df2*>(s.q)[j] = df_from(q[u]);  // double-float copy for the gather
+      else s.q[j] = q[u];
+      if (cache)
+        cache_scaled<MIXED>(m, s, invT, cs, j, sl[u], PRESSURE ? meta[u] & 3 : 0, (meta[u] >> 2) & 1, meta[u] >> 8, Mc,
+                            mult, r[u]);
+    }
+  }
+}
+
+// Every reaction with 1/Kc from one exponential of its own: the form for cells
+// the scaled one does not hold for (a Gibbs factor past e^170, T outside
+// [250, 16000) K, coefficients outside the fixed-point range, NaN).
+template <int G, bool MIXED>
+__device__ __noinline__ void reactions_direct(const MechView& m, const SlotPtrs& s, double invT, double lnT,
+                                              double lnRTp, bool coop_tb, bool cache, CellScalars* cs) {
+  const Grp<G> g;
+  const int ns = m.ns;
+  for (int j = g.lane; j < m.nr; j += G) {
+    const uint32_t sl = m.slots[j];
+    const int ra = sl & 255, rb = (sl >> 8) & 255, pa = (sl >> 16) & 255, pb = sl >> 24;
+    const int meta = m.meta[j];
+    const int kind = meta & 3;
+    const bool rev = (meta >> 2) & 1;
+    const double lnk = fma(-m.EaR[j], invT, fma(m.bexp[j], lnT, m.lnA[j]));
+    double k = exp_fast(lnk, m.etab);
+    const double Pf = __dmul_rn(s.C[ra], s.C[rb]);
+    double Rb = 0.0, rfac = 0.0, PfRb = Pf;  // prod C^nu'' / Kc, 1/Kc and Pf - Rb
+    if (rev) {
+      // ln E with ln(RT/p_ref) in it: its dnu multiples come out of the differences
+      rfac = exp_fast((s.gRT[pa] - s.gRT[ra]) + (s.gRT[pb] - s.gRT[rb]), m.etab);
+      Rb = __dmul_rn(rfac, __dmul_rn(s.C[pa], s.C[pb]));
+      PfRb = __dsub_rn(Pf, Rb);
+    }
+    double mfac = 1.0;
+    double dlnk = 0.0;  // d ln k / dT (cache only)
+    if (cache) dlnk = __dmul_rn(fma(m.EaR[j], invT, m.bexp[j]), invT);
+    if (kind != 0) {
+      const int slot = meta >> 8;
+      const double Mc = third_body_conc<G>(m, s, slot, coop_tb);
+      double dkdM = 0.0;
+      if (kind == 1) {
+        mfac = Mc;
+      } else {
+        // Troe: the multiplier and derivatives from the falloff passes above
+        // (Troe reactions hold slots 0..ntroe-1)
+        if (cache) {
+          dlnk = s.tro[7 * m.ntroe + slot];
+          dkdM = k * s.tro[8 * m.ntroe + slot];
+        }
+        k = k * s.tro[6 * m.ntroe + slot];
+      }
+      if (cache) cache_pressure<MIXED>(s, slot, Mc, dkdM, dlnk, rfac);
+    }
+    // q = m k (prod C^nu' - prod C^nu'' / Kc); the third-body factor only where there is one
+    const double q0 = __dmul_rn(k, PfRb);
+    double qj = q0;
+    if (kind == 1) qj = __dmul_rn(mfac, qj);
+    if (MIXED) reinterpret_cast<df2*>(s.q)[j] = df_from(qj);  // double-float copy for the gather
+    else s.q[j] = qj;
+    if (cache) {
+      const double kr = __dmul_rn(k, rfac);
+      // d q_j / dT at fixed concentrations (without the third-body factor):
+      // d ln k/dT q0 + d ln Kc/dT k prod C^nu''/Kc, q0 = k (prod C^nu' - prod C^nu''/Kc),
+      // with d ln Kc/dT = (sum_products h/RT - sum_reactants h/RT - dnu) / T
+      // summed from the per-species (h/RT - 1)/T
+      const double dlnKc = __dsub_rn(__dadd_rn(s.dC[pa], s.dC[pb]), __dadd_rn(s.dC[ra], s.dC[rb]));
+      const double qT = fma(dlnk, q0, __dmul_rn(dlnKc, __dmul_rn(k, Rb)));
+      cache_reaction<MIXED>(s, cs, j, k, kr, qT);
+    }
+  }
+}
+
 // ------------------------------------------------------------ chemistry RHS
 // out = f(uu) + src (src may be null).  p > 0: constant-pressure reactor at
 // pressure p; p < 0: constant-volume reactor of density -p (Eq. cv_reactor with
@@ -774,13 +1058,22 @@ __device__ __forceinline__ void rhs_eval(const MechView& m, const SlotPtrs& s, c
   const int ns = m.ns;
   const double T = uu[ns];
   const double invT = rcp_newton(T);
-  const double lnT = log_fast(T);
+  // log2 T in fixed point gives ln T (0.6 ulp) and the rate constants' T^b
+  const bool t_fx = below(T, fx::T_HI) && !below(T, fx::T_LO);
+  uint64_t lgT = 0;
+  double lnT;
+  if (t_fx) {
+    lgT = fx::log2_fixed(T, c_fx_inv_c, c_fx_log2_c);
+    lnT = fx::from_fixed59(fx::mulhi(lgT, RK_FX_LN2));
+  } else {
+    lnT = log_fast(T);
+  }
   const double lnRTp = LN_R_OVER_PREF + lnT;  // ln(R T / p_ref)
   // species pass 1: thermo, Gibbs factors, sum Y/W
   double S = 0.0;
   int ghi = 0;  // max over species of the high word of |g/RT + ln(RT/p_ref)| (integer compare)
   for (int k = g.lane; k < ns; k += G) {
-    const double* c = (T < m.Tmid[k]) ? m.lo : m.hi;
+    const double* c = below(T, m.Tmid[k]) ? m.lo : m.hi;
     const double a1 = c[k], a2 = c[ns + k], a3 = c[2 * ns + k], a4 = c[3 * ns + k], a5 = c[4 * ns + k];
     const double cp = fma(fma(fma(fma(a5, T, a4), T, a3), T, a2), T, a1);
     const double hp = fma(fma(fma(c[8 * ns + k], T, c[7 * ns + k]), T, c[6 * ns + k]), T, c[5 * ns + k]);
@@ -790,8 +1083,9 @@ __device__ __forceinline__ void rhs_eval(const MechView& m, const SlotPtrs& s, c
     const double grt = hrt - sr;
     s.cp[k] = cp;
     s.hRT[k] = hrt;
-    s.gRT[k] = grt;
-    ghi = max(ghi, __double2hiint(grt + lnRTp) & 0x7fffffff);
+    const double a = grt + lnRTp;  // ln E
+    s.gRT[k] = a;
+    ghi = max(ghi, __double2hiint(a) & 0x7fffffff);
     if (cache) {
       const double dcp = fma(fma(fma(c[16 * ns + k], T, c[15 * ns + k]), T, c[14 * ns + k]), T, a2);
       s.dcp[k] = dcp;
@@ -808,13 +1102,14 @@ __device__ __forceinline__ void rhs_eval(const MechView& m, const SlotPtrs& s, c
   }
   S = g.sum(S);
   ghi = g.imax(ghi);
-  const bool direct_kc = ghi >= G_OVERFLOW_HI;  // some |g/RT + ln(RT/p_ref)| >= 170, also NaN
+  // the scaled form of the reactions holds while every |g/RT + ln(RT/p_ref)| < 170
+  // (false for NaN too) and T is inside the fixed-point range
+  const bool zf = m.fx && ghi < G_OVERFLOW_HI && t_fx;
   // auxiliary-temperature system (Eq. chemical_source_balanced): the species
   // components are rho Y_k, so C_k = u_k / W_k and d(rho Y_k)/dt = W_k w_k:
   // the constant-volume arithmetic with unit density
   const bool aux = m.nx > 0;
-  const bool cv = p < 0.0 || aux;
-  const double esh = cv ? 1.0 : 0.0;  // h/RT -> u/RT and cp/R -> cv/R shift
+  const bool cv = __double2hiint(p) < 0 || aux;  // p < 0 (never -0 or NaN)
   const double invS = rcp_newton(S);
   // rho = p / (R T S), 1/rho = R T S / p, with 1/p (or 1/rho) from the caller
   const double rho = aux ? 1.0 : (cv ? -p : p * invT * invS * INV_R);
@@ -830,14 +1125,15 @@ __device__ __forceinline__ void rhs_eval(const MechView& m, const SlotPtrs& s, c
     s.C[k] = Ck;
     if (MIXED && cache) s.fC[k] = __double2float_rn(Ck);
     if (cache && cs->prec == 3) s.C2[k] = df_from(Ck);
-    if (!direct_kc) {
-      // E = e^{g/RT} (RT/p_ref), Einv = 1/E: 1/Kc of a reaction is the product of
-      // E over its products and Einv over its reactants (the pressure factor
-      // (RT/p_ref)^dnu included); CE = C E, so k/Kc prod C^nu'' is three products
-      // (in FP64 at every precision level: the equilibrium constants come from these)
-      const double a = s.gRT[k] + lnRTp;
-      exp_pm(a, m.etab, &s.E[k], &s.Einv[k]);
-      s.CE[k] = __dmul_rn(Ck, s.E[k]);
+    if (zf) {
+      // A = ln E log2 e in fixed point, E = e^{g/RT} (RT/p_ref) = 2^A and z = C E; A
+      // replaces ln E.  z and the A of a rate constant come from one rounded A,
+      // so its rounding cancels between the two
+      const uint64_t A = fx::log2e_fixed(s.gRT[k]);
+      const double E = fx::exp2_double(A, m.etab);
+      reinterpret_cast<uint64_t*>(s.gRT)[k] = A;
+      s.E[k] = E;
+      s.CE[k] = __dmul_rn(Ck, E);
     }
     if (coop_tb) {
 #pragma unroll
@@ -946,133 +1242,53 @@ __device__ __forceinline__ void rhs_eval(const MechView& m, const SlotPtrs& s, c
     g.sync();
   }
   // reactions: rate coefficients and rates of progress
-  const double m_lnRTp = -lnRTp;
-  for (int j = g.lane; j < m.nr; j += G) {
-    const uint32_t sl = m.slots[j];
-    const int ra = sl & 255, rb = (sl >> 8) & 255, pa = (sl >> 16) & 255, pb = sl >> 24;
-    const int meta = m.meta[j];
-    const int kind = meta & 3;
-    const bool rev = (meta >> 2) & 1;
-    const int dnu = ((meta >> 4) & 15) - 4;
-    const double lnk = fma(-m.EaR[j], invT, fma(m.bexp[j], lnT, m.lnA[j]));
-    double k = (MIXED || cs->prec == 3 || cs->prec >= 5) ? exp_mixed(lnk, m.etab) : exp_fast(lnk, m.etab);
-    const double Pf = __dmul_rn(s.C[ra], s.C[rb]);
-    // Rb = prod C^nu'' / Kc (the caching evaluation keeps it), rfac = 1/Kc
-    // (caching only), PfRb = Pf - Rb: from the per-species factors as
-    // (C_pa E_pa C_pb E_pb) (1/E_ra 1/E_rb) subtracted from Pf in one fma
-    double Rb = 0.0, rfac = 0.0, PfRb = Pf;
-    if (rev) {
-      if (!direct_kc) {
-        const double X = __dmul_rn(s.CE[pa], s.CE[pb]);
-        const double Y = __dmul_rn(s.Einv[ra], s.Einv[rb]);
-        PfRb = fma(-X, Y, Pf);
-        if (cache) {
-          Rb = __dmul_rn(X, Y);
-          rfac = __dmul_rn(__dmul_rn(s.E[pa], s.E[pb]), Y);
-        }
-      } else {
-        const double dl = dnu > 0 ? lnRTp : (dnu < 0 ? m_lnRTp : 0.0);
-        rfac = exp_fast(s.gRT[pa] + s.gRT[pb] - s.gRT[ra] - s.gRT[rb] + dl, m.etab);
-        Rb = __dmul_rn(rfac, __dmul_rn(s.C[pa], s.C[pb]));
-        PfRb = __dsub_rn(Pf, Rb);
-      }
-    }
-    double mfac = 1.0;
-    double dlnk = 0.0;  // d ln k / dT (cache only)
-    if (cache) dlnk = __dmul_rn(fma(m.EaR[j], invT, m.bexp[j]), invT);
-    if (kind != 0) {
-      const int slot = meta >> 8;
-      double Mc;
-      if (coop_tb) {
-        Mc = s.tb[4 * slot];
-      } else {
-        const double* e = m.eff + (size_t)slot * ns;
-        Mc = 0.0;
-        for (int q = 0; q < ns; ++q) Mc = fma(e[q], s.C[q], Mc);
-      }
-      double dkdM = 0.0;
-      if (kind == 1) {
-        mfac = Mc;
-      } else {
-        // Troe: the multiplier and derivatives from the falloff passes above
-        // (Troe reactions hold slots 0..ntroe-1)
-        if (cache) {
-          dlnk = s.tro[7 * nt + slot];
-          dkdM = k * s.tro[8 * nt + slot];
-        }
-        k = k * s.tro[6 * nt + slot];
-      }
-      if (cache) {
-        double* t = s.tb + 4 * (meta >> 8);
-        t[0] = Mc;
-        t[1] = dkdM;
-        t[2] = dlnk;
-        t[3] = rfac;
-        if (MIXED) {
-          float* tf = s.ftb + 4 * (meta >> 8);
-          tf[0] = __double2float_rn(Mc);
-          tf[1] = __double2float_rn(dkdM);
-          tf[2] = __double2float_rn(dlnk);
-          tf[3] = __double2float_rn(rfac);
-        }
-      }
-    }
-    // q = m k (prod C^nu' - prod C^nu'' / Kc); the third-body factor only where there is one
-    const double q0 = __dmul_rn(k, PfRb);
-    double qj = q0;
-    if (kind == 1) qj = __dmul_rn(mfac, qj);
-    if (MIXED) reinterpret_cast<df2*>(s.q)[j] = df_from(qj);  // double-float copy for the gather
-    else s.q[j] = qj;
-    if (cache) {
-      const double kr = __dmul_rn(k, rfac);
-      // d q_j / dT at fixed concentrations (without the third-body factor):
-      // d ln k/dT q0 + d ln Kc/dT k prod C^nu''/Kc, q0 = k (prod C^nu' - prod C^nu''/Kc),
-      // with d ln Kc/dT = (sum_products h/RT - sum_reactants h/RT - dnu) / T
-      // summed from the per-species (h/RT - 1)/T
-      const double dlnKc = __dsub_rn(__dadd_rn(s.dC[pa], s.dC[pb]), __dadd_rn(s.dC[ra], s.dC[rb]));
-      const double qT = fma(dlnk, q0, __dmul_rn(dlnKc, __dmul_rn(k, Rb)));
-      if (cs->prec == 3) {  // double-float copies for the J v core, in the same storage
-        reinterpret_cast<df2*>(s.qT)[j] = df_from(qT);
-        reinterpret_cast<df2*>(s.kc)[j] = df_from(k);
-        reinterpret_cast<df2*>(s.krc)[j] = df_from(kr);
-      } else if (cs->prec == 6) {  // FP32 copies for the FP32 J v, in the same storage
-        s.xk[j] = __double2float_rn(k);
-        s.xkr[j] = __double2float_rn(kr);
-        s.xqT[j] = __double2float_rn(qT);
-      } else {
-        s.qT[j] = qT;
-        s.kc[j] = k;
-        s.krc[j] = kr;
-      }
-      if (MIXED) {
-        s.fkc[j] = __double2float_rn(k);
-        s.fkr[j] = __double2float_rn(kr);
-      }
-    }
+  int qe = 0;  // largest exponent of the lane's rates
+  if (zf) {
+    const fx::Temp ft = fx::temperature(lgT, fx::recip_fixed70(T, invT));
+    int j0 = 0;
+    for (; j0 < m.ntb; j0 += G) reactions_scaled<G, MIXED, true, 1>(m, s, ft, invT, coop_tb, cache, cs, j0, g.lane, &qe);
+    constexpr int U = RK_UNROLL;
+    for (; j0 < m.nr; j0 += U * G)
+      reactions_scaled<G, MIXED, false, U>(m, s, ft, invT, coop_tb, cache, cs, j0, g.lane, &qe);
+  } else {
+    reactions_direct<G, MIXED>(m, s, invT, lnT, lnRTp, coop_tb, cache, cs);
   }
   g.sync();
   // species pass 2: w = nu^T q, dY/dt and the sums of the temperature equation
   double Sh = 0.0, cb = 0.0;
+  const bool zjv = zf && !MIXED && cs->prec != 3 && cs->prec != 6;
   double Ax = 0.0, Bx = 0.0;  // auxiliary T: sum (u_k/RT) F_k / W_k and sum (cv_k/R) F_k / W_k
   bool tc_om = false;  // w already in part[0..ns) from the tensor cores
   if constexpr (TC) tc_om = gather_tc<G>(m, s, s.q, s.part);
-  if (MIXED) gather_pieces_df<G>(m, g.lane, reinterpret_cast<const df2*>(s.q), reinterpret_cast<df2*>(s.part));
-  else if (!tc_om) gather_pieces<G, double>(m, g.lane, m.csr_nu, s.q, s.part);
-  g.sync();
+  // in fixed point, except where krc's storage is taken (by the caches of the
+  // direct form and of precision 3) or a rate is not finite
+  int em = -1;
+  if (MIXED) {
+    gather_pieces_df<G>(m, g.lane, reinterpret_cast<const df2*>(s.q), reinterpret_cast<df2*>(s.part));
+    g.sync();
+  } else if (!tc_om) {
+    if (zf && !(cache && cs->prec == 3)) em = m.gfix ? gather_fixed<G>(m, s, qe) : gather_listed<G>(m, s);
+    if (em == -1) gather_rows<G>(m, s);
+  }
   for (int k = g.lane; k < ns; k += G) {
     double om;
     if (MIXED) {
       om = piece_sum_df(m, reinterpret_cast<const df2*>(s.part), k);
       if (cache) s.fom[k] = __double2float_rn(om);
     } else {
-      om = tc_om ? s.part[k] : piece_sum(m, s.part, k);
+      om = gathered_row(m, s, k, em);
     }
     if (cache) s.om[k] = om;
     const double r = __dmul_rn(__dmul_rn(m.W[k], om), invrho);
     const double Fk = src ? __dadd_rn(r, src[k]) : r;
     out[k] = Fk;
-    Sh = fma(s.hRT[k] - esh, om, Sh);
-    cb = fma(uu[k] * (s.cp[k] - esh), m.invW[k], cb);
+    double hk = s.hRT[k], ck = s.cp[k];
+    if (cv) {  // internal energies and cv (uniform; the subtractions cost 64 cycles each)
+      hk -= 1.0;
+      ck -= 1.0;
+    }
+    Sh = fma(hk, om, Sh);
+    cb = fma(uu[k] * ck, m.invW[k], cb);
     if (aux) {
       Ax = fma((s.hRT[k] - 1.0) * Fk, m.invW[k], Ax);
       Bx = fma((s.cp[k] - 1.0) * Fk, m.invW[k], Bx);
@@ -1080,17 +1296,18 @@ __device__ __forceinline__ void rhs_eval(const MechView& m, const SlotPtrs& s, c
     if (cache) {
       // per-species factors of the analytic J v, written over arrays the
       // remaining RHS no longer reads (lane-private entries k):
-      //   E: rho/W_k   Einv: W_k/rho   gRT: h_k/RT - esh
+      //   E: rho/W_k (times E_k for the scaled J v)   Einv: W_k/rho   gRT: h_k/RT - esh
       //   hRT: (cp_k/R - h_k/RT) w_k / T   dcp: Y_k (dcp_k/dT) / W_k   cp: (cp_k/R - esh) / W_k
-      s.E[k] = rho * m.invW[k];
+      const double rW = rho * m.invW[k];
+      s.E[k] = zjv ? s.E[k] * rW : rW;
       s.Einv[k] = m.W[k] * invrho;
-      s.gRT[k] = s.hRT[k] - esh;
+      s.gRT[k] = hk;
       s.hRT[k] = (s.cp[k] - s.hRT[k]) * invT * om;
       s.dcp[k] = uu[k] * s.dcp[k] * m.invW[k];
-      s.cp[k] = (s.cp[k] - esh) * m.invW[k];
+      s.cp[k] = ck * m.invW[k];
       if (cs->prec == 6) {  // FP32 copies for the FP32 J v
         s.xC[k] = __double2float_rn(s.C[k]);
-        s.xE[k] = __double2float_rn(s.E[k]);
+        s.xE[k] = __double2float_rn(rW);
         s.xEinv[k] = __double2float_rn(s.Einv[k]);
         s.xom[k] = __double2float_rn(om);
         s.xg[k] = __double2float_rn(s.gRT[k]);
@@ -1154,7 +1371,10 @@ __device__ __forceinline__ void rhs_eval(const MechView& m, const SlotPtrs& s, c
     cs->cb = cb;
     cs->invcb = invcb;
     cs->Sh = Sh;
+    cs->TSh = T * Sh;
+    cs->irc = invrho * invcb;
     cs->cv = cv;
+    cs->zf = zjv;
   }
   g.sync();
 }
@@ -1178,6 +1398,89 @@ __device__ __forceinline__ void rhs_dispatch(const MechView& m, const SlotPtrs& 
   else rhs_eval_call<G, MIXED, TC>(m, s, uu, src, p, out, cache, cs);
 }
 
+// d[M] of a pressure-dependent reaction from dC: summed over the species by the
+// whole group (mp), or by the reaction's own lane when there are many slots.
+template <int G>
+__device__ __forceinline__ double third_body_rate(const MechView& m, const double* dC, int slot, bool coop_tb,
+                                                  const double (&mp)[MAXM]) {
+  double dM = 0.0;
+  if (coop_tb) {
+#pragma unroll
+    for (int q = 0; q < MAXM; ++q)
+      if (q == slot) dM = mp[q];
+  } else {
+    const double* e = m.eff + (size_t)slot * m.ns;
+    for (int q = 0; q < m.ns; ++q) dM = fma(e[q], dC[q], dM);
+  }
+  return dM;
+}
+
+// dq_j = d q_j/dT vT + kappa_j d(z_ra z_rb - z_pa z_pb) of reactions j0 + lane + u G
+// (as reactions_scaled): six FP64 instructions a reaction.
+template <int G, bool PRESSURE, int U>
+__device__ __forceinline__ void jvp_scaled(const MechView& m, const SlotPtrs& s, double vT, bool coop_tb,
+                                           const double (&mp)[MAXM], int j0, int lane, int* qe) {
+  double dq[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int j = min(j0 + lane + u * G, m.nr - 1);
+    const uint32_t sl = m.slots[j];
+    const int ra = sl & 255, rb = (sl >> 8) & 255, pa = (sl >> 16) & 255, pb = sl >> 24;
+    const int meta = m.meta[j];
+    const bool rev = (meta >> 2) & 1;
+    const double za = s.CE[ra], zb = s.CE[rb], zp = s.CE[pa], zq = s.CE[pb];
+    const double dD0 = fma(s.dC[ra], zb, za * s.dC[rb]);
+    const double dD1 = fma(-s.dC[pa], zq, fma(-zp, s.dC[pb], dD0));
+    const double kap = s.kc[j];
+    dq[u] = fma(s.qT[j], vT, kap * (rev ? dD1 : dD0));
+    if (PRESSURE && (meta & 3) != 0) {
+      const int slot = meta >> 8;
+      const double* t = s.tb + 4 * slot;
+      double D = za * zb;
+      if (rev) D = fma(-zp, zq, D);
+      const double dM = third_body_rate<G>(m, s.arg, slot, coop_tb, mp);
+      dq[u] = (meta & 3) == 1 ? t[0] * dq[u] + dM * (kap * D) : dq[u] + t[1] * dM * D;
+    }
+    *qe = max(*qe, (__double2hiint(dq[u]) >> 20) & 0x7ff);
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+    if (j0 + lane + u * G < m.nr) s.q[j0 + lane + u * G] = dq[u];
+}
+
+// The reaction rates' derivatives from k and k/Kc (caches not in the scaled form).
+template <int G, bool DFG>
+__device__ __forceinline__ void jvp_reactions(const MechView& m, const SlotPtrs& s, double vT, bool coop_tb,
+                                              const double (&mp)[MAXM]) {
+  const Grp<G> g;
+  for (int j = g.lane; j < m.nr; j += G) {
+    const uint32_t sl = m.slots[j];
+    const int ra = sl & 255, rb = (sl >> 8) & 255, pa = (sl >> 16) & 255, pb = sl >> 24;
+    const int meta = m.meta[j];
+    const int kind = meta & 3;
+    const double dPf = fma(s.dC[ra], s.C[rb], s.C[ra] * s.dC[rb]);
+    const double dPb = fma(s.dC[pa], s.C[pb], s.C[pa] * s.dC[pb]);
+    const double k = s.kc[j], kr = s.krc[j];
+    double dq = fma(s.qT[j], vT, fma(k, dPf, -kr * dPb));
+    if (kind != 0) {
+      const int slot = meta >> 8;
+      const double* t = s.tb + 4 * slot;
+      const double Pf = s.C[ra] * s.C[rb];
+      const double Pb = s.C[pa] * s.C[pb];
+      const double dM = third_body_rate<G>(m, s.dC, slot, coop_tb, mp);
+      if (kind == 1) dq = t[0] * dq + dM * (k * Pf - kr * Pb);
+      else dq = dq + t[1] * dM * (Pf - t[3] * Pb);
+    }
+    if (DFG) reinterpret_cast<df2*>(s.q)[j] = df_from(dq);
+    else s.q[j] = dq;
+  }
+}
+template <int G>
+__device__ __noinline__ void jvp_reactions_call(const MechView& m, const SlotPtrs& s, double vT, bool coop_tb,
+                                                const double (&mp)[MAXM]) {
+  jvp_reactions<G, false>(m, s, vT, coop_tb, mp);
+}
+
 // Analytic Jacobian-vector product out = J(u_n) v, using the values cached by
 // the last rhs_eval(..., cache = true) at u_n.  v, out: N-vectors.  Inlined
 // (unlike rhs_eval, nothing requires two call sites to produce the same bits),
@@ -1194,59 +1497,53 @@ __device__ __forceinline__ void jvp_eval(const MechView& m, const SlotPtrs& s, c
   a = g.sum(a);
   const double drr = cs.cv ? 0.0 : -fma(a, cs.invS, vT * invT);  // d rho / rho (0 at fixed volume)
   const bool coop_tb = m.ntb > 0 && m.ntb <= MAXM;
+  const bool zf = !DFG && cs.zf;
+  int qe = 0;  // largest exponent of the lane's dq
   double mp[MAXM];
 #pragma unroll
   for (int t = 0; t < MAXM; ++t) mp[t] = 0.0;
   for (int k = g.lane; k < ns; k += G) {
-    const double dCk = fma(s.C[k], drr, s.E[k] * v[k]);  // E: rho / W_k
-    s.dC[k] = dCk;
-    if (coop_tb) {
+    const double ev = s.E[k] * v[k];  // E: rho / W_k, scaled form: E_k rho / W_k
+    // dC, or dz = E dC in the scaled form
+    const double d = fma(zf ? s.CE[k] : s.C[k], drr, ev);
+    s.dC[k] = d;
+    if (m.ntb > 0) {
+      const double dCk = zf ? fma(s.C[k], drr, cs.rho * m.invW[k] * v[k]) : d;
+      if (zf) s.arg[k] = dCk;
+      if (coop_tb) {
 #pragma unroll
-      for (int t = 0; t < MAXM; ++t)
-        if (t < m.ntb) mp[t] = fma(m.eff[t * ns + k], dCk, mp[t]);
+        for (int t = 0; t < MAXM; ++t)
+          if (t < m.ntb) mp[t] = fma(m.eff[t * ns + k], dCk, mp[t]);
+      }
     }
   }
   if (coop_tb) sum_first<G>(g, mp, m.ntb);  // d[M]_t, identical on every lane
   g.sync();
-  for (int j = g.lane; j < m.nr; j += G) {
-    const uint32_t sl = m.slots[j];
-    const int ra = sl & 255, rb = (sl >> 8) & 255, pa = (sl >> 16) & 255, pb = sl >> 24;
-    const int meta = m.meta[j];
-    const int kind = meta & 3;
-    const double dPf = fma(s.dC[ra], s.C[rb], s.C[ra] * s.dC[rb]);
-    const double dPb = fma(s.dC[pa], s.C[pb], s.C[pa] * s.dC[pb]);
-    const double k = s.kc[j], kr = s.krc[j];
-    double dq = fma(s.qT[j], vT, fma(k, dPf, -kr * dPb));
-    if (kind != 0) {
-      const int slot = meta >> 8;
-      const double* t = s.tb + 4 * slot;
-      const double Pf = s.C[ra] * s.C[rb];
-      const double Pb = s.C[pa] * s.C[pb];
-      double dM = 0.0;
-      if (coop_tb) {
-#pragma unroll
-        for (int q = 0; q < MAXM; ++q)
-          if (q == slot) dM = mp[q];
-      } else {
-        const double* e = m.eff + (size_t)slot * ns;
-        for (int q = 0; q < ns; ++q) dM = fma(e[q], s.dC[q], dM);
-      }
-      if (kind == 1) dq = t[0] * dq + dM * (k * Pf - kr * Pb);
-      else dq = dq + t[1] * dM * (Pf - t[3] * Pb);
-    }
-    if (DFG) reinterpret_cast<df2*>(s.q)[j] = df_from(dq);
-    else s.q[j] = dq;
+  if (zf) {
+    int j0 = 0;
+    for (; j0 < m.ntb; j0 += G) jvp_scaled<G, true, 1>(m, s, vT, coop_tb, mp, j0, g.lane, &qe);
+    constexpr int U = RK_UNROLL;
+    for (; j0 < m.nr; j0 += U * G) jvp_scaled<G, false, U>(m, s, vT, coop_tb, mp, j0, g.lane, &qe);
+  } else if constexpr (DFG) {
+    jvp_reactions<G, true>(m, s, vT, coop_tb, mp);
+  } else {
+    jvp_reactions_call<G>(m, s, vT, coop_tb, mp);
   }
   g.sync();
   bool tc_om = false;  // d w already in part[0..ns) from the tensor cores
   if constexpr (TC) tc_om = gather_tc<G>(m, s, s.q, s.part);
-  if (DFG) gather_pieces_df<G>(m, g.lane, reinterpret_cast<const df2*>(s.q), reinterpret_cast<df2*>(s.part));
-  else if (!tc_om) gather_pieces<G, double>(m, g.lane, m.csr_nu, s.q, s.part);
-  g.sync();
+  int em = -1;
+  if (DFG) {
+    gather_pieces_df<G>(m, g.lane, reinterpret_cast<const df2*>(s.q), reinterpret_cast<df2*>(s.part));
+    g.sync();
+  } else if (!tc_om) {
+    if (zf) em = m.gfix ? gather_fixed<G>(m, s, qe) : gather_listed<G>(m, s);
+    if (em == -1) gather_rows<G>(m, s);
+  }
   double dSh = 0.0, dcb = 0.0;
   for (int k = g.lane; k < ns; k += G) {
     const double dom = DFG ? piece_sum_df(m, reinterpret_cast<const df2*>(s.part), k)
-                           : (tc_om ? s.part[k] : piece_sum(m, s.part, k));
+                           : gathered_row(m, s, k, em);
     out[k] = s.Einv[k] * fma(-s.om[k], drr, dom);  // Einv: W_k / rho
     dSh = fma(s.gRT[k], dom, fma(s.hRT[k], vT, dSh));
     dcb = fma(s.dcp[k], vT, fma(s.cp[k], v[k], dcb));
@@ -1281,7 +1578,7 @@ __device__ __forceinline__ void jvp_eval(const MechView& m, const SlotPtrs& s, c
     dcb = t2[1];
   }
   if (g.lane == 0) {
-    out[ns] = (-(vT * cs.Sh + T * dSh) + T * cs.Sh * (drr + dcb * cs.invcb)) * (cs.invrho * cs.invcb);
+    out[ns] = fma(cs.TSh, fma(dcb, cs.invcb, drr), -fma(vT, cs.Sh, T * dSh)) * cs.irc;
   }
   g.sync();
 }
@@ -1443,11 +1740,16 @@ __device__ __noinline__ void jvp_eval_f32(const MechView& m, const SlotPtrs& s, 
     s.fq[j] = dq;
   }
   g.sync();
-  gather_pieces<G, float>(m, g.lane, m.csr_nuf, s.fq, s.fpart);
+  for (int p = g.lane; p < m.npiece; p += G) {
+    float acc = 0.f;
+    for (int e = m.piece_ptr[p]; e < m.piece_ptr[p + 1]; ++e) acc = fmaf(m.csr_nuf[e], s.fq[m.csr_j[e]], acc);
+    s.fpart[p] = acc;
+  }
   g.sync();
   float dSh = 0.f, dcb = 0.f;
   for (int k = g.lane; k < ns; k += G) {
-    const float dom = piece_sum(m, s.fpart, k);
+    float dom = 0.f;
+    for (int p = m.spec_piece[k]; p < m.spec_piece[k + 1]; ++p) dom += s.fpart[p];
     const float om = s.fom[k];
     const float vk = __double2float_rn(v[k]);
     out[k] = (double)(m.Wf[k] * (dom - om * drr) * invrho);
@@ -1462,14 +1764,6 @@ __device__ __noinline__ void jvp_eval_f32(const MechView& m, const SlotPtrs& s, 
   }
   if (g.lane == 0) out[ns] = (double)((-(vT * Sh + T * dSh) + T * Sh * (drr + dcb * invcb)) * (invrho * invcb));
   g.sync();
-}
-
-// A small nonzero integer held as a double, as a float, with integer
-// operations only (sign, exponent rebased from 1023 to 127, the top 20
-// significand bits of the high word): exact for |n| < 2^21.
-__device__ __forceinline__ float small_int_to_float(double x) {
-  const int hi = __double2hiint(x);
-  return __int_as_float((hi & (int)0x80000000) | ((((hi >> 20) & 0x7ff) - 896) << 23) | ((hi & 0xfffff) << 3));
 }
 
 // The analytic J v of jvp_eval in FP32 arithmetic (precision level 6): the
@@ -1509,7 +1803,10 @@ __device__ __forceinline__ void jvp_eval_f32x(const MechView& m, const SlotPtrs&
         if (t < m.ntb) mp[t] = fmaf(f(m.eff[t * ns + k]), dCk, mp[t]);
     }
   }
-  if (g.lane == 0) fdC[ns] = 0.f;  // the empty reaction slot (its C = 1 is in xC)
+  if (g.lane == 0) {
+    fdC[ns] = 0.f;  // the empty reaction slot (its C = 1 is in xC)
+    fq[m.nr] = 0.f;  // the rate that pads the pieces
+  }
   if (coop_tb) sum_first<G>(g, mp, m.ntb);
   g.sync();
   for (int j = g.lane; j < m.nr; j += G) {
@@ -1541,16 +1838,18 @@ __device__ __forceinline__ void jvp_eval_f32x(const MechView& m, const SlotPtrs&
     fq[j] = dq;
   }
   g.sync();
-  for (int p = g.lane; p < m.npiece; p += G) {  // d w = nu^T dq
+  for (int p = g.lane; p < m.gnpp; p += G) {  // d w = nu^T dq, in the fixed-point gather's pieces
     float acc = 0.f;
-    const int e1 = m.piece_ptr[p + 1];
-    for (int e = m.piece_ptr[p]; e < e1; ++e) acc = fmaf(small_int_to_float(m.csr_nu[e]), fq[m.csr_j[e]], acc);
+    for (int i = 0; i < m.glen; ++i) acc += fq[m.gidx[((i >> 3) * m.gnpp + p) * 8 + (i & 7)] >> 3];
     fpart[p] = acc;
   }
   g.sync();
   float dSh = 0.f, dcb = 0.f;
   for (int k = g.lane; k < ns; k += G) {
-    const float dom = piece_sum(m, static_cast<const float*>(fpart), k);
+    float dom = 0.f;
+    int p = m.gspec[2 * k];
+    for (; p < m.gspec[2 * k + 1]; ++p) dom += fpart[p];
+    for (; p < m.gspec[2 * k + 2]; ++p) dom -= fpart[p];
     out[k] = (double)(s.xEinv[k] * fmaf(-s.xom[k], drr, dom));  // xEinv: W_k / rho
     dSh = fmaf(s.xg[k], dom, fmaf(s.xh[k], vT, dSh));
     dcb = fmaf(s.xdcp[k], vT, fmaf(s.xcp[k], f(v[k]), dcb));
@@ -1629,8 +1928,10 @@ __device__ inline float group_dot_f(const Grp<G>& g, const double* a, const doub
 // FP64 instruction still takes its issue and pipe slot); J = 0: n = jn at run
 // time guards each of the MAXM terms.  Either way the same operations in the
 // same order for the terms that exist.
-template <int G, int J>
-__device__ __forceinline__ void cgs_pass(const SlotPtrs& s, int N, int jn, double (&hcol)[MAXM]) {
+// WW: w^T w before the pass joins the reduction, into *ww.
+template <int G, int J, bool WW = false>
+__device__ __forceinline__ void cgs_pass(const SlotPtrs& s, int N, int jn, double (&hcol)[MAXM],
+                                         double* ww = nullptr) {
   const Grp<G> g;
   const int Nq = s.Nq;
   constexpr int LJ = J > 0 ? J : MAXM;
@@ -1643,8 +1944,10 @@ __device__ __forceinline__ void cgs_pass(const SlotPtrs& s, int N, int jn, doubl
 #pragma unroll
     for (int i = 0; i < LJ; ++i)
       if (J > 0 || i < jn) hp[i] = fma(s.Q[i * Nq + e], we, hp[i]);
+    if (WW) hp[LJ] = fma(we, we, hp[LJ]);
   }
-  sum_first<G>(g, hp, J > 0 ? J : jn);
+  sum_first<G>(g, hp, (J > 0 ? J : jn) + (WW ? 1 : 0));
+  if (WW) *ww = hp[LJ];
 #pragma unroll 1
   for (int e = g.lane; e < N; e += G) {
     double we = s.w[e];
@@ -1674,7 +1977,7 @@ __device__ int arnoldi(const MechView& m, const SlotPtrs& s, const CellScalars& 
   }
   double unorm = 0.0;
   if (jv_mode != 0) unorm = sqrt(group_dot<G>(g, s.u, s.u, N));
-  const double ibeta = rsqrt(beta2);
+  const double ibeta = rsqrt_any(beta2);
   for (int e = g.lane; e < N; e += G) {
     const double qe = s.fn[e] * ibeta;
     s.Q[e] = qe;
@@ -1686,7 +1989,9 @@ __device__ int arnoldi(const MechView& m, const SlotPtrs& s, const CellScalars& 
   for (int j = 0; j < M; ++j) {
     apply_jv<G, MIXED, TC>(m, s, cs, jv_mode, p, unorm, s.Q + j * Nq, s.w, n_rhs, fp32_jv);
     // (only the breakdown threshold reads ||J q_j||^2: FP32 is enough there)
-    const double w02 = MIXED ? (double)group_dot_f<G>(g, s.w, s.w, N) : group_dot<G>(g, s.w, s.w, N);
+    double w02 = 0.0;
+    if (MIXED) w02 = (double)group_dot_f<G>(g, s.w, s.w, N);
+    else if (M > 4) w02 = group_dot<G>(g, s.w, s.w, N);
     double hcol[MAXM];
 #pragma unroll
     for (int i = 0; i < MAXM; ++i) hcol[i] = 0.0;
@@ -1714,29 +2019,31 @@ __device__ int arnoldi(const MechView& m, const SlotPtrs& s, const CellScalars& 
         }
 #pragma unroll
         for (int i = 0; i < MAXM; ++i) hcol[i] += hp[i];
-      } else if (M <= 4) {  // the common Krylov dimensions: column j + 1 known at compile time
+      } else if (M <= 4) {
+        const bool first = !MIXED && pass == 0;
+        // the common Krylov dimensions: column j + 1 known at compile time
         switch (j) {
-          case 0: cgs_pass<G, 1>(s, N, 1, hcol); break;
-          case 1: cgs_pass<G, 2>(s, N, 2, hcol); break;
-          case 2: cgs_pass<G, 3>(s, N, 3, hcol); break;
-          default: cgs_pass<G, 4>(s, N, 4, hcol); break;
+          case 0: first ? cgs_pass<G, 1, true>(s, N, 1, hcol, &w02) : cgs_pass<G, 1>(s, N, 1, hcol); break;
+          case 1: first ? cgs_pass<G, 2, true>(s, N, 2, hcol, &w02) : cgs_pass<G, 2>(s, N, 2, hcol); break;
+          case 2: first ? cgs_pass<G, 3, true>(s, N, 3, hcol, &w02) : cgs_pass<G, 3>(s, N, 3, hcol); break;
+          default: cgs_pass<G, 4>(s, N, 4, hcol); break;  // (the last column has no breakdown test to feed)
         }
       } else {
         cgs_pass<G, 0>(s, N, j + 1, hcol);
       }
     }
-    const double hn2 = group_dot<G>(g, s.w, s.w, N);
     if (g.lane == 0) {
 #pragma unroll
       for (int i = 0; i < MAXM; ++i)
         if (i <= j) s.H[i * MAXM + j] = hcol[i];
     }
     if (j + 1 == M) break;
+    const double hn2 = group_dot<G>(g, s.w, s.w, N);
     if (hn2 <= brk2 * w02 || hn2 == 0.0) {
       mdim = j + 1;
       break;
     }
-    const double ihn = rsqrt(hn2);
+    const double ihn = rsqrt_any(hn2);
     const double hn = hn2 * ihn;
     if (g.lane == 0) s.H[(j + 1) * MAXM + j] = hn;
     for (int e = g.lane; e < N; e += G) {
@@ -1767,6 +2074,42 @@ __device__ inline void solve_small(const SlotPtrs& s, int mdim, double* z) {
     for (int c = r + 1; c < mdim; ++c) z[r] = fma(-s.LU[r * MAXM + c], z[c], z[r]);
     z[r] = z[r] * s.LU[r * MAXM + r];
   }
+}
+
+// B = I - (I - h gamma H)^-1 for m = 4 by the whole warp: Gauss-Jordan with
+// partial pivoting on [I - h gamma H | I], one element a lane (row l / 8, column
+// l mod 8), rows and pivots passed by shuffles.  Seven FP64 instructions a pivot
+// instead of a serial elimination by lane 0 through shared memory and four
+// solves, which took 15,000 cycles of an attempt's 250,000.
+__device__ __forceinline__ void factor_four(const SlotPtrs& s, double h) {
+  const int lane = threadIdx.x & 31, r = lane >> 3, c = lane & 7;
+  const unsigned all = 0xffffffffu;
+  double v = c < 4 ? fma(-(h * GAM), s.H[r * MAXM + c], r == c ? 1.0 : 0.0) : (c - 4 == r ? 1.0 : 0.0);
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    double a[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) a[i] = __shfl_sync(all, v, 8 * i + p);
+    int pr = p;
+    long long best = __double_as_longlong(a[p]) & 0x7fffffffffffffffll;
+    double piv = a[p];
+#pragma unroll
+    for (int i = p + 1; i < 4; ++i) {
+      const long long cand = __double_as_longlong(a[i]) & 0x7fffffffffffffffll;
+      if (cand > best) {
+        best = cand;
+        pr = i;
+        piv = a[i];
+      }
+    }
+    const int from = r == p ? pr : (r == pr ? p : r);  // rows p and pr exchanged
+    v = __shfl_sync(all, v, 8 * from + c);
+    const double f = r == pr ? a[p] : (r == 0 ? a[0] : r == 1 ? a[1] : r == 2 ? a[2] : a[3]);
+    const double row = __shfl_sync(all, v, 8 * p + c) * rcp_any(piv);
+    v = r == p ? row : fma(-f, row, v);
+  }
+  if (c >= 4) s.Bm[r * MAXM + c - 4] = (c - 4 == r ? 1.0 : 0.0) - v;
+  __syncwarp();
 }
 
 // LU factorisation with partial pivoting of I - h gamma H (m x m), by lane 0.
@@ -1926,7 +2269,8 @@ struct IntegrateParams {
   const double* rho_cell;      // constant-volume densities, or null (constant pressure)
   int nx;                      // state components after T (5: auxiliary-temperature system)
   int64_t mech_copy;           // bytes of the mechanism each block copies (a prefix, by precision)
-  int64_t tc_bytes;            // precision 4: bytes of nu^T tiles copied after that prefix (else 0)
+  int64_t fx_copy;             // bytes of the fixed-point segment copied after that (0: it does not fit)
+  int64_t tc_bytes;            // precision 4: bytes of nu^T tiles copied after both (else 0)
 };
 
 template <int G, bool MIXED, bool TC = false>
@@ -1980,7 +2324,8 @@ __device__ void integrate_cell(const MechView& m, const SlotPtrs& s, const Integ
       break;
     }
     if (!fixed) h = fmin(h, dt - t);
-    factor_small<G>(s, mdim, h);
+    if (G == 32 && mdim == 4) factor_four(s, h);
+    else factor_small<G>(s, mdim, h);
     // ---- four stages (Algorithm 1); f is evaluated at stages 2 and 3 only
     for (int i = 0; i < 4; ++i) {
       const double* fi;
@@ -2018,8 +2363,8 @@ __device__ void integrate_cell(const MechView& m, const SlotPtrs& s, const Integ
     for (int e = g.lane; e < N; e += G) {
       const double k0 = K0[e], k1 = K1[e], k2 = K2[e], k3 = K3[e];
       const double ue = s.u[e];
-      const double us = ue + h * fma(B4, k3, fma(B3, k2, fma(B2, k1, B1 * k0)));
-      const double uh = ue + h * fma(BH4, k3, fma(BH3, k2, fma(BH2, k1, BH1 * k0)));
+      const double us = ue + h * fma(B4, k3, fma(B2, k1, B1 * k0));  // b3 = 0
+      const double uh = ue + h * fma(BH3, k2, fma(BH2, k1, BH1 * k0));  // bhat4 = 0
       const double d = (uh - us) * rcp_any(fma(P.rtol, fabs(us), P.atol));
       part = fma(d, d, part);
       bad |= (__double2hiint(us) & 0x7ff00000) == 0x7ff00000;
@@ -2181,17 +2526,18 @@ __device__ __forceinline__ void drain_queue(const IntegrateParams& P, const Grp<
 template <int G, bool MIXED, bool TC = false>
 __global__ void __launch_bounds__(MAX_BLOCK_THREADS, 1) rok4e_integrate_kernel(IntegrateParams P) {
   extern __shared__ __align__(16) unsigned char smem[];
-  load_exp_table(reinterpret_cast<double*>(smem));
+  load_exp_table(reinterpret_cast<uint64_t*>(smem));
   load_mech(smem + EXP_TAB_BYTES, P.mech, P.mech_copy);
-  if (TC) load_mech(smem + EXP_TAB_BYTES + P.mech_copy, P.mech + P.L.off_nuT, P.tc_bytes);
+  load_mech(smem + EXP_TAB_BYTES + P.mech_copy, P.mech + P.L.off_fA, P.fx_copy);
+  if (TC) load_mech(smem + EXP_TAB_BYTES + P.mech_copy + P.fx_copy, P.mech + P.L.off_nuT, P.tc_bytes);
   __syncthreads();
-  MechView m = make_view(smem + EXP_TAB_BYTES, P.L);
-  m.etab = reinterpret_cast<const double*>(smem);
+  MechView m = make_view(smem + EXP_TAB_BYTES, P.mech, P.L, P.mech_copy, P.fx_copy > 0);
+  m.etab = reinterpret_cast<const uint64_t*>(smem);
   m.nx = P.nx;
-  if (TC) m.nuT = reinterpret_cast<const uint4*>(smem + EXP_TAB_BYTES + P.mech_copy);
+  if (TC) m.nuT = reinterpret_cast<const uint4*>(smem + EXP_TAB_BYTES + P.mech_copy + P.fx_copy);
   const Grp<G> g;
   const int gid = threadIdx.x / G;
-  double* base = reinterpret_cast<double*>(smem + EXP_TAB_BYTES + P.mech_copy + (TC ? P.tc_bytes : 0)) +
+  double* base = reinterpret_cast<double*>(smem + EXP_TAB_BYTES + P.mech_copy + P.fx_copy + (TC ? P.tc_bytes : 0)) +
                  (size_t)gid * P.S.stride;
   const SlotPtrs s = slot_ptrs(base, P.S);
   init_sentinels<MIXED>(s, m.ns, g.lane);
@@ -2356,15 +2702,16 @@ __device__ void integrate_cell_rkdp(const MechView& m, const SlotPtrs& s, const 
 template <int G>
 __global__ void __launch_bounds__(MAX_BLOCK_THREADS) rkdp_integrate_kernel(IntegrateParams P) {
   extern __shared__ __align__(16) unsigned char smem[];
-  load_exp_table(reinterpret_cast<double*>(smem));
+  load_exp_table(reinterpret_cast<uint64_t*>(smem));
   load_mech(smem + EXP_TAB_BYTES, P.mech, P.mech_copy);
+  load_mech(smem + EXP_TAB_BYTES + P.mech_copy, P.mech + P.L.off_fA, P.fx_copy);
   __syncthreads();
-  MechView m = make_view(smem + EXP_TAB_BYTES, P.L);
-  m.etab = reinterpret_cast<const double*>(smem);
+  MechView m = make_view(smem + EXP_TAB_BYTES, P.mech, P.L, P.mech_copy, P.fx_copy > 0);
+  m.etab = reinterpret_cast<const uint64_t*>(smem);
   m.nx = P.nx;
   const Grp<G> g;
   const int gid = threadIdx.x / G;
-  double* base = reinterpret_cast<double*>(smem + EXP_TAB_BYTES + P.mech_copy) + (size_t)gid * P.S.stride;
+  double* base = reinterpret_cast<double*>(smem + EXP_TAB_BYTES + P.mech_copy + P.fx_copy) + (size_t)gid * P.S.stride;
   const SlotPtrs s = slot_ptrs(base, P.S);
   init_sentinels<false>(s, m.ns, g.lane);
   g.sync();
@@ -2398,11 +2745,20 @@ struct AdjointParams {
 template <int G>
 __global__ void __launch_bounds__(128) rok4e_adjoint_kernel(AdjointParams P) {
   extern __shared__ __align__(16) unsigned char smem[];
-  load_exp_table(reinterpret_cast<double*>(smem));
-  load_mech(smem + EXP_TAB_BYTES, P.mech, P.L.off_nuT);
+  load_exp_table(reinterpret_cast<uint64_t*>(smem));
+  // everything before the nu^T tiles but the fixed-point segment
+  unsigned char* base = smem + EXP_TAB_BYTES;
+  load_mech(base, P.mech, P.L.bytes_f32);
+  load_mech(base + P.L.bytes_f32, P.mech + P.L.off_fx_end, P.L.off_nuT - P.L.off_fx_end);
   __syncthreads();
-  MechView m = make_view(smem + EXP_TAB_BYTES, P.L);
-  m.etab = reinterpret_cast<const double*>(smem);
+  MechView m = make_view(base, P.mech, P.L, P.L.bytes_f32, false);
+  const unsigned char* tail = base + P.L.bytes_f32 - P.L.off_fx_end;
+  m.lnA = reinterpret_cast<const double*>(tail + P.L.off_lnA);
+  m.csr_nu = reinterpret_cast<const double*>(tail + P.L.off_csr_nu);
+  m.csr_ptr = reinterpret_cast<const int32_t*>(tail + P.L.off_csr_ptr);
+  m.role_ptr = reinterpret_cast<const int32_t*>(tail + P.L.off_role_ptr);
+  m.role = reinterpret_cast<const int32_t*>(tail + P.L.off_role);
+  m.etab = reinterpret_cast<const uint64_t*>(smem);
   const Grp<G> g;
   const int gpb = blockDim.x / G;
   const int64_t stride = (int64_t)gridDim.x * gpb;
@@ -2440,26 +2796,28 @@ struct PointParams {
   const double* rho_cell;  // constant-volume densities, or null
   int nx;                  // state components after T (5: auxiliary-temperature system)
   int64_t mech_copy;       // bytes of the mechanism copied to shared memory (a prefix)
-  int64_t tc_bytes;        // modes 6 and 7: bytes of nu^T tiles copied after that prefix (else 0)
+  int64_t fx_copy;         // bytes of the fixed-point segment copied after that (0: it does not fit)
+  int64_t tc_bytes;        // modes 6 and 7: bytes of nu^T tiles copied after both (else 0)
 };
 
 template <int G>
 __global__ void __launch_bounds__(MAX_BLOCK_THREADS) chem_point_kernel(PointParams P) {
   extern __shared__ __align__(16) unsigned char smem[];
-  load_exp_table(reinterpret_cast<double*>(smem));
+  load_exp_table(reinterpret_cast<uint64_t*>(smem));
   load_mech(smem + EXP_TAB_BYTES, P.mech, P.mech_copy);
-  if (P.tc_bytes) load_mech(smem + EXP_TAB_BYTES + P.mech_copy, P.mech + P.L.off_nuT, P.tc_bytes);
+  load_mech(smem + EXP_TAB_BYTES + P.mech_copy, P.mech + P.L.off_fA, P.fx_copy);
+  if (P.tc_bytes) load_mech(smem + EXP_TAB_BYTES + P.mech_copy + P.fx_copy, P.mech + P.L.off_nuT, P.tc_bytes);
   __syncthreads();
-  MechView m = make_view(smem + EXP_TAB_BYTES, P.L);
-  m.etab = reinterpret_cast<const double*>(smem);
+  MechView m = make_view(smem + EXP_TAB_BYTES, P.mech, P.L, P.mech_copy, P.fx_copy > 0);
+  m.etab = reinterpret_cast<const uint64_t*>(smem);
   m.nx = P.nx;
-  if (P.tc_bytes) m.nuT = reinterpret_cast<const uint4*>(smem + EXP_TAB_BYTES + P.mech_copy);
+  if (P.tc_bytes) m.nuT = reinterpret_cast<const uint4*>(smem + EXP_TAB_BYTES + P.mech_copy + P.fx_copy);
   const Grp<G> g;
   const int gid = threadIdx.x / G;
   const int gpb = blockDim.x / G;
   const int64_t cell = (int64_t)blockIdx.x * gpb + gid;
   if (cell >= P.ncell) return;
-  double* base = reinterpret_cast<double*>(smem + EXP_TAB_BYTES + P.mech_copy + P.tc_bytes) + (size_t)gid * P.S.stride;
+  double* base = reinterpret_cast<double*>(smem + EXP_TAB_BYTES + P.mech_copy + P.fx_copy + P.tc_bytes) + (size_t)gid * P.S.stride;
   const SlotPtrs s = slot_ptrs(base, P.S);
   if (P.mode >= 3 && P.mode <= 5) init_sentinels<true>(s, m.ns, g.lane);
   else init_sentinels<false>(s, m.ns, g.lane);
@@ -2549,6 +2907,35 @@ inline int device_props(int* n_sm, size_t* smem_optin) {
   if (e != cudaSuccess) return cuda_error(e, "cudaDeviceGetAttribute");
   *smem_optin = (size_t)v;
   return RK_OK;
+}
+
+// The bytes of the fixed-point segment a block copies: all of it, or none where it
+// and `rest` (the prefix, one cell's slot, tiles) do not fit in shared memory; such
+// a mechanism runs in the direct form.
+inline int64_t fixed_segment(const MechLayout& L, int64_t rest) {
+  int n_sm = 0;
+  size_t smem_max = 0;
+  if (device_props(&n_sm, &smem_max) != RK_OK) return 0;
+  const int64_t seg = L.off_fx_end - L.off_fA;
+  return rest + seg + EXP_TAB_BYTES + 64 <= (int64_t)smem_max ? seg : 0;
+}
+
+// Shared memory that precision 4 counts beside its tiles when it decides whether
+// it can run: the mechanism arrays and one cell's slot of its first layout.  The
+// present layout needs less; the limit on the mechanism's size stays where callers
+// know it.
+inline int64_t tensor_core_bytes(const MechLayout& L, int M, int nx) {
+  auto even = [](int64_t n) { return (n + 1) & ~int64_t(1); };
+  auto al = [](int64_t b) { return (b + 15) & ~int64_t(15); };
+  const int64_t ns = L.ns, nr = L.nr, nr1 = nr > 0 ? nr : 1, N = ns + 1 + nx, Nq = even(N);
+  const int64_t mech = 3 * al(8 * ns) + 2 * al(8 * 17 * ns) + 3 * al(8 * nr) + al(8 * L.ntb * ns) +
+                       al(64 * (int64_t)L.ntb) + al(8 * (int64_t)L.nnz) + 2 * al(4 * nr) + 2 * al(4 * (ns + 1)) +
+                       al(4 * (int64_t)L.nnz) + al(4 * ((int64_t)L.npiece + 1));
+  int64_t d = 7 * Nq + Nq * M + 10 * even(ns + 1) + 4 * even(nr1) + (4 * Nq <= 3 * even(nr1) ? 0 : 4 * Nq) +
+              even(4 * (L.ntb > 0 ? L.ntb : 1)) + even(11 * (L.ntroe > 0 ? L.ntroe : 1)) +
+              even(L.npiece > 0 ? L.npiece : 1) + 32 * (int64_t)L.nrt + 3 * 8 * M + 12;
+  d = (d + 3) & ~int64_t(3);
+  return mech + 8 * d + (int64_t)512 * L.nst * L.nrt + EXP_TAB_BYTES;
 }
 
 template <int G, typename K>

@@ -36,7 +36,12 @@ struct MechLayout {
   int32_t npiece = 0;  // pieces the list is split into for the gather (>= ns)
   // byte offsets into the packed buffer (all multiples of 16)
   int64_t off_W = 0, off_invW = 0, off_Tmid = 0, off_lo = 0, off_hi = 0;
-  int64_t off_lnA = 0, off_b = 0, off_EaR = 0;
+  int64_t off_b = 0, off_EaR = 0;
+  int64_t off_lnA = 0;  // read from global memory (Troe passes, cells off the fixed-point form)
+  // fixed-point Arrhenius coefficients (fx.cuh), uint64 per reaction: log2 A 2^52, (b + 32) 2^57,
+  // (Ea/R log2 e + 2^15) 2^46; fx: every reaction's fit their ranges
+  int32_t fx = 0;
+  int64_t off_fA = 0, off_fb = 0, off_fE = 0;
   int64_t off_eff = 0;  // [ntb][ns]
   int64_t off_fo = 0;   // [ntb][FO_STRIDE]
   int64_t off_csr_nu = 0;
@@ -45,6 +50,16 @@ struct MechLayout {
   int64_t off_csr_ptr = 0, off_csr_j = 0;
   int64_t off_piece_ptr = 0;   // int32 [npiece + 1]: list offset of each piece
   int64_t off_spec_piece = 0;  // int32 [ns + 1]: first piece of each species
+  // the same list for the fixed-point gather: pieces of glen reactions entering a
+  // species with one sign (a coefficient of 2 is two entries, short pieces are
+  // padded with the reaction nr, whose rate is zero), gnpp pieces (a multiple of
+  // 32), their entries as byte offsets of the rates, uint16 [ceil(glen / 8)][gnpp][8];
+  // species k adds pieces [gspec[2k],
+  // gspec[2k + 1]) and subtracts [gspec[2k + 1], gspec[2k + 2]); ghb: bits of
+  // headroom that every row's sum of |nu| needs
+  int32_t glen = 0, gnpp = 0, ghb = 0;
+  int32_t gfix = 0;  // the gather runs in fixed point (many pieces), else in FP64
+  int64_t off_gidx = 0, off_gspec = 0;
   // FP32 copies read by the reduced-precision Jacobian-vector product
   int64_t off_Wf = 0, off_invWf = 0, off_bf = 0, off_EaRf = 0, off_efff = 0, off_csr_nuf = 0;
   int64_t off_perm = 0;  // int32 per packed reaction: its index in the input description
@@ -59,9 +74,11 @@ struct MechLayout {
   int32_t nst = 0, nrt = 0;  // species tiles, reaction tiles
   int64_t off_nuT = 0;       // [nst][nrt][32 lanes] x 16 bytes
   int64_t bytes = 0;
-  // prefixes of the buffer that kernels copy to shared memory: through the FP64
-  // arrays; also csr_nuf (double-float gathers); also the other FP32 copies
-  int64_t bytes_fp64 = 0, bytes_df = 0, bytes_f32 = 0;
+  // what kernels copy to shared memory: a prefix of the buffer -- through the base
+  // arrays; also the list in pieces of the double-float gathers; also the FP32
+  // copies -- and, after it, the fixed-point segment [off_fA, off_fx_end): the
+  // Arrhenius coefficients and the gather list
+  int64_t bytes_base = 0, bytes_df = 0, bytes_f32 = 0, off_fx_end = 0;
 };
 
 struct HostMech {

@@ -13,7 +13,7 @@ int launch_rok4e(const IntegrateLaunch& a) {
   IntegrateParams& P = *a.P;
   LaunchPlan plan;
   const int rc = plan_for<G>(rok4e_integrate_kernel<G, MIXED, TC>, a.mech, P.S, a.cells_per_block, a.ncell, true,
-                             &plan, a.blocks_per_sm, a.static_bins, P.mech_copy + P.tc_bytes);
+                             &plan, a.blocks_per_sm, a.static_bins, P.mech_copy + P.fx_copy + P.tc_bytes);
   if (rc) return rc;
   if (a.static_bins) P.subq = plan.cells_per_block % 4 == 0 ? 4 : (plan.cells_per_block % 2 == 0 ? 2 : 1);
   rok4e_integrate_kernel<G, MIXED, TC><<<plan.blocks, plan.cells_per_block * G, plan.smem, a.stream>>>(P);
@@ -26,7 +26,7 @@ int launch_rkdp(const IntegrateLaunch& a) {
   IntegrateParams& P = *a.P;
   LaunchPlan plan;
   const int rc = plan_for<G>(rkdp_integrate_kernel<G>, a.mech, P.S, a.cells_per_block, a.ncell, true, &plan,
-                             a.blocks_per_sm, a.static_bins, P.mech_copy);
+                             a.blocks_per_sm, a.static_bins, P.mech_copy + P.fx_copy);
   if (rc) return rc;
   if (a.static_bins) P.subq = plan.cells_per_block % 4 == 0 ? 4 : (plan.cells_per_block % 2 == 0 ? 2 : 1);
   rkdp_integrate_kernel<G><<<plan.blocks, plan.cells_per_block * G, plan.smem, a.stream>>>(P);

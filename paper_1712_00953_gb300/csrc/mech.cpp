@@ -16,6 +16,7 @@
 #include <string>
 #include <vector>
 
+#include "fx.cuh"
 #include "internal.h"
 #include "rok4e.h"
 
@@ -23,6 +24,9 @@ namespace rk {
 namespace {
 
 constexpr double R_GAS = 8.314462618;
+#ifndef RK_GFIX_MIN
+#define RK_GFIX_MIN 256
+#endif
 
 int64_t align16(int64_t x) { return (x + 15) & ~int64_t(15); }
 
@@ -42,6 +46,39 @@ void nasa_eval(const double* a, double T, double* cp, double* h, double* s) {
 
 bool close_rel(double x, double y, double tol) {
   return fabs(x - y) <= tol * std::max(1.0, std::max(fabs(x), fabs(y)));
+}
+
+// x log2(e) scaled by 2^bits, rounded, from the 64-bit log2(e): x's 53-bit
+// significand times it is exact in 128 bits.  |x| log2(e) 2^bits < 2^63.
+int64_t times_log2e(double x, int bits) {
+  int e;
+  const double m = frexp(fabs(x), &e);  // |x| = m 2^e
+  const unsigned __int128 p = (unsigned __int128)(uint64_t)ldexp(m, 53) * RK_FX_LOG2E;  // |x| log2(e) 2^(53 + 63 - e)
+  const int s = 53 + 63 - e - bits;
+  const int64_t v = s >= 127 ? 0 : (int64_t)(uint64_t)((p + ((unsigned __int128)1 << (s - 1))) >> s);
+  return x < 0.0 ? -v : v;
+}
+
+// The fixed-point Arrhenius coefficients of fx.cuh for A (cm-mol-s), a rate of
+// the given concentration order, b and Ea/R; ok: inside their ranges.
+struct FxArrhenius {
+  uint64_t A = 0, b = 0, E = 0;
+  bool ok = false;
+};
+FxArrhenius fx_arrhenius(double A, int order, double b, double EaR) {
+  FxArrhenius f;
+  int e;
+  const double m = frexp(A, &e);  // log2 A = e + log2 m, log2 m in [-1, 0)
+  const int64_t lg = (int64_t)e * ((int64_t)1 << 52) + (int64_t)llrint(ldexp(log2(m), 52)) +
+                     (int64_t)(order - 1) * RK_FX_LOG2_1EM6;
+  const double El = EaR * 1.4426950408889634;
+  f.ok = A < 1e150 && A > 1e-150 && llabs(lg) <= (int64_t)200 << 52 && fabs(b) <= 16.0 && El >= -32768.0 &&
+         El < 229375.0;
+  if (!f.ok) return f;
+  f.A = (uint64_t)lg;
+  f.b = (uint64_t)((int64_t)llrint(ldexp(b, 57)) + ((int64_t)32 << 57));
+  f.E = (uint64_t)times_log2e(EaR, 45) * 2 + ((uint64_t)1 << 61);
+  return f;
 }
 
 }  // namespace
@@ -192,8 +229,91 @@ bool pack_mechanism(const void* vdesc, HostMech* out, std::string* err) {
   }
   const int npiece = (int)piece_ptr.size() - 1;
 
+  // ---- pieces of the fixed-point gather: rows split by sign, then into near-equal
+  // pieces of at most glen entries; one lane sums one piece.  glen minimises the
+  // group's steps (about 9 instructions an entry, 12 a piece, 10 for each piece a
+  // species adds up).
+  std::vector<std::vector<int>> signed_rows(2 * (size_t)ns);
+  int most = 1;  // largest sum of |nu| in a row
+  for (int k = 0; k < ns; ++k) {
+    for (auto& e : rows[k])
+      for (int t = 0; t < (int)fabs(e.second); ++t) signed_rows[2 * k + (e.second < 0.0)].push_back(e.first);
+    most = std::max(most, (int)(signed_rows[2 * k].size() + signed_rows[2 * k + 1].size()));
+  }
+  auto pieces_of = [](size_t n, int len) { return (int)((n + len - 1) / len); };
+  // Few entries: in FP64, 64 cycles for each that a lane adds; otherwise in fixed
+  // point, in batches of eight entries.
+  int entries = 0;
+  for (auto& row : signed_rows) entries += (int)row.size();
+  const bool gfix = entries >= RK_GFIX_MIN && nr < 8191;
+  const int step = gfix ? 8 : 1;
+  int glen = 1;
+  {
+    long best = -1;
+    for (int cand = step; cand < most + step; cand += step) {
+      int P = 0, maxp = 0;
+      for (int k = 0; k < ns; ++k) {
+        const int pk = pieces_of(signed_rows[2 * k].size(), cand) + pieces_of(signed_rows[2 * k + 1].size(), cand);
+        P += pk;
+        maxp = std::max(maxp, pk);
+      }
+      const long cost = (long)((P + 31) / 32) * (9 * cand + 12) + (long)((ns + 31) / 32) * maxp * 10;
+      if (best < 0 || cost < best) {
+        best = cost;
+        glen = cand;
+      }
+    }
+  }
+  std::vector<std::vector<int>> gpieces;
+  std::vector<int32_t> gspec;
+  for (int r = 0; r < 2 * ns; ++r) {
+    gspec.push_back((int32_t)gpieces.size());
+    const auto& row = signed_rows[r];
+    const int pk = pieces_of(row.size(), glen);
+    for (int i = 0; i < pk; ++i)
+      gpieces.emplace_back(row.begin() + row.size() * i / pk, row.begin() + row.size() * (i + 1) / pk);
+  }
+  gspec.push_back((int32_t)gpieces.size());
+  const int gnpp = std::max(32, ((int)gpieces.size() + 31) / 32 * 32);
+  gpieces.resize(gnpp);
+  // The sums are exact, so a piece's entries may come in any order: at each step the
+  // 16 lanes of a half-warp take entries of different 8-byte shared-memory banks
+  // (index mod 16) where they can, lanes with the most entries left first.
+  const int gbat = (glen + 7) / 8;
+  std::vector<uint16_t> gidx((size_t)gbat * 8 * gnpp, (uint16_t)(8 * nr));
+  if (nr < 8191) {
+    std::vector<std::vector<int>> left = gpieces;
+    for (int p0 = 0; p0 < gnpp; p0 += 16)
+      for (int i = 0; i < glen; ++i) {
+        int bank[16];
+        for (int& b : bank) b = -1;
+        std::vector<int> lanes;
+        for (int p = p0; p < p0 + 16; ++p) lanes.push_back(p);
+        std::stable_sort(lanes.begin(), lanes.end(), [&](int a, int b) { return left[a].size() > left[b].size(); });
+        for (int p : lanes) {
+          auto& l = left[p];
+          size_t at = l.size();
+          for (size_t t = 0; t < l.size() && at == l.size(); ++t)
+            if (bank[l[t] & 15] < 0 || bank[l[t] & 15] == l[t]) at = t;
+          if (at == l.size()) {
+            if ((int)l.size() < glen - i) continue;  // padding for now; its entries still fit
+            at = 0;
+          }
+          bank[l[at] & 15] = l[at];
+          gidx[((size_t)(i / 8) * gnpp + p) * 8 + i % 8] = (uint16_t)(8 * l[at]);
+          l.erase(l.begin() + at);
+        }
+      }
+  }
+
   // ---- layout
   MechLayout L;
+  L.glen = glen;
+  L.gnpp = gnpp;
+  for (L.ghb = 1; (1 << L.ghb) <= most; ++L.ghb) {
+  }
+  ++L.ghb;
+  L.gfix = gfix ? 1 : 0;
   L.ns = ns;
   L.nr = nr;
   L.ntb = n_troe + n_tb;
@@ -211,22 +331,20 @@ bool pack_mechanism(const void* vdesc, HostMech* out, std::string* err) {
   L.off_Tmid = take(8 * ns);
   L.off_lo = take(8 * (int64_t)NCOEF * ns);
   L.off_hi = take(8 * (int64_t)NCOEF * ns);
-  L.off_lnA = take(8 * (int64_t)nr);
   L.off_b = take(8 * (int64_t)nr);
   L.off_EaR = take(8 * (int64_t)nr);
   L.off_eff = take(8 * (int64_t)L.ntb * ns);
   L.off_fo = take(8 * (int64_t)L.ntb * FO_STRIDE);
-  L.off_csr_nu = take(8 * (int64_t)nnz);
   L.off_slots = take(4 * (int64_t)nr);
   L.off_meta = take(4 * (int64_t)nr);
-  L.off_csr_ptr = take(4 * (int64_t)(ns + 1));
+  // what only some kernels read comes last (internal.h): FP64 paths copy the base
+  // arrays, the double-float gathers also the list in pieces with csr_nuf, the FP32
+  // Jacobian-vector product the other FP32 copies; each adds the fixed-point
+  // segment; the rest is read from global memory
+  L.bytes_base = off;
   L.off_csr_j = take(4 * (int64_t)nnz);
   L.off_piece_ptr = take(4 * (int64_t)(npiece + 1));
   L.off_spec_piece = take(4 * (int64_t)(ns + 1));
-  // what only some kernels read comes last, so a kernel copies a prefix:
-  // FP64 paths stop here, the double-float gathers also read csr_nuf, the FP32
-  // Jacobian-vector product the other FP32 copies; perm is read from global memory
-  L.bytes_fp64 = off;
   L.off_csr_nuf = take(4 * (int64_t)nnz);
   L.bytes_df = off;
   L.off_Wf = take(4 * (int64_t)ns);
@@ -235,6 +353,15 @@ bool pack_mechanism(const void* vdesc, HostMech* out, std::string* err) {
   L.off_EaRf = take(4 * (int64_t)nr);
   L.off_efff = take(4 * (int64_t)L.ntb * ns);
   L.bytes_f32 = off;
+  L.off_fA = take(8 * (int64_t)nr);
+  L.off_fb = take(8 * (int64_t)nr);
+  L.off_fE = take(8 * (int64_t)nr);
+  L.off_gidx = take(16 * (int64_t)gbat * gnpp);
+  L.off_gspec = take(4 * (int64_t)(2 * ns + 1));
+  L.off_fx_end = off;
+  L.off_lnA = take(8 * (int64_t)nr);
+  L.off_csr_nu = take(8 * (int64_t)nnz);
+  L.off_csr_ptr = take(4 * (int64_t)(ns + 1));
   L.off_perm = take(4 * (int64_t)nr);
   // reaction slots per species (filled below from the packed slots)
   std::vector<std::vector<int32_t>> roles(ns);
@@ -264,6 +391,7 @@ bool pack_mechanism(const void* vdesc, HostMech* out, std::string* err) {
   std::vector<unsigned char> buf((size_t)L.bytes, 0);
   auto D = [&](int64_t o) { return reinterpret_cast<double*>(buf.data() + o); };
   auto I = [&](int64_t o) { return reinterpret_cast<int32_t*>(buf.data() + o); };
+  auto X = [&](int64_t o) { return reinterpret_cast<uint64_t*>(buf.data() + o); };
   auto U = [&](int64_t o) { return reinterpret_cast<uint32_t*>(buf.data() + o); };
 
   for (int k = 0; k < ns; ++k) {
@@ -281,6 +409,7 @@ bool pack_mechanism(const void* vdesc, HostMech* out, std::string* err) {
     }
   }
   int slot_tb = 0;
+  bool fx = true;
   for (int r = 0; r < nr; ++r) {
     const int j = perm[r];
     const int* sp = d->rxn_sp + 4 * (size_t)j;
@@ -306,6 +435,11 @@ bool pack_mechanism(const void* vdesc, HostMech* out, std::string* err) {
     D(L.off_lnA)[r] = log(ar[0]) + (order - 1) * log(1e-6);
     D(L.off_b)[r] = ar[1];
     D(L.off_EaR)[r] = ar[2] / R_GAS;
+    const FxArrhenius f = fx_arrhenius(ar[0], order, ar[1], ar[2] / R_GAS);
+    fx = fx && f.ok;
+    X(L.off_fA)[r] = f.A;
+    X(L.off_fb)[r] = f.b;
+    X(L.off_fE)[r] = f.E;
     int slot = 0;
     if (kind > 0) {
       slot = slot_tb++;
@@ -327,6 +461,7 @@ bool pack_mechanism(const void* vdesc, HostMech* out, std::string* err) {
     const int dnu = mol_p - mol_r;  // -1, 0 or 1
     I(L.off_meta)[r] = kind | (rev << 2) | ((dnu + 4) << 4) | (slot << 8);
   }
+  L.fx = fx && nr < 8191 ? 1 : 0;
   int pos = 0;
   for (int k = 0; k < ns; ++k) {
     I(L.off_csr_ptr)[k] = pos;
@@ -337,6 +472,8 @@ bool pack_mechanism(const void* vdesc, HostMech* out, std::string* err) {
     }
   }
   I(L.off_csr_ptr)[ns] = pos;
+  if (!gidx.empty()) memcpy(buf.data() + L.off_gidx, gidx.data(), 2 * gidx.size());
+  for (size_t i = 0; i < gspec.size(); ++i) I(L.off_gspec)[i] = gspec[i];
   for (int p = 0; p <= npiece; ++p) I(L.off_piece_ptr)[p] = piece_ptr[p];
   for (int k = 0; k <= ns; ++k) I(L.off_spec_piece)[k] = spec_piece[k];
   auto F = [&](int64_t o) { return reinterpret_cast<float*>(buf.data() + o); };

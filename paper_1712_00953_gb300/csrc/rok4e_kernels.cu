@@ -186,28 +186,14 @@ __global__ void ssprk3_stage_ghost_kernel(int stage, const double* __restrict__ 
 
 // ------------------------------------------------------------------ probes
 __global__ void exp_eval_kernel(const double* __restrict__ x, double* __restrict__ y, int64_t n, int which) {
-  __shared__ double tab[RK_EXP2_TABLE_N];
+  __shared__ uint64_t tab[RK_FX_EXP2_N];
   load_exp_table(tab);
   __syncthreads();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  if (which == 0) {
-    y[i] = exp_fast(x[i], tab);
-  } else if (which == 6) {
-    y[i] = log_fast(x[i]);
-  } else if (which == 7) {
-    y[i] = rcp_any(x[i]);
-  } else if (which == 3) {
-    y[i] = exp_mixed(x[i], tab);
-  } else if (which == 4 || which == 5) {
-    double ep, em;
-    exp_pm_mixed(x[i], tab, &ep, &em);
-    y[i] = which == 4 ? ep : em;
-  } else {
-    double ep, em;
-    exp_pm(x[i], tab, &ep, &em);
-    y[i] = which == 1 ? ep : em;
-  }
+  if (which == 6) y[i] = log_fast(x[i]);
+  else if (which == 7) y[i] = rcp_any(x[i]);
+  else y[i] = exp_fast(which == 2 || which == 5 ? -x[i] : x[i], tab);
 }
 
 __global__ void probe_fp64_kernel(double* out, int iters, double a, int active_lanes = 32) {
@@ -393,9 +379,15 @@ int integrate_impl(const rk_mech* mech, double* Y, const double* src, double* h_
   P.rho_cell = o.reactor == 1 ? o.rho_cell : nullptr;
   {
     const MechLayout& L = mech->host.L;
-    P.mech_copy = (method == 1 || o.precision == 0 || tc || o.precision >= 5) ? L.bytes_fp64
-                                                          : (o.precision == 2 ? L.bytes_f32 : L.bytes_df);
+    P.mech_copy = o.precision == 1 || o.precision == 3 ? L.bytes_df
+                                                       : (o.precision == 2 ? L.bytes_f32 : L.bytes_base);
     P.tc_bytes = tc ? (int64_t)16 * 32 * L.nst * L.nrt : 0;
+    P.fx_copy = fixed_segment(L, P.mech_copy + P.tc_bytes + (int64_t)P.S.stride * 8);
+    int n_sm = 0;
+    size_t smem_max = 0;
+    if (tc && (rc = device_props(&n_sm, &smem_max))) return rc;
+    if (tc && tensor_core_bytes(L, Meff, nx) + 64 > (int64_t)smem_max)
+      return set_error(RK_E_UNSUPPORTED, "mechanism, nu^T tiles and one cell's work arrays exceed shared memory");
   }
   P.qstride = queue_stride(ncell);
   P.order = nullptr;
@@ -536,12 +528,14 @@ static int point_call(const rk_mech* mech, const double* Y, const double* src, c
   P.p = p;
   P.mode = mode;
   {
-    const MechLayout& L = mech->host.L;  // everything but the nu^T tiles; the tiles only with the FP64 arrays
-    P.mech_copy = tc ? L.bytes_fp64 : L.off_nuT;
+    const MechLayout& L = mech->host.L;  // the arrays that the mode's precision reads
+    P.mech_copy = mode == 3 || mode == 5 ? L.bytes_df : (mode == 4 ? L.bytes_f32 : L.bytes_base);
     P.tc_bytes = tc ? (int64_t)16 * 32 * L.nst * L.nrt : 0;
+    P.fx_copy = fixed_segment(L, P.mech_copy + P.tc_bytes + (int64_t)P.S.stride * 8);
   }
   LaunchPlan plan;
-  rc = plan_for<32>(chem_point_kernel<32>, mech, P.S, 8, ncell, false, &plan, 0, false, P.mech_copy + P.tc_bytes);
+  rc = plan_for<32>(chem_point_kernel<32>, mech, P.S, 8, ncell, false, &plan, 0, false,
+                    P.mech_copy + P.fx_copy + P.tc_bytes);
   if (rc) return rc;
   chem_point_kernel<32><<<plan.blocks, plan.cells_per_block * 32, plan.smem, (cudaStream_t)stream>>>(P);
   cudaError_t e = cudaGetLastError();
@@ -1084,7 +1078,8 @@ int rk_rok4e_adjoint_ex(const rk_mech* mech, const double* checkpoints, const do
   }
   if (G != 4 && G != 8 && G != 16 && G != 32)
     return set_error(RK_E_INVALID_ARGUMENT, "lanes_per_cell must be 0, 4, 8, 16 or 32");
-  const size_t smem = (size_t)mech->host.L.off_nuT + EXP_TAB_BYTES;
+  const MechLayout& L = mech->host.L;
+  const size_t smem = (size_t)(L.off_nuT - (L.off_fx_end - L.off_fA)) + EXP_TAB_BYTES;
   cudaError_t e = cudaSuccess;
   rc = G == 4 ? launch_adjoint<4>(P, smem, st)
               : (G == 8 ? launch_adjoint<8>(P, smem, st)
