@@ -68,15 +68,19 @@ constexpr double BH1 = -0.217819895945721, BH2 = 1.03130847478467, BH3 = 0.18651
 constexpr double PI_ALPHA = 0.7 / 4.0, PI_BETA = 0.4 / 4.0;
 constexpr double FAC_MIN = 0.2, FAC_MAX = 5.0, SAFETY = 0.8, ERR_FLOOR = 1e-10;
 constexpr double BREAKDOWN_TOL = 1e-12, T_END_TOL = 1e-12, H_MIN_FRAC = 1e-12;
-#ifndef RK_UNROLL
-#define RK_UNROLL 2
-#endif
+constexpr float LOG2_ERR_FLOOR = -33.219281f;  // log2(1e-10)
 constexpr int G_OVERFLOW_HI = 0x40654000;  // high word of 170.0
 constexpr int MAXM = RK_MAX_KRYLOV;
 // Threads per block of the per-cell kernels: 8 warps, so each thread may hold
 // up to 255 registers (one such block fills an SM's register file, which the
 // cells' shared-memory slots limit the SM to anyway).
 constexpr int MAX_BLOCK_THREADS = 256;
+#ifndef RK_WIDE_MIN
+#define RK_WIDE_MIN 8
+#endif
+constexpr int WIDE_MIN_CELLS_PER_SM = RK_WIDE_MIN;
+// the explicit integrator fits 128 registers with one warp per cell
+constexpr int rkdp_threads(int G) { return G == 32 ? 512 : MAX_BLOCK_THREADS; }
 constexpr int EXP_TAB_BYTES = RK_FX_EXP2_N * 8;  // leads the dynamic shared memory
 
 static __constant__ uint64_t c_exp2_table[RK_FX_EXP2_N] = {RK_FX_EXP2_VALUES};
@@ -250,11 +254,11 @@ struct MechView {
 };
 
 // The view of a block that copied the buffer's first `prefix` bytes to base and,
-// with fxseg, the fixed-point segment after them; lnA, csr_ptr and csr_nu are read
+// the segment after them (fxseg: its fixed-point part too); lnA, b, Ea/R, csr_ptr and csr_nu are read
 // from the whole buffer in global memory, gbase.
 __host__ __device__ inline MechView make_view(const unsigned char* base, const unsigned char* gbase,
                                               const MechLayout& L, int64_t prefix, bool fxseg) {
-  const unsigned char* fbase = base + prefix - L.off_fA;  // the segment's arrays sit at fbase + their offset
+  const unsigned char* fbase = base + prefix - L.off_lo;  // the segment's arrays sit at fbase + their offset
   MechView m;
   m.ns = L.ns;
   m.nr = L.nr;
@@ -265,16 +269,16 @@ __host__ __device__ inline MechView make_view(const unsigned char* base, const u
   m.W = reinterpret_cast<const double*>(base + L.off_W);
   m.invW = reinterpret_cast<const double*>(base + L.off_invW);
   m.Tmid = reinterpret_cast<const double*>(base + L.off_Tmid);
-  m.lo = reinterpret_cast<const double*>(base + L.off_lo);
-  m.hi = reinterpret_cast<const double*>(base + L.off_hi);
+  m.lo = reinterpret_cast<const double*>(fbase + L.off_lo);
+  m.hi = reinterpret_cast<const double*>(fbase + L.off_hi);
   m.lnA = reinterpret_cast<const double*>(gbase + L.off_lnA);
   m.fA = reinterpret_cast<const uint64_t*>(fbase + L.off_fA);
   m.fb = reinterpret_cast<const uint64_t*>(fbase + L.off_fb);
   m.fE = reinterpret_cast<const uint64_t*>(fbase + L.off_fE);
   m.fx = fxseg && L.fx != 0;
   m.gcsr_j = reinterpret_cast<const int32_t*>(gbase + L.off_csr_j);
-  m.bexp = reinterpret_cast<const double*>(base + L.off_b);
-  m.EaR = reinterpret_cast<const double*>(base + L.off_EaR);
+  m.bexp = reinterpret_cast<const double*>(gbase + L.off_b);
+  m.EaR = reinterpret_cast<const double*>(gbase + L.off_EaR);
   m.eff = reinterpret_cast<const double*>(base + L.off_eff);
   m.fo = reinterpret_cast<const double*>(base + L.off_fo);
   m.csr_nu = reinterpret_cast<const double*>(gbase + L.off_csr_nu);
@@ -310,7 +314,7 @@ __host__ __device__ inline MechView make_view(const unsigned char* base, const u
 struct SlotLayout {
   int N, ns, nr, ntb, M;
   int u, src, fn, arg, fr, F, w, Q, K;        // N-vectors (Q: M of them, K: 4)
-  int C, dC, cp, hRT, dcp, gRT, E, Einv, CE, om;  // species (+1 sentinel entry)
+  int C, dC, cp, hRT, gRT, E, CE, om;  // species (+1 sentinel entry)
   int q, kc, krc, qT;                         // reactions (qT: d q_j / dT at u_n, for J v)
   int tb;                                     // [ntb][4]: [M], dk/d[M], dlnk/dT, 1/Kc
   int tro;                                    // [11][ntroe]: Troe falloff scratch
@@ -319,17 +323,20 @@ struct SlotLayout {
   int dig;                                    // BF16 digits of q, [8][16 nrt] (precision 4, else -1)
   int fj;   // precision 6: FP32 species factors of the J v, when they do not fit beside the
             // FP32 reaction caches in the kc/krc/qT storage (else -1)
-  int H, LU, piv, red, Bm;                    // small (Bm: I - (I - h gamma H)^-1)
+  int H, LU, piv, Bm;                    // small (Bm: I - (I - h gamma H)^-1)
   int fbase;  // FP32 region (mixed precision only), offset in doubles
   int fC, fdC, fh, fcp, fdcp, fom, fq, fkc, fkr, ftb, fQ, fw, fpart;  // offsets in floats from fbase
   int stride;
 };
 
 // mixed: the FP32 arrays of precision levels 1 and 2; df: the double-float
-// species arrays of precision level 3 (left out otherwise, which lets a 53-species
-// mechanism keep 7 cells per block instead of 6).
-inline SlotLayout make_slot(const MechLayout& L, int M, bool mixed = false, int nx = 0, bool df = false,
-                            bool tc = false, bool f32jv = false) {
+// species arrays of precision level 3; src: the slot keeps the cell's source.
+// Arrays whose lives do not meet share storage, so that an SM holds more cells
+// (a warp each): with 19.2 kB at 53 species / 325 reactions instead of 22.7, and a
+// mechanism copy of 22 instead of 48 kB, ten instead of eight.
+enum SlotKind { SLOT_ROK4E, SLOT_RKDP, SLOT_POINT };
+inline SlotLayout make_slot(const MechLayout& L, int M, SlotKind kind, bool mixed, int nx, bool df, bool tc,
+                            bool f32jv, bool src) {
   SlotLayout s;
   s.N = L.ns + 1 + nx;
   s.ns = L.ns;
@@ -344,24 +351,25 @@ inline SlotLayout make_slot(const MechLayout& L, int M, bool mixed = false, int 
   };
   const int N = s.N, ns1 = L.ns + 1;
   s.u = take(N);
-  s.src = take(N);
+  s.src = src ? take(N) : -1;
   s.fn = take(N);
   s.arg = take(N);
-  s.fr = take(N);
-  s.F = take(N);
+  // a stage's f may overwrite its argument, except in the auxiliary-temperature
+  // system, whose T row reads the argument after the species rows are written
+  s.fr = kind != SLOT_RKDP && nx > 0 ? take(N) : s.arg;
+  s.F = kind != SLOT_ROK4E ? take(N) : -1;  // RKDP: a stage vector; point kernel: V
   s.w = take(N);
   const int Nq = (N + 1) & ~1;  // stride between Krylov / stage vectors
   s.Q = take(Nq * M);
-  s.C = take(ns1);
+  s.CE = take(ns1);
+  // C is read beside CE only by third-body sums and the reduced-precision J v
+  s.C = L.ntb > 0 || mixed || df || f32jv ? take(ns1) : s.CE;
   s.dC = take(ns1);
   s.cp = take(ns1);
   s.hRT = take(ns1);
-  s.dcp = take(ns1);
   s.gRT = take(ns1);
   s.E = take(ns1);
-  s.Einv = take(ns1);
-  s.CE = take(ns1);
-  s.om = take(ns1);
+  s.om = s.gRT;  // w is kept (caching evaluation) when the Gibbs factors are done with
   // reactions, and entry nr: the zero rate that pads the gather's pieces
   s.q = take(L.nr + 1);
   s.kc = take(L.nr + 1);
@@ -375,18 +383,21 @@ inline SlotLayout make_slot(const MechLayout& L, int M, bool mixed = false, int 
   s.K = (4 * Nq <= 2 * nr_even) ? s.kc : take(4 * Nq);
   s.tb = take(4 * (L.ntb > 0 ? L.ntb : 1));
   s.tro = take(11 * (L.ntroe > 0 ? L.ntroe : 1));
-  s.part = take(2 * L.gnpp > L.npiece ? 2 * L.gnpp : L.npiece);  // (hi, lo) words of the fixed-point gather
+  // the gather's pieces ((hi, lo) words in fixed point); LU and its pivots, used
+  // only to form B, share them
+  int np = 2 * L.gnpp > L.npiece ? 2 * L.gnpp : L.npiece;
+  np = np > (M + 1) * MAXM ? np : (M + 1) * MAXM;
+  s.part = take(np);
   s.C2 = df ? take(ns1) : -1;
   s.dC2 = df ? take(ns1) : -1;
   s.dig = tc ? take(2 * 16 * L.nrt) : -1;  // 8 x 16 nrt BF16 = 2 x 16 nrt doubles
   // precision 6 keeps its FP32 reaction caches in the first half of the kc/krc/qT
-  // storage and its 8 FP32 species arrays in the second half when they fit there
-  s.fj = (f32jv && 8 * ns1 > 3 * nr_even) ? take((8 * ns1 + 1) / 2) : -1;
+  // storage and its 6 FP32 species arrays in the second half when they fit there
+  s.fj = (f32jv && 6 * ns1 > 3 * nr_even) ? take((6 * ns1 + 1) / 2) : -1;
   // M x M matrices stored with row stride MAXM: M rows
   s.H = take(M * MAXM);
-  s.LU = take(M * MAXM);
-  s.piv = take(MAXM);
-  s.red = take(4);
+  s.LU = s.part;
+  s.piv = s.part + M * MAXM;
   s.Bm = take(M * MAXM);
   s.fbase = o;
   int fo = 0;
@@ -415,6 +426,19 @@ inline SlotLayout make_slot(const MechLayout& L, int M, bool mixed = false, int 
   o += (fo + 1) / 2;
   s.stride = (o + 3) & ~3;
   return s;
+}
+
+// Float with the value of x truncated, and back, by integer moves (a conversion
+// takes the FP64 unit as long as an FP64 operation): below 2^-126 zero, from 2^127
+// infinity; x >= 0.
+__device__ __forceinline__ float float_bits(double x) {
+  const int hi = __double2hiint(x), e = hi >> 20;
+  const float f = __int_as_float(((hi - (896 << 20)) << 3) | (int)((unsigned)__double2loint(x) >> 29));
+  return e < 897 ? 0.f : (e >= 1150 ? INFINITY : f);
+}
+__device__ __forceinline__ double double_bits(float f) {  // for normal f > 0
+  const int b = __float_as_int(f);
+  return __hiloint2double((b >> 3) + (896 << 20), b << 29);
 }
 
 // A group of G lanes inside one warp.
@@ -509,6 +533,7 @@ __device__ __forceinline__ void sum_first(const Grp<G>& g, T (&v)[MAXM], int n) 
 struct CellScalars {
   double T, invT, lnT, S, invS, rho, invrho, cb, invcb, Sh;
   double TSh, irc;  // T Sh, 1 / (rho cb)
+  double Hs, Ds;    // sum (cp_k/R - h_k/RT) w_k / T, sum Y_k d(cp_k/R)/dT / W_k
   double pinv;  // 1 / p (constant pressure) or 1 / rho (constant volume): set by the caller
   int prec;     // precision level (3: mixed exp in the RHS, double-float J v core): set by the caller
   // auxiliary-temperature system: sum_k (cp_k/R - 1) F_k / W_k, the T row
@@ -520,13 +545,13 @@ struct CellScalars {
 
 struct SlotPtrs {
   double *u, *src, *fn, *arg, *fr, *F, *w, *Q, *K;
-  double *C, *dC, *cp, *hRT, *dcp, *gRT, *E, *Einv, *CE, *om, *q, *kc, *krc, *qT, *tb, *tro, *part;
+  double *C, *dC, *cp, *hRT, *gRT, *E, *CE, *om, *q, *kc, *krc, *qT, *tb, *tro, *part;
   df2 *C2, *dC2;
   uint16_t* dig;
   // precision 6: FP32 J v caches in the kc/krc/qT storage -- per reaction k, k/Kc, dq/dT;
-  // per species C, rho/W, W/rho, w, h/RT - esh, (cp - h)/T w / RT, Y dcp/dT / W, cp / W
-  float *xk, *xkr, *xqT, *xC, *xE, *xEinv, *xom, *xg, *xh, *xdcp, *xcp;
-  double *H, *LU, *piv, *red, *Bm;
+  // per species C, rho/W, W/rho, w, h/RT - esh, cp / W
+  float *xk, *xkr, *xqT, *xC, *xE, *xEinv, *xom, *xg, *xcp;
+  double *H, *LU, *piv, *Bm;
   float *fC, *fdC, *fh, *fcp, *fdcp, *fom, *fq, *fkc, *fkr, *ftb, *fQ, *fw, *fpart;  // mixed precision
   int Nq;  // stride between Krylov / stage vectors
 };
@@ -534,11 +559,11 @@ struct SlotPtrs {
 __device__ inline SlotPtrs slot_ptrs(double* b, const SlotLayout& s) {
   SlotPtrs p;
   p.u = b + s.u;
-  p.src = b + s.src;
+  p.src = b + (s.src >= 0 ? s.src : 0);  // not read where the slot has none
   p.fn = b + s.fn;
   p.arg = b + s.arg;
   p.fr = b + s.fr;
-  p.F = b + s.F;
+  p.F = b + (s.F >= 0 ? s.F : 0);  // not read where the slot has none
   p.w = b + s.w;
   p.Q = b + s.Q;
   p.K = b + s.K;
@@ -546,10 +571,8 @@ __device__ inline SlotPtrs slot_ptrs(double* b, const SlotLayout& s) {
   p.dC = b + s.dC;
   p.cp = b + s.cp;
   p.hRT = b + s.hRT;
-  p.dcp = b + s.dcp;
   p.gRT = b + s.gRT;
   p.E = b + s.E;
-  p.Einv = b + s.Einv;
   p.CE = b + s.CE;
   p.om = b + s.om;
   p.q = b + s.q;
@@ -573,16 +596,13 @@ __device__ inline SlotPtrs slot_ptrs(double* b, const SlotLayout& s) {
     p.xEinv = X + 2 * ns1;
     p.xom = X + 3 * ns1;
     p.xg = X + 4 * ns1;
-    p.xh = X + 5 * ns1;
-    p.xdcp = X + 6 * ns1;
-    p.xcp = X + 7 * ns1;
+    p.xcp = X + 5 * ns1;
   }
   p.tb = b + s.tb;
   p.H = b + s.H;
   p.LU = b + s.LU;
   p.piv = b + s.piv;
   p.Bm = b + s.Bm;
-  p.red = b + s.red;
   float* f = reinterpret_cast<float*>(b + s.fbase);
   p.fC = f + s.fC;
   p.fdC = f + s.fdC;
@@ -881,8 +901,6 @@ __device__ __forceinline__ void cache_reaction(const SlotPtrs& s, const CellScal
 // exponential and the product with kappa stay on the integer pipes (fx.cuh),
 // and two FP64 instructions are left, the difference of the two products; the
 // form with k, E and 1/E in FP64 took sixteen (28 with the caches, now 11).
-// scaled_rate has no branch, so U reactions' chains interleave: one alone is
-// ~500 cycles of latency for ~150 of issue.
 struct ScaledRate {
   uint64_t lg, ks;  // log2 kappa in fixed point; kappa = ks 2^(kn - 63)
   int kn;
@@ -905,7 +923,7 @@ __device__ __forceinline__ ScaledRate scaled_rate(const MechView& m, const SlotP
 }
 // What the caching right-hand side at u_n keeps of one reaction.
 template <bool MIXED>
-__device__ __forceinline__ void cache_scaled(const MechView& m, const SlotPtrs& s, double invT, CellScalars* cs, int j,
+__device__ __forceinline__ void cache_scaled(const MechView& m, const SlotPtrs& s, double T, double invT, CellScalars* cs, int j,
                                              uint32_t sl, int kind, bool rev, int slot, double Mc, double mult,
                                              const ScaledRate& r) {
   const int ra = sl & 255, rb = (sl >> 8) & 255, pa = (sl >> 16) & 255, pb = sl >> 24;
@@ -913,19 +931,19 @@ __device__ __forceinline__ void cache_scaled(const MechView& m, const SlotPtrs& 
   const int nt = m.ntroe;
   const double kap0 = fx::pack(r.ks, r.kn);
   const double kap = kind == 2 ? kap0 * mult : kap0;
-  double dlnk = __dmul_rn(fma(m.EaR[j], invT, m.bexp[j]), invT);  // d ln k / dT
-  if (kind == 2) dlnk = s.tro[7 * nt + slot];
-  // d q_j / dT at fixed concentrations (without the third-body factor):
-  // d ln k/dT q + d ln Kc/dT k prod C^nu''/Kc, with d ln Kc/dT =
-  // (sum_products h/RT - sum_reactants h/RT - dnu) / T summed from the
-  // per-species (h/RT - 1)/T
+  double dlnk = fma(m.EaR[j], invT, m.bexp[j]);  // T d ln k / dT
+  if (kind == 2) dlnk = s.tro[7 * nt + slot] * T;
+  // T d q_j / dT at fixed concentrations (without the third-body factor; the J v
+  // multiplies it by vT / T): T d ln k/dT q + T d ln Kc/dT k prod C^nu''/Kc, with
+  // T d ln Kc/dT = sum_products h/RT - sum_reactants h/RT - dnu summed from the
+  // per-species h/RT - 1
   const double t0 = __dmul_rn(dlnk, r.D);
   const double dlnKc = __dsub_rn(__dadd_rn(s.dC[pa], s.dC[pb]), __dadd_rn(s.dC[ra], s.dC[rb]));
   const double t1 = fma(dlnKc, __dmul_rn(r.zr, r.zs), t0);
   const double qT = __dmul_rn(kap, rev ? t1 : t0);
   if (!MIXED && cs->prec != 3 && cs->prec != 6) {
     // the scaled Jacobian-vector product: kappa, d q/dT and the slot's d kappa/d[M]
-    if (kind != 0) cache_pressure<MIXED>(s, slot, Mc, kind == 2 ? kap0 * s.tro[8 * nt + slot] : 0.0, dlnk, 0.0);
+    if (kind != 0) cache_pressure<MIXED>(s, slot, Mc, kind == 2 ? kap0 * s.tro[8 * nt + slot] : 0.0, 0.0, 0.0);
     s.kc[j] = kap;
     s.qT[j] = qT;
   } else {
@@ -933,46 +951,36 @@ __device__ __forceinline__ void cache_scaled(const MechView& m, const SlotPtrs& 
     const double k = __dmul_rn(kap, Er);
     const double kr = rev ? __dmul_rn(kap, __dmul_rn(s.E[pa], s.E[pb])) : 0.0;
     if (kind != 0)
-      cache_pressure<MIXED>(s, slot, Mc, kind == 2 ? kap0 * Er * s.tro[8 * nt + slot] : 0.0, dlnk,
+      cache_pressure<MIXED>(s, slot, Mc, kind == 2 ? kap0 * Er * s.tro[8 * nt + slot] : 0.0, dlnk * invT,
                             rev ? fx::exp2_double(A[pa] + A[pb] - A[ra] - A[rb], m.etab) : 0.0);
     cache_reaction<MIXED>(s, cs, j, k, kr, qT);
   }
 }
-// Reactions j0 + lane + u G, u < U (indices past the last are computed as the last
-// and not stored).  PRESSURE: the first ones, some of them third-body or falloff.
-template <int G, bool MIXED, bool PRESSURE, int U>
-__device__ __forceinline__ void reactions_scaled(const MechView& m, const SlotPtrs& s, const fx::Temp& ft, double invT,
-                                                 bool coop_tb, bool cache, CellScalars* cs, int j0, int lane, int* qe) {
-  ScaledRate r[U];
-  uint32_t sl[U];
-  int meta[U];
-  double q[U];
-  double Mc = 0.0, mult = 1.0;
-#pragma unroll
-  for (int u = 0; u < U; ++u) {
-    const int j = min(j0 + lane + u * G, m.nr - 1);
-    sl[u] = m.slots[j];
-    meta[u] = m.meta[j];
-    r[u] = scaled_rate(m, s, ft, j, sl[u], (meta[u] >> 2) & 1);
-    double Dm = r[u].D;  // with the third-body or falloff multiplier
-    if (PRESSURE && (meta[u] & 3) != 0) {
-      Mc = third_body_conc<G>(m, s, meta[u] >> 8, coop_tb);
-      mult = (meta[u] & 3) == 1 ? Mc : s.tro[6 * m.ntroe + (meta[u] >> 8)];
-      Dm = __dmul_rn(Dm, mult);
-    }
-    q[u] = fx::mul_sig(r[u].ks, r[u].kn, Dm);
-    *qe = max(*qe, (__double2hiint(q[u]) >> 20) & 0x7ff);
+// Reaction j0 + lane (a lane past the last computes the last and stores nothing).
+// PRESSURE: the first ones, some of them third-body or falloff.  One reaction at a
+// time: two interleaved gained nothing (the warps' chains hide each other) and their
+// code cost 4 % through the instruction cache.
+template <int G, bool MIXED, bool PRESSURE>
+__device__ __forceinline__ void reactions_scaled(const MechView& m, const SlotPtrs& s, const fx::Temp& ft, double T,
+                                                 double invT, bool coop_tb, bool cache, CellScalars* cs, int j0,
+                                                 int lane, int* qe) {
+  const int j = min(j0 + lane, m.nr - 1);
+  const uint32_t sl = m.slots[j];
+  const int meta = m.meta[j], kind = PRESSURE ? meta & 3 : 0;
+  const bool rev = (meta >> 2) & 1;
+  const ScaledRate r = scaled_rate(m, s, ft, j, sl, rev);
+  double Mc = 0.0, mult = 1.0, Dm = r.D;  // Dm: with the third-body or falloff multiplier
+  if (kind != 0) {
+    Mc = third_body_conc<G>(m, s, meta >> 8, coop_tb);
+    mult = kind == 1 ? Mc : s.tro[6 * m.ntroe + (meta >> 8)];
+    Dm = __dmul_rn(Dm, mult);
   }
-#pragma unroll
-  for (int u = 0; u < U; ++u) {
-    const int j = j0 + lane + u * G;
-    if (j < m.nr) {
-      if (MIXED) reinterpret_cast<df2*>(s.q)[j] = df_from(q[u]);  // double-float copy for the gather
-      else s.q[j] = q[u];
-      if (cache)
-        cache_scaled<MIXED>(m, s, invT, cs, j, sl[u], PRESSURE ? meta[u] & 3 : 0, (meta[u] >> 2) & 1, meta[u] >> 8, Mc,
-                            mult, r[u]);
-    }
+  const double q = fx::mul_sig(r.ks, r.kn, Dm);
+  *qe = max(*qe, (__double2hiint(q) >> 20) & 0x7ff);
+  if (j0 + lane < m.nr) {
+    if (MIXED) reinterpret_cast<df2*>(s.q)[j] = df_from(q);  // double-float copy for the gather
+    else s.q[j] = q;
+    if (cache) cache_scaled<MIXED>(m, s, T, invT, cs, j, sl, kind, rev, meta >> 8, Mc, mult, r);
   }
 }
 
@@ -980,7 +988,7 @@ __device__ __forceinline__ void reactions_scaled(const MechView& m, const SlotPt
 // the scaled one does not hold for (a Gibbs factor past e^170, T outside
 // [250, 16000) K, coefficients outside the fixed-point range, NaN).
 template <int G, bool MIXED>
-__device__ __noinline__ void reactions_direct(const MechView& m, const SlotPtrs& s, double invT, double lnT,
+__device__ __noinline__ void reactions_direct(const MechView& m, const SlotPtrs& s, double T, double invT, double lnT,
                                               double lnRTp, bool coop_tb, bool cache, CellScalars* cs) {
   const Grp<G> g;
   const int ns = m.ns;
@@ -1033,7 +1041,7 @@ __device__ __noinline__ void reactions_direct(const MechView& m, const SlotPtrs&
       // with d ln Kc/dT = (sum_products h/RT - sum_reactants h/RT - dnu) / T
       // summed from the per-species (h/RT - 1)/T
       const double dlnKc = __dsub_rn(__dadd_rn(s.dC[pa], s.dC[pb]), __dadd_rn(s.dC[ra], s.dC[rb]));
-      const double qT = fma(dlnk, q0, __dmul_rn(dlnKc, __dmul_rn(k, Rb)));
+      const double qT = fma(dlnk * T, q0, __dmul_rn(dlnKc, __dmul_rn(k, Rb)));  // T d q/dT
       cache_reaction<MIXED>(s, cs, j, k, kr, qT);
     }
   }
@@ -1043,7 +1051,7 @@ __device__ __noinline__ void reactions_direct(const MechView& m, const SlotPtrs&
 // out = f(uu) + src (src may be null).  p > 0: constant-pressure reactor at
 // pressure p; p < 0: constant-volume reactor of density -p (Eq. cv_reactor with
 // internal energies u_k/RT = h_k/RT - 1 and c_v/R = c_p/R - 1 per species).  uu, out: N-vectors in shared memory
-// (out must not alias uu).  When `cache` is set, the values the analytic
+// (out may be uu itself, except in the auxiliary-temperature system).  When `cache` is set, the values the analytic
 // Jacobian-vector product reuses are kept (rate coefficients, w, d(cp/R)/dT
 // and the cell scalars).  Inlined into the 32-lane FP64 integrator and called
 // through rhs_eval_call elsewhere; each product that meets a sum is written as
@@ -1070,16 +1078,33 @@ __device__ __forceinline__ void rhs_eval(const MechView& m, const SlotPtrs& s, c
   }
   const double lnRTp = LN_R_OVER_PREF + lnT;  // ln(R T / p_ref)
   // species pass 1: thermo, Gibbs factors, sum Y/W
+  // T times the factors 2/3, 3/4, 4/5, 3/2, 4/3 of the nested polynomials, one a lane
+  // (G >= 8 lanes) and one FP64 multiplication for all
+  double th, t21, t23, t34, t45, t32, t43;
+  {
+    const int l = g.lane & 7;
+    const double f = l == 0 ? 2.0 / 3.0 : l == 1 ? 0.75 : l == 2 ? 0.8 : l == 3 ? 1.5 : l == 4 ? 4.0 / 3.0 : 0.5;
+    const double t = __dmul_rn(T, f);
+    t23 = __shfl_sync(g.mask, t, 0, G);
+    t34 = __shfl_sync(g.mask, t, 1, G);
+    t45 = __shfl_sync(g.mask, t, 2, G);
+    t32 = __shfl_sync(g.mask, t, 3, G);
+    t43 = __shfl_sync(g.mask, t, 4, G);
+    th = __shfl_sync(g.mask, t, 5, G);
+    t21 = cache ? 2.0 * T : 0.0;
+  }
   double S = 0.0;
+  double Ds = 0.0;  // sum Y_k (dcp_k/R/dT) / W_k (caching only)
   int ghi = 0;  // max over species of the high word of |g/RT + ln(RT/p_ref)| (integer compare)
   for (int k = g.lane; k < ns; k += G) {
     const double* c = below(T, m.Tmid[k]) ? m.lo : m.hi;
     const double a1 = c[k], a2 = c[ns + k], a3 = c[2 * ns + k], a4 = c[3 * ns + k], a5 = c[4 * ns + k];
+    // nested with the polynomials' factors in multiples of T: seven coefficients a range
     const double cp = fma(fma(fma(fma(a5, T, a4), T, a3), T, a2), T, a1);
-    const double hp = fma(fma(fma(c[8 * ns + k], T, c[7 * ns + k]), T, c[6 * ns + k]), T, c[5 * ns + k]);
-    const double hrt = fma(c[9 * ns + k], invT, fma(hp, T, a1));
-    const double sp = fma(fma(fma(c[12 * ns + k], T, c[11 * ns + k]), T, c[10 * ns + k]), T, a2);
-    const double sr = fma(a1, lnT, fma(sp, T, c[13 * ns + k]));
+    const double hp = fma(fma(fma(fma(a5, t45, a4), t34, a3), t23, a2), th, a1);
+    const double hrt = fma(c[5 * ns + k], invT, hp);
+    const double sp = fma(fma(fma(a5, t34, a4), t23, a3), th, a2);
+    const double sr = fma(a1, lnT, fma(sp, T, c[6 * ns + k]));
     const double grt = hrt - sr;
     s.cp[k] = cp;
     s.hRT[k] = hrt;
@@ -1087,11 +1112,11 @@ __device__ __forceinline__ void rhs_eval(const MechView& m, const SlotPtrs& s, c
     s.gRT[k] = a;
     ghi = max(ghi, __double2hiint(a) & 0x7fffffff);
     if (cache) {
-      const double dcp = fma(fma(fma(c[16 * ns + k], T, c[15 * ns + k]), T, c[14 * ns + k]), T, a2);
-      s.dcp[k] = dcp;
-      // (h/RT - 1)/T, whose sum over a reaction's products less its reactants is
-      // d ln Kc/dT; kept in dC, which the J v overwrites later (sentinel entry 0)
-      s.dC[k] = __dmul_rn(hrt - 1.0, invT);
+      const double dcp = fma(fma(fma(a5, t43, a4), t32, a3), t21, a2);
+      Ds = fma(__dmul_rn(uu[k], dcp), m.invW[k], Ds);
+      // h/RT - 1, whose sum over a reaction's products less its reactants is
+      // T d ln Kc/dT; kept in dC, which the J v overwrites later (sentinel entry 0)
+      s.dC[k] = hrt - 1.0;
       if (MIXED) {
         s.fh[k] = __double2float_rn(hrt);
         s.fcp[k] = __double2float_rn(cp);
@@ -1246,17 +1271,17 @@ __device__ __forceinline__ void rhs_eval(const MechView& m, const SlotPtrs& s, c
   if (zf) {
     const fx::Temp ft = fx::temperature(lgT, fx::recip_fixed70(T, invT));
     int j0 = 0;
-    for (; j0 < m.ntb; j0 += G) reactions_scaled<G, MIXED, true, 1>(m, s, ft, invT, coop_tb, cache, cs, j0, g.lane, &qe);
-    constexpr int U = RK_UNROLL;
-    for (; j0 < m.nr; j0 += U * G)
-      reactions_scaled<G, MIXED, false, U>(m, s, ft, invT, coop_tb, cache, cs, j0, g.lane, &qe);
+    for (; j0 < m.ntb; j0 += G) reactions_scaled<G, MIXED, true>(m, s, ft, T, invT, coop_tb, cache, cs, j0, g.lane, &qe);
+    for (; j0 < m.nr; j0 += G)
+      reactions_scaled<G, MIXED, false>(m, s, ft, T, invT, coop_tb, cache, cs, j0, g.lane, &qe);
   } else {
-    reactions_direct<G, MIXED>(m, s, invT, lnT, lnRTp, coop_tb, cache, cs);
+    reactions_direct<G, MIXED>(m, s, T, invT, lnT, lnRTp, coop_tb, cache, cs);
   }
   g.sync();
   // species pass 2: w = nu^T q, dY/dt and the sums of the temperature equation
   double Sh = 0.0, cb = 0.0;
   const bool zjv = zf && !MIXED && cs->prec != 3 && cs->prec != 6;
+  double Hs = 0.0;
   double Ax = 0.0, Bx = 0.0;  // auxiliary T: sum (u_k/RT) F_k / W_k and sum (cv_k/R) F_k / W_k
   bool tc_om = false;  // w already in part[0..ns) from the tensor cores
   if constexpr (TC) tc_om = gather_tc<G>(m, s, s.q, s.part);
@@ -1281,14 +1306,15 @@ __device__ __forceinline__ void rhs_eval(const MechView& m, const SlotPtrs& s, c
     if (cache) s.om[k] = om;
     const double r = __dmul_rn(__dmul_rn(m.W[k], om), invrho);
     const double Fk = src ? __dadd_rn(r, src[k]) : r;
-    out[k] = Fk;
     double hk = s.hRT[k], ck = s.cp[k];
+    const double ufac = uu[k];
+    out[k] = Fk;  // (out may be uu)
     if (cv) {  // internal energies and cv (uniform; the subtractions cost 64 cycles each)
       hk -= 1.0;
       ck -= 1.0;
     }
     Sh = fma(hk, om, Sh);
-    cb = fma(uu[k] * ck, m.invW[k], cb);
+    cb = fma(ufac * ck, m.invW[k], cb);
     if (aux) {
       Ax = fma((s.hRT[k] - 1.0) * Fk, m.invW[k], Ax);
       Bx = fma((s.cp[k] - 1.0) * Fk, m.invW[k], Bx);
@@ -1296,23 +1322,20 @@ __device__ __forceinline__ void rhs_eval(const MechView& m, const SlotPtrs& s, c
     if (cache) {
       // per-species factors of the analytic J v, written over arrays the
       // remaining RHS no longer reads (lane-private entries k):
-      //   E: rho/W_k (times E_k for the scaled J v)   Einv: W_k/rho   gRT: h_k/RT - esh
-      //   hRT: (cp_k/R - h_k/RT) w_k / T   dcp: Y_k (dcp_k/dT) / W_k   cp: (cp_k/R - esh) / W_k
+      //   E: rho/W_k (times E_k for the scaled J v)   hRT: h_k/RT (u_k/RT at fixed volume)
+      //   cp: (cp_k/R, or cv_k/R) / W_k
+      // and the sum of (cp_k/R - h_k/RT) w_k / T
+      Hs = fma((s.cp[k] - s.hRT[k]) * invT, om, Hs);
       const double rW = rho * m.invW[k];
       s.E[k] = zjv ? s.E[k] * rW : rW;
-      s.Einv[k] = m.W[k] * invrho;
-      s.gRT[k] = hk;
-      s.hRT[k] = (s.cp[k] - s.hRT[k]) * invT * om;
-      s.dcp[k] = uu[k] * s.dcp[k] * m.invW[k];
+      if (cv) s.hRT[k] = hk;
       s.cp[k] = ck * m.invW[k];
       if (cs->prec == 6) {  // FP32 copies for the FP32 J v
         s.xC[k] = __double2float_rn(s.C[k]);
         s.xE[k] = __double2float_rn(rW);
-        s.xEinv[k] = __double2float_rn(s.Einv[k]);
+        s.xEinv[k] = __double2float_rn(m.W[k] * invrho);
         s.xom[k] = __double2float_rn(om);
-        s.xg[k] = __double2float_rn(s.gRT[k]);
-        s.xh[k] = __double2float_rn(s.hRT[k]);
-        s.xdcp[k] = __double2float_rn(s.dcp[k]);
+        s.xg[k] = __double2float_rn(hk);
         s.xcp[k] = __double2float_rn(s.cp[k]);
       }
     }
@@ -1324,6 +1347,19 @@ __device__ __forceinline__ void rhs_eval(const MechView& m, const SlotPtrs& s, c
     cb = t4[1];
     Ax = t4[2];
     Bx = t4[3];
+    if (cache) {
+      double t2[2] = {Hs, Ds};
+      sum_many<G, 2>(g, t2);
+      Hs = t2[0];
+      Ds = t2[1];
+    }
+  } else if (cache) {
+    double t4[4] = {Sh, cb, Hs, Ds};
+    sum_many<G, 4>(g, t4);
+    Sh = t4[0];
+    cb = t4[1];
+    Hs = t4[2];
+    Ds = t4[3];
   } else {
     double t2[2] = {Sh, cb};
     sum_many<G, 2>(g, t2);
@@ -1372,6 +1408,8 @@ __device__ __forceinline__ void rhs_eval(const MechView& m, const SlotPtrs& s, c
     cs->invcb = invcb;
     cs->Sh = Sh;
     cs->TSh = T * Sh;
+    cs->Hs = Hs;
+    cs->Ds = Ds;
     cs->irc = invrho * invcb;
     cs->cv = cv;
     cs->zf = zjv;
@@ -1415,42 +1453,36 @@ __device__ __forceinline__ double third_body_rate(const MechView& m, const doubl
   return dM;
 }
 
-// dq_j = d q_j/dT vT + kappa_j d(z_ra z_rb - z_pa z_pb) of reactions j0 + lane + u G
-// (as reactions_scaled): six FP64 instructions a reaction.
-template <int G, bool PRESSURE, int U>
-__device__ __forceinline__ void jvp_scaled(const MechView& m, const SlotPtrs& s, double vT, bool coop_tb,
+// dq_j = T d q_j/dT vTT + kappa_j d(z_ra z_rb - z_pa z_pb), vTT = vT / T, of reaction
+// j0 + lane (as reactions_scaled): six FP64 instructions.
+template <int G, bool PRESSURE>
+__device__ __forceinline__ void jvp_scaled(const MechView& m, const SlotPtrs& s, double vTT, bool coop_tb,
                                            const double (&mp)[MAXM], int j0, int lane, int* qe) {
-  double dq[U];
-#pragma unroll
-  for (int u = 0; u < U; ++u) {
-    const int j = min(j0 + lane + u * G, m.nr - 1);
-    const uint32_t sl = m.slots[j];
-    const int ra = sl & 255, rb = (sl >> 8) & 255, pa = (sl >> 16) & 255, pb = sl >> 24;
-    const int meta = m.meta[j];
-    const bool rev = (meta >> 2) & 1;
-    const double za = s.CE[ra], zb = s.CE[rb], zp = s.CE[pa], zq = s.CE[pb];
-    const double dD0 = fma(s.dC[ra], zb, za * s.dC[rb]);
-    const double dD1 = fma(-s.dC[pa], zq, fma(-zp, s.dC[pb], dD0));
-    const double kap = s.kc[j];
-    dq[u] = fma(s.qT[j], vT, kap * (rev ? dD1 : dD0));
-    if (PRESSURE && (meta & 3) != 0) {
-      const int slot = meta >> 8;
-      const double* t = s.tb + 4 * slot;
-      double D = za * zb;
-      if (rev) D = fma(-zp, zq, D);
-      const double dM = third_body_rate<G>(m, s.arg, slot, coop_tb, mp);
-      dq[u] = (meta & 3) == 1 ? t[0] * dq[u] + dM * (kap * D) : dq[u] + t[1] * dM * D;
-    }
-    *qe = max(*qe, (__double2hiint(dq[u]) >> 20) & 0x7ff);
+  const int j = min(j0 + lane, m.nr - 1);
+  const uint32_t sl = m.slots[j];
+  const int ra = sl & 255, rb = (sl >> 8) & 255, pa = (sl >> 16) & 255, pb = sl >> 24;
+  const int meta = m.meta[j];
+  const bool rev = (meta >> 2) & 1;
+  const double za = s.CE[ra], zb = s.CE[rb], zp = s.CE[pa], zq = s.CE[pb];
+  const double dD0 = fma(s.dC[ra], zb, za * s.dC[rb]);
+  const double dD1 = fma(-s.dC[pa], zq, fma(-zp, s.dC[pb], dD0));
+  const double kap = s.kc[j];
+  double dq = fma(s.qT[j], vTT, kap * (rev ? dD1 : dD0));
+  if (PRESSURE && (meta & 3) != 0) {
+    const int slot = meta >> 8;
+    const double* t = s.tb + 4 * slot;
+    double D = za * zb;
+    if (rev) D = fma(-zp, zq, D);
+    const double dM = third_body_rate<G>(m, s.arg, slot, coop_tb, mp);
+    dq = (meta & 3) == 1 ? t[0] * dq + dM * (kap * D) : dq + t[1] * dM * D;
   }
-#pragma unroll
-  for (int u = 0; u < U; ++u)
-    if (j0 + lane + u * G < m.nr) s.q[j0 + lane + u * G] = dq[u];
+  *qe = max(*qe, (__double2hiint(dq) >> 20) & 0x7ff);
+  if (j0 + lane < m.nr) s.q[j] = dq;
 }
 
 // The reaction rates' derivatives from k and k/Kc (caches not in the scaled form).
 template <int G, bool DFG>
-__device__ __forceinline__ void jvp_reactions(const MechView& m, const SlotPtrs& s, double vT, bool coop_tb,
+__device__ __forceinline__ void jvp_reactions(const MechView& m, const SlotPtrs& s, double vTT, bool coop_tb,
                                               const double (&mp)[MAXM]) {
   const Grp<G> g;
   for (int j = g.lane; j < m.nr; j += G) {
@@ -1461,7 +1493,7 @@ __device__ __forceinline__ void jvp_reactions(const MechView& m, const SlotPtrs&
     const double dPf = fma(s.dC[ra], s.C[rb], s.C[ra] * s.dC[rb]);
     const double dPb = fma(s.dC[pa], s.C[pb], s.C[pa] * s.dC[pb]);
     const double k = s.kc[j], kr = s.krc[j];
-    double dq = fma(s.qT[j], vT, fma(k, dPf, -kr * dPb));
+    double dq = fma(s.qT[j], vTT, fma(k, dPf, -kr * dPb));
     if (kind != 0) {
       const int slot = meta >> 8;
       const double* t = s.tb + 4 * slot;
@@ -1476,9 +1508,9 @@ __device__ __forceinline__ void jvp_reactions(const MechView& m, const SlotPtrs&
   }
 }
 template <int G>
-__device__ __noinline__ void jvp_reactions_call(const MechView& m, const SlotPtrs& s, double vT, bool coop_tb,
+__device__ __noinline__ void jvp_reactions_call(const MechView& m, const SlotPtrs& s, double vTT, bool coop_tb,
                                                 const double (&mp)[MAXM]) {
-  jvp_reactions<G, false>(m, s, vT, coop_tb, mp);
+  jvp_reactions<G, false>(m, s, vTT, coop_tb, mp);
 }
 
 // Analytic Jacobian-vector product out = J(u_n) v, using the values cached by
@@ -1495,7 +1527,8 @@ __device__ __forceinline__ void jvp_eval(const MechView& m, const SlotPtrs& s, c
   double a = 0.0;
   for (int k = g.lane; k < ns; k += G) a = fma(v[k], m.invW[k], a);
   a = g.sum(a);
-  const double drr = cs.cv ? 0.0 : -fma(a, cs.invS, vT * invT);  // d rho / rho (0 at fixed volume)
+  const double vTT = vT * invT;
+  const double drr = cs.cv ? 0.0 : -fma(a, cs.invS, vTT);  // d rho / rho (0 at fixed volume)
   const bool coop_tb = m.ntb > 0 && m.ntb <= MAXM;
   const bool zf = !DFG && cs.zf;
   int qe = 0;  // largest exponent of the lane's dq
@@ -1521,13 +1554,12 @@ __device__ __forceinline__ void jvp_eval(const MechView& m, const SlotPtrs& s, c
   g.sync();
   if (zf) {
     int j0 = 0;
-    for (; j0 < m.ntb; j0 += G) jvp_scaled<G, true, 1>(m, s, vT, coop_tb, mp, j0, g.lane, &qe);
-    constexpr int U = RK_UNROLL;
-    for (; j0 < m.nr; j0 += U * G) jvp_scaled<G, false, U>(m, s, vT, coop_tb, mp, j0, g.lane, &qe);
+    for (; j0 < m.ntb; j0 += G) jvp_scaled<G, true>(m, s, vTT, coop_tb, mp, j0, g.lane, &qe);
+    for (; j0 < m.nr; j0 += G) jvp_scaled<G, false>(m, s, vTT, coop_tb, mp, j0, g.lane, &qe);
   } else if constexpr (DFG) {
-    jvp_reactions<G, true>(m, s, vT, coop_tb, mp);
+    jvp_reactions<G, true>(m, s, vTT, coop_tb, mp);
   } else {
-    jvp_reactions_call<G>(m, s, vT, coop_tb, mp);
+    jvp_reactions_call<G>(m, s, vTT, coop_tb, mp);
   }
   g.sync();
   bool tc_om = false;  // d w already in part[0..ns) from the tensor cores
@@ -1544,19 +1576,19 @@ __device__ __forceinline__ void jvp_eval(const MechView& m, const SlotPtrs& s, c
   for (int k = g.lane; k < ns; k += G) {
     const double dom = DFG ? piece_sum_df(m, reinterpret_cast<const df2*>(s.part), k)
                            : gathered_row(m, s, k, em);
-    out[k] = s.Einv[k] * fma(-s.om[k], drr, dom);  // Einv: W_k / rho
-    dSh = fma(s.gRT[k], dom, fma(s.hRT[k], vT, dSh));
-    dcb = fma(s.dcp[k], vT, fma(s.cp[k], v[k], dcb));
+    out[k] = m.W[k] * cs.invrho * fma(-s.om[k], drr, dom);
+    dSh = fma(s.hRT[k], dom, dSh);
+    dcb = fma(s.cp[k], v[k], dcb);
   }
   if (m.nx > 0) {
     // auxiliary temperature: d w_T = (-vT B - T sum_k (u_k/RT) dF_k/W_k + dX/R - w_T dcb) / cb,
     // dF_k = W_k dw_k, X = |v|^2/2 S_rho - v . S_m + S_E, dv = (d(rho v) - v d rho) / rho
     double D1 = 0.0;
-    for (int k = g.lane; k < ns; k += G) D1 = fma(s.gRT[k], out[k] * m.invW[k], D1);  // gRT: h/RT - 1
+    for (int k = g.lane; k < ns; k += G) D1 = fma(s.hRT[k], out[k] * m.invW[k], D1);  // hRT: h/RT - 1
     double t2[2] = {D1, dcb};
     sum_many<G, 2>(g, t2);
     D1 = t2[0];
-    dcb = t2[1];
+    dcb = fma(cs.Ds, vT, t2[1]);
     if (g.lane == 0) {
       const double irc = cs.irho_c;
       const double dv0 = (v[ns + 2] - cs.vel[0] * v[ns + 1]) * irc;
@@ -1574,8 +1606,8 @@ __device__ __forceinline__ void jvp_eval(const MechView& m, const SlotPtrs& s, c
   {
     double t2[2] = {dSh, dcb};
     sum_many<G, 2>(g, t2);
-    dSh = t2[0];
-    dcb = t2[1];
+    dSh = fma(cs.Hs, vT, t2[0]);
+    dcb = fma(cs.Ds, vT, t2[1]);
   }
   if (g.lane == 0) {
     out[ns] = fma(cs.TSh, fma(dcb, cs.invcb, drr), -fma(vT, cs.Sh, T * dSh)) * cs.irc;
@@ -1616,7 +1648,7 @@ __device__ __forceinline__ void jvp_eval_df(const MechView& m, const SlotPtrs& s
   }
   if (coop_tb) sum_first<G>(g, mp, m.ntb);
   g.sync();
-  const df2 vT2 = df_from(vT);
+  const df2 vT2 = df_from(vT * invT);  // qT holds T d q/dT
   const df2* k2 = reinterpret_cast<const df2*>(s.kc);
   const df2* kr2 = reinterpret_cast<const df2*>(s.krc);
   const df2* qT2 = reinterpret_cast<const df2*>(s.qT);
@@ -1657,15 +1689,15 @@ __device__ __forceinline__ void jvp_eval_df(const MechView& m, const SlotPtrs& s
   double dSh = 0.0, dcb = 0.0;
   for (int k = g.lane; k < ns; k += G) {
     const double dom = piece_sum_df(m, reinterpret_cast<const df2*>(s.part), k);
-    out[k] = s.Einv[k] * fma(-s.om[k], drr, dom);  // Einv: W_k / rho
-    dSh = fma(s.gRT[k], dom, fma(s.hRT[k], vT, dSh));
-    dcb = fma(s.dcp[k], vT, fma(s.cp[k], v[k], dcb));
+    out[k] = m.W[k] * cs.invrho * fma(-s.om[k], drr, dom);
+    dSh = fma(s.hRT[k], dom, dSh);
+    dcb = fma(s.cp[k], v[k], dcb);
   }
   {
     double t2[2] = {dSh, dcb};
     sum_many<G, 2>(g, t2);
-    dSh = t2[0];
-    dcb = t2[1];
+    dSh = fma(cs.Hs, vT, t2[0]);
+    dcb = fma(cs.Ds, vT, t2[1]);
   }
   if (g.lane == 0) {
     out[ns] = (-(vT * cs.Sh + T * dSh) + T * cs.Sh * (drr + dcb * cs.invcb)) * (cs.invrho * cs.invcb);
@@ -1818,7 +1850,7 @@ __device__ __forceinline__ void jvp_eval_f32x(const MechView& m, const SlotPtrs&
     const float dPf = fmaf(fdC[ra], Crb, Cra * fdC[rb]);
     const float dPb = fmaf(fdC[pa], Cpb, Cpa * fdC[pb]);
     const float k = s.xk[j], kr = s.xkr[j];
-    float dq = fmaf(s.xqT[j], vT, fmaf(k, dPf, -kr * dPb));
+    float dq = fmaf(s.xqT[j], vT * invT, fmaf(k, dPf, -kr * dPb));  // xqT: T d q/dT
     if (kind != 0) {
       const int slot = meta >> 8;
       const double* t = s.tb + 4 * slot;
@@ -1851,14 +1883,14 @@ __device__ __forceinline__ void jvp_eval_f32x(const MechView& m, const SlotPtrs&
     for (; p < m.gspec[2 * k + 1]; ++p) dom += fpart[p];
     for (; p < m.gspec[2 * k + 2]; ++p) dom -= fpart[p];
     out[k] = (double)(s.xEinv[k] * fmaf(-s.xom[k], drr, dom));  // xEinv: W_k / rho
-    dSh = fmaf(s.xg[k], dom, fmaf(s.xh[k], vT, dSh));
-    dcb = fmaf(s.xdcp[k], vT, fmaf(s.xcp[k], f(v[k]), dcb));
+    dSh = fmaf(s.xg[k], dom, dSh);
+    dcb = fmaf(s.xcp[k], f(v[k]), dcb);
   }
   {
     float t2[2] = {dSh, dcb};
     sum_many<G, 2>(g, t2);
-    dSh = t2[0];
-    dcb = t2[1];
+    dSh = fmaf(f(cs.Hs), vT, t2[0]);
+    dcb = fmaf(f(cs.Ds), vT, t2[1]);
   }
   if (g.lane == 0) {
     const float Sh = f(cs.Sh);
@@ -1923,15 +1955,14 @@ __device__ inline float group_dot_f(const Grp<G>& g, const double* a, const doub
 // enough").
 //
 // One FP64 Gram-Schmidt pass of w against the basis vectors q_0..q_{n-1}:
-// h = Q^T w (one batched reduction), w <- w - Q h, and hcol += h.  J > 0: n = J
+// h = Q^T w (one batched reduction), w <- w - Q h; lane i returns h_i (i < n).  J > 0: n = J
 // is known at compile time, so no term carries a predicate (a predicated-off
 // FP64 instruction still takes its issue and pipe slot); J = 0: n = jn at run
 // time guards each of the MAXM terms.  Either way the same operations in the
 // same order for the terms that exist.
 // WW: w^T w before the pass joins the reduction, into *ww.
 template <int G, int J, bool WW = false>
-__device__ __forceinline__ void cgs_pass(const SlotPtrs& s, int N, int jn, double (&hcol)[MAXM],
-                                         double* ww = nullptr) {
+__device__ __forceinline__ double cgs_pass(const SlotPtrs& s, int N, int jn, double* ww = nullptr) {
   const Grp<G> g;
   const int Nq = s.Nq;
   constexpr int LJ = J > 0 ? J : MAXM;
@@ -1956,9 +1987,10 @@ __device__ __forceinline__ void cgs_pass(const SlotPtrs& s, int N, int jn, doubl
       if (J > 0 || i < jn) we = fma(-hp[i], s.Q[i * Nq + e], we);
     s.w[e] = we;
   }
+  double mine = hp[0];
 #pragma unroll
-  for (int i = 0; i < LJ; ++i)
-    if (J > 0 || i < jn) hcol[i] += hp[i];
+  for (int i = 1; i < LJ; ++i) mine = g.lane == i ? hp[i] : mine;
+  return mine;
 }
 
 template <int G, bool MIXED = false, bool TC = false>
@@ -1992,10 +2024,9 @@ __device__ int arnoldi(const MechView& m, const SlotPtrs& s, const CellScalars& 
     double w02 = 0.0;
     if (MIXED) w02 = (double)group_dot_f<G>(g, s.w, s.w, N);
     else if (M > 4) w02 = group_dot<G>(g, s.w, s.w, N);
-    double hcol[MAXM];
-#pragma unroll
-    for (int i = 0; i < MAXM; ++i) hcol[i] = 0.0;
+    double hcol = 0.0;  // lane i: h_ij
     for (int pass = 0; pass < 2; ++pass) {
+      double hpass;
       if (MIXED && pass == 0) {
         double hp[MAXM];
         float part[MAXM];
@@ -2017,26 +2048,24 @@ __device__ int arnoldi(const MechView& m, const SlotPtrs& s, const CellScalars& 
             if (i <= j) we = fma(-hp[i], s.Q[i * Nq + e], we);
           s.w[e] = we;
         }
+        hpass = hp[0];
 #pragma unroll
-        for (int i = 0; i < MAXM; ++i) hcol[i] += hp[i];
+        for (int i = 1; i < MAXM; ++i) hpass = g.lane == i ? hp[i] : hpass;
       } else if (M <= 4) {
         const bool first = !MIXED && pass == 0;
         // the common Krylov dimensions: column j + 1 known at compile time
         switch (j) {
-          case 0: first ? cgs_pass<G, 1, true>(s, N, 1, hcol, &w02) : cgs_pass<G, 1>(s, N, 1, hcol); break;
-          case 1: first ? cgs_pass<G, 2, true>(s, N, 2, hcol, &w02) : cgs_pass<G, 2>(s, N, 2, hcol); break;
-          case 2: first ? cgs_pass<G, 3, true>(s, N, 3, hcol, &w02) : cgs_pass<G, 3>(s, N, 3, hcol); break;
-          default: cgs_pass<G, 4>(s, N, 4, hcol); break;  // (the last column has no breakdown test to feed)
+          case 0: hpass = first ? cgs_pass<G, 1, true>(s, N, 1, &w02) : cgs_pass<G, 1>(s, N, 1); break;
+          case 1: hpass = first ? cgs_pass<G, 2, true>(s, N, 2, &w02) : cgs_pass<G, 2>(s, N, 2); break;
+          case 2: hpass = first ? cgs_pass<G, 3, true>(s, N, 3, &w02) : cgs_pass<G, 3>(s, N, 3); break;
+          default: hpass = cgs_pass<G, 4>(s, N, 4); break;  // (the last column has no breakdown test to feed)
         }
       } else {
-        cgs_pass<G, 0>(s, N, j + 1, hcol);
+        hpass = cgs_pass<G, 0>(s, N, j + 1);
       }
+      hcol = pass == 0 ? hpass : hcol + hpass;
     }
-    if (g.lane == 0) {
-#pragma unroll
-      for (int i = 0; i < MAXM; ++i)
-        if (i <= j) s.H[i * MAXM + j] = hcol[i];
-    }
+    if (g.lane <= j) s.H[g.lane * MAXM + j] = hcol;
     if (j + 1 == M) break;
     const double hn2 = group_dot<G>(g, s.w, s.w, N);
     if (hn2 <= brk2 * w02 || hn2 == 0.0) {
@@ -2164,8 +2193,7 @@ __device__ inline void factor_small(const SlotPtrs& s, int mdim, double h) {
 
 // One stage of the transformed form (Eq. s_stage_row_transformed) with the
 // low-rank inverse (Eq. solve_kry_jac), in two parts.  stage_rhs: F_i = f_i +
-// G_i with G_i = sum_{j<i} (gamma_ij / gamma) k_j (F_i and G_i left in s.F and
-// s.w) and the partial sums of Q^T F_i.  stage_solve: c = (I - (I - h gamma
+// G_i with G_i = sum_{j<i} (gamma_ij / gamma) k_j (G_i left in s.w) and the partial sums of Q^T F_i.  stage_solve: c = (I - (I - h gamma
 // H)^-1) Q^T F_i (B = I - (I - h gamma H)^-1 from factor_small) and
 // k_i = F_i - Q c - G_i.  I >= 0: the stage known at compile time; MD > 0: the
 // basis dimension known at compile time, so no term carries a predicate (a
@@ -2194,7 +2222,6 @@ __device__ __forceinline__ void stage_rhs(const SlotPtrs& s, int N, int i_rt, in
     else if (i == 2) Ge = fma(g32, K1[e], g31 * K0[e]);
     else if (i == 3) Ge = fma(g43, K2[e], fma(g42, K1[e], g41 * K0[e]));
     const double Fe = fi[e] + Ge;
-    s.F[e] = Fe;
     s.w[e] = Ge;
 #pragma unroll
     for (int l = 0; l < LM; ++l)
@@ -2203,7 +2230,8 @@ __device__ __forceinline__ void stage_rhs(const SlotPtrs& s, int N, int i_rt, in
 }
 
 template <int G, int MD>
-__device__ __forceinline__ void stage_solve(const SlotPtrs& s, int N, int i, int mdim_rt, double (&part)[MAXM]) {
+__device__ __forceinline__ void stage_solve(const SlotPtrs& s, int N, int i, int mdim_rt, const double* fi,
+                                            double (&part)[MAXM]) {
   const Grp<G> g;
   const int Nq = s.Nq;
   const int mdim = MD > 0 ? MD : mdim_rt;
@@ -2226,7 +2254,8 @@ __device__ __forceinline__ void stage_solve(const SlotPtrs& s, int N, int i, int
 #pragma unroll
     for (int l = 0; l < LM; ++l)
       if (MD > 0 || l < mdim) acc = fma(s.Q[l * Nq + e], cz[l], acc);
-    Ki[e] = (s.F[e] - acc) - s.w[e];
+    const double Ge = s.w[e];
+    Ki[e] = ((fi[e] + Ge) - acc) - Ge;  // F_i as in stage_rhs
   }
   g.sync();
 }
@@ -2269,7 +2298,7 @@ struct IntegrateParams {
   const double* rho_cell;      // constant-volume densities, or null (constant pressure)
   int nx;                      // state components after T (5: auxiliary-temperature system)
   int64_t mech_copy;           // bytes of the mechanism each block copies (a prefix, by precision)
-  int64_t fx_copy;             // bytes of the fixed-point segment copied after that (0: it does not fit)
+  int64_t fx_copy;             // bytes of the segment copied after that (without its fixed-point part where that does not fit)
   int64_t tc_bytes;            // precision 4: bytes of nu^T tiles copied after both (else 0)
 };
 
@@ -2279,7 +2308,7 @@ __device__ void integrate_cell(const MechView& m, const SlotPtrs& s, const Integ
   const int ns = m.ns, N = ns + 1 + m.nx, Nq = s.Nq;
   for (int e = g.lane; e < N; e += G) {
     s.u[e] = P.Y[cell * N + e];
-    s.src[e] = P.src ? P.src[cell * N + e] : 0.0;
+    if (P.S.src >= 0) s.src[e] = P.src ? P.src[cell * N + e] : 0.0;
   }
   g.sync();
   const double* srcp = P.src ? s.src : nullptr;
@@ -2294,7 +2323,8 @@ __device__ void integrate_cell(const MechView& m, const SlotPtrs& s, const Integ
   }
   if (fixed) h = P.fixed_h;
   const long long n_fixed = fixed ? llround(dt / P.fixed_h) : 0;
-  double t = 0.0, h_last = h;
+  double t = 0.0, left = dt, h_last = h;
+  const double tol_t = T_END_TOL * dt, inv_N = 1.0 / N;
   float lg_err_prev = 0.f;  // log2 err_n; err_n = 1 before the first step
   int n_acc = 0, n_rej = 0, n_rhs = 0, status = RK_CELL_OK, n_att = 0;
   CellScalars cs;
@@ -2316,14 +2346,14 @@ __device__ void integrate_cell(const MechView& m, const SlotPtrs& s, const Integ
     }
     if (fixed) {
       if (n_acc >= n_fixed) break;
-    } else if (dt - t <= T_END_TOL * dt) {
+    } else if (__double_as_longlong(left) <= __double_as_longlong(tol_t)) {  // (tol_t > 0; negative bits are below)
       break;
     }
     if (n_att >= P.max_attempts) {
       status = RK_CELL_MAX_ATTEMPTS;
       break;
     }
-    if (!fixed) h = fmin(h, dt - t);
+    if (!fixed && __double_as_longlong(left) < __double_as_longlong(h)) h = left;  // both positive
     if (G == 32 && mdim == 4) factor_four(s, h);
     else factor_small<G>(s, mdim, h);
     // ---- four stages (Algorithm 1); f is evaluated at stages 2 and 3 only
@@ -2351,10 +2381,10 @@ __device__ void integrate_cell(const MechView& m, const SlotPtrs& s, const Integ
           case 2: stage_rhs<G, 4, 2>(s, N, 2, 4, fi, part); break;
           default: stage_rhs<G, 4, 3>(s, N, 3, 4, fi, part); break;
         }
-        stage_solve<G, 4>(s, N, i, 4, part);
+        stage_solve<G, 4>(s, N, i, 4, fi, part);
       } else {
         stage_rhs<G, 0, -1>(s, N, i, mdim, fi, part);
-        stage_solve<G, 0>(s, N, i, mdim, part);
+        stage_solve<G, 0>(s, N, i, mdim, fi, part);
       }
     }
     // ---- solutions, error estimate
@@ -2370,7 +2400,7 @@ __device__ void integrate_cell(const MechView& m, const SlotPtrs& s, const Integ
       bad |= (__double2hiint(us) & 0x7ff00000) == 0x7ff00000;
       s.arg[e] = us;
     }
-    const double err = sqrt(g.sum(part) * (1.0 / N));
+    const double err2 = g.sum(part) * inv_N;  // err*^2
     bad = g.any(bad);
     const int att = n_att;
     n_att += 1;
@@ -2383,16 +2413,17 @@ __device__ void integrate_cell(const MechView& m, const SlotPtrs& s, const Integ
     } else {
       // h* = h min(5, max(0.2, 0.8 err_n^beta / err*^alpha)), the factor in
       // FP32 as 2^(beta log2 err_n - alpha log2 err*) (log2 err_n kept from
-      // acceptance); the accept test err <= 1 stays FP64
-      const bool fin = (__double2hiint(err) & 0x7ff00000) != 0x7ff00000;
+      // acceptance; the logarithm of the square halved).  err* <= 1 is err*^2 <= 1,
+      // compared through the bits
+      const bool fin = (__double2hiint(err2) & 0x7ff00000) != 0x7ff00000;
       float fac = (float)FAC_MIN;
       if (fin) {
-        lg_err = __log2f(fmaxf(__double2float_rn(err), (float)ERR_FLOOR));
+        lg_err = fmaxf(0.5f * __log2f(float_bits(err2)), LOG2_ERR_FLOOR);
         fac = fminf((float)FAC_MAX,
                     fmaxf((float)FAC_MIN, (float)SAFETY * exp2f((float)PI_BETA * lg_err_prev - (float)PI_ALPHA * lg_err)));
       }
-      hnew = h * (double)fac;
-      accept = fin && err <= 1.0;
+      hnew = h * double_bits(fac);
+      accept = fin && __double_as_longlong(err2) <= 0x3ff0000000000000ll;
     }
     if (P.trace && att < P.trace_cap && g.lane == 0) P.trace[cell * P.trace_cap + att] = accept ? h : -h;
     if (accept) {
@@ -2403,11 +2434,13 @@ __device__ void integrate_cell(const MechView& m, const SlotPtrs& s, const Integ
       for (int e = g.lane; e < N; e += G) s.u[e] = s.arg[e];
       g.sync();
       t += h;
+      left = dt - t;
       if (!fixed) lg_err_prev = lg_err;
       n_acc += 1;
       h_last = hnew;
       h = hnew;
-      const bool done = fixed ? (n_acc >= n_fixed) : (dt - t <= T_END_TOL * dt);
+      const bool done =
+          fixed ? (n_acc >= n_fixed) : __double_as_longlong(left) <= __double_as_longlong(tol_t);
       fresh = !done;
     } else {
       n_rej += 1;
@@ -2451,7 +2484,6 @@ __device__ inline void init_sentinels(const SlotPtrs& s, int ns, int lane) {
     s.hRT[ns] = 0.0;
     s.gRT[ns] = 0.0;
     s.E[ns] = 1.0;
-    s.Einv[ns] = 1.0;
     s.CE[ns] = 1.0;
     if (MIXED) {
       s.fC[ns] = 1.f;
@@ -2523,15 +2555,15 @@ __device__ __forceinline__ void drain_queue(const IntegrateParams& P, const Grp<
   }
 }
 
-template <int G, bool MIXED, bool TC = false>
-__global__ void __launch_bounds__(MAX_BLOCK_THREADS, 1) rok4e_integrate_kernel(IntegrateParams P) {
+template <int G, bool MIXED, bool TC = false, int THREADS = MAX_BLOCK_THREADS>
+__global__ void __launch_bounds__(THREADS, 1) rok4e_integrate_kernel(IntegrateParams P) {
   extern __shared__ __align__(16) unsigned char smem[];
   load_exp_table(reinterpret_cast<uint64_t*>(smem));
   load_mech(smem + EXP_TAB_BYTES, P.mech, P.mech_copy);
-  load_mech(smem + EXP_TAB_BYTES + P.mech_copy, P.mech + P.L.off_fA, P.fx_copy);
+  load_mech(smem + EXP_TAB_BYTES + P.mech_copy, P.mech + P.L.off_lo, P.fx_copy);
   if (TC) load_mech(smem + EXP_TAB_BYTES + P.mech_copy + P.fx_copy, P.mech + P.L.off_nuT, P.tc_bytes);
   __syncthreads();
-  MechView m = make_view(smem + EXP_TAB_BYTES, P.mech, P.L, P.mech_copy, P.fx_copy > 0);
+  MechView m = make_view(smem + EXP_TAB_BYTES, P.mech, P.L, P.mech_copy, P.fx_copy > P.L.off_fA - P.L.off_lo);
   m.etab = reinterpret_cast<const uint64_t*>(smem);
   m.nx = P.nx;
   if (TC) m.nuT = reinterpret_cast<const uint4*>(smem + EXP_TAB_BYTES + P.mech_copy + P.fx_copy);
@@ -2575,7 +2607,7 @@ __device__ void integrate_cell_rkdp(const MechView& m, const SlotPtrs& s, const 
   const int ns = m.ns, N = ns + 1 + m.nx, Nq = s.Nq;
   for (int e = g.lane; e < N; e += G) {
     s.u[e] = P.Y[cell * N + e];
-    s.src[e] = P.src ? P.src[cell * N + e] : 0.0;
+    if (P.S.src >= 0) s.src[e] = P.src ? P.src[cell * N + e] : 0.0;
   }
   g.sync();
   const double* srcp = P.src ? s.src : nullptr;
@@ -2700,13 +2732,13 @@ __device__ void integrate_cell_rkdp(const MechView& m, const SlotPtrs& s, const 
 }
 
 template <int G>
-__global__ void __launch_bounds__(MAX_BLOCK_THREADS) rkdp_integrate_kernel(IntegrateParams P) {
+__global__ void __launch_bounds__(rkdp_threads(G), 1) rkdp_integrate_kernel(IntegrateParams P) {
   extern __shared__ __align__(16) unsigned char smem[];
   load_exp_table(reinterpret_cast<uint64_t*>(smem));
   load_mech(smem + EXP_TAB_BYTES, P.mech, P.mech_copy);
-  load_mech(smem + EXP_TAB_BYTES + P.mech_copy, P.mech + P.L.off_fA, P.fx_copy);
+  load_mech(smem + EXP_TAB_BYTES + P.mech_copy, P.mech + P.L.off_lo, P.fx_copy);
   __syncthreads();
-  MechView m = make_view(smem + EXP_TAB_BYTES, P.mech, P.L, P.mech_copy, P.fx_copy > 0);
+  MechView m = make_view(smem + EXP_TAB_BYTES, P.mech, P.L, P.mech_copy, P.fx_copy > P.L.off_fA - P.L.off_lo);
   m.etab = reinterpret_cast<const uint64_t*>(smem);
   m.nx = P.nx;
   const Grp<G> g;
@@ -2746,7 +2778,7 @@ template <int G>
 __global__ void __launch_bounds__(128) rok4e_adjoint_kernel(AdjointParams P) {
   extern __shared__ __align__(16) unsigned char smem[];
   load_exp_table(reinterpret_cast<uint64_t*>(smem));
-  // everything before the nu^T tiles but the fixed-point segment
+  // everything before the nu^T tiles but the integrators' segment
   unsigned char* base = smem + EXP_TAB_BYTES;
   load_mech(base, P.mech, P.L.bytes_f32);
   load_mech(base + P.L.bytes_f32, P.mech + P.L.off_fx_end, P.L.off_nuT - P.L.off_fx_end);
@@ -2754,6 +2786,10 @@ __global__ void __launch_bounds__(128) rok4e_adjoint_kernel(AdjointParams P) {
   MechView m = make_view(base, P.mech, P.L, P.L.bytes_f32, false);
   const unsigned char* tail = base + P.L.bytes_f32 - P.L.off_fx_end;
   m.lnA = reinterpret_cast<const double*>(tail + P.L.off_lnA);
+  m.bexp = reinterpret_cast<const double*>(tail + P.L.off_b);
+  m.EaR = reinterpret_cast<const double*>(tail + P.L.off_EaR);
+  m.lo = reinterpret_cast<const double*>(tail + P.L.off_lo17);
+  m.hi = reinterpret_cast<const double*>(tail + P.L.off_hi17);
   m.csr_nu = reinterpret_cast<const double*>(tail + P.L.off_csr_nu);
   m.csr_ptr = reinterpret_cast<const int32_t*>(tail + P.L.off_csr_ptr);
   m.role_ptr = reinterpret_cast<const int32_t*>(tail + P.L.off_role_ptr);
@@ -2796,7 +2832,7 @@ struct PointParams {
   const double* rho_cell;  // constant-volume densities, or null
   int nx;                  // state components after T (5: auxiliary-temperature system)
   int64_t mech_copy;       // bytes of the mechanism copied to shared memory (a prefix)
-  int64_t fx_copy;         // bytes of the fixed-point segment copied after that (0: it does not fit)
+  int64_t fx_copy;         // bytes of the segment copied after that (without its fixed-point part where that does not fit)
   int64_t tc_bytes;        // modes 6 and 7: bytes of nu^T tiles copied after both (else 0)
 };
 
@@ -2805,10 +2841,10 @@ __global__ void __launch_bounds__(MAX_BLOCK_THREADS) chem_point_kernel(PointPara
   extern __shared__ __align__(16) unsigned char smem[];
   load_exp_table(reinterpret_cast<uint64_t*>(smem));
   load_mech(smem + EXP_TAB_BYTES, P.mech, P.mech_copy);
-  load_mech(smem + EXP_TAB_BYTES + P.mech_copy, P.mech + P.L.off_fA, P.fx_copy);
+  load_mech(smem + EXP_TAB_BYTES + P.mech_copy, P.mech + P.L.off_lo, P.fx_copy);
   if (P.tc_bytes) load_mech(smem + EXP_TAB_BYTES + P.mech_copy + P.fx_copy, P.mech + P.L.off_nuT, P.tc_bytes);
   __syncthreads();
-  MechView m = make_view(smem + EXP_TAB_BYTES, P.mech, P.L, P.mech_copy, P.fx_copy > 0);
+  MechView m = make_view(smem + EXP_TAB_BYTES, P.mech, P.L, P.mech_copy, P.fx_copy > P.L.off_fA - P.L.off_lo);
   m.etab = reinterpret_cast<const uint64_t*>(smem);
   m.nx = P.nx;
   if (P.tc_bytes) m.nuT = reinterpret_cast<const uint4*>(smem + EXP_TAB_BYTES + P.mech_copy + P.fx_copy);
@@ -2909,15 +2945,15 @@ inline int device_props(int* n_sm, size_t* smem_optin) {
   return RK_OK;
 }
 
-// The bytes of the fixed-point segment a block copies: all of it, or none where it
-// and `rest` (the prefix, one cell's slot, tiles) do not fit in shared memory; such
-// a mechanism runs in the direct form.
-inline int64_t fixed_segment(const MechLayout& L, int64_t rest) {
+// The bytes of the segment a block copies: all of it, or the thermo coefficients
+// alone where it and `rest` (the prefix, one cell's slot, tiles) do not fit in
+// shared memory; such a mechanism runs in the direct form.
+inline int64_t segment_bytes(const MechLayout& L, int64_t rest) {
   int n_sm = 0;
   size_t smem_max = 0;
-  if (device_props(&n_sm, &smem_max) != RK_OK) return 0;
-  const int64_t seg = L.off_fx_end - L.off_fA;
-  return rest + seg + EXP_TAB_BYTES + 64 <= (int64_t)smem_max ? seg : 0;
+  const int64_t seg = L.off_fx_end - L.off_lo;
+  if (device_props(&n_sm, &smem_max) != RK_OK) return seg;
+  return rest + seg + EXP_TAB_BYTES + 64 <= (int64_t)smem_max ? seg : L.off_fA - L.off_lo;
 }
 
 // Shared memory that precision 4 counts beside its tiles when it decides whether
@@ -2940,7 +2976,8 @@ inline int64_t tensor_core_bytes(const MechLayout& L, int M, int nx) {
 
 template <int G, typename K>
 int plan_for(K kernel, const rk_mech* mech, const SlotLayout& S, int want_cells, int64_t ncell, bool persistent,
-             LaunchPlan* plan, int want_blocks_per_sm = 0, bool fill_device = false, int64_t copy_bytes = -1) {
+             LaunchPlan* plan, int want_blocks_per_sm = 0, bool fill_device = false, int64_t copy_bytes = -1,
+             int max_threads = MAX_BLOCK_THREADS) {
   int n_sm = 0;
   size_t smem_max = 0;
   int rc = device_props(&n_sm, &smem_max);
@@ -2951,7 +2988,7 @@ int plan_for(K kernel, const rk_mech* mech, const SlotLayout& S, int want_cells,
   if (mech_bytes + slot_bytes > smem_max)
     return set_error(RK_E_UNSUPPORTED, "mechanism plus one cell's work arrays exceed shared memory");
   int cells = (int)((smem_max - mech_bytes) / slot_bytes);
-  cells = cells > MAX_BLOCK_THREADS / G ? MAX_BLOCK_THREADS / G : cells;
+  cells = cells > max_threads / G ? max_threads / G : cells;
   if (want_cells > 0 && want_cells < cells) cells = want_cells;
   if (!persistent && (int64_t)cells > ncell) cells = (int)(ncell > 0 ? ncell : 1);
   size_t smem = mech_bytes + (size_t)cells * slot_bytes;
@@ -2991,6 +3028,8 @@ struct IntegrateLaunch {
 };
 template <int G, bool MIXED, bool TC>
 int launch_rok4e(const IntegrateLaunch& a);
+template <int THREADS>
+int launch_rok4e_wide(const IntegrateLaunch& a);  // FP64, one warp per cell, more than eight cells a block
 template <int G>
 int launch_rkdp(const IntegrateLaunch& a);
 template <int G>

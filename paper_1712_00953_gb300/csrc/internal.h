@@ -17,8 +17,9 @@
 
 namespace rk {
 
-// Thermo coefficients stored per species and per range, coefficient-major
-// ([NCOEF][ns]):
+// The seven NASA-7 coefficients a1..a7 per species and per range, coefficient-major
+// ([7][ns], off_lo and off_hi); and, for the adjoint, with the factors of its
+// polynomials divided out ([NCOEF][ns], off_lo17 and off_hi17):
 //   0..4   a1..a5                 cp/R = a1 + T(a2 + T(a3 + T(a4 + T a5)))
 //   5..8   a2/2, a3/3, a4/4, a5/5 h/RT = a1 + T(c5 + T(c6 + T(c7 + T c8))) + a6/T
 //   9      a6
@@ -35,9 +36,8 @@ struct MechLayout {
   int32_t nnz = 0;  // entries of the species-major stoichiometry list
   int32_t npiece = 0;  // pieces the list is split into for the gather (>= ns)
   // byte offsets into the packed buffer (all multiples of 16)
-  int64_t off_W = 0, off_invW = 0, off_Tmid = 0, off_lo = 0, off_hi = 0;
-  int64_t off_b = 0, off_EaR = 0;
-  int64_t off_lnA = 0;  // read from global memory (Troe passes, cells off the fixed-point form)
+  int64_t off_W = 0, off_invW = 0, off_Tmid = 0, off_lo = 0, off_hi = 0, off_lo17 = 0, off_hi17 = 0;
+  int64_t off_lnA = 0, off_b = 0, off_EaR = 0;  // read from global memory (d ln k/dT, Troe, the direct form)
   // fixed-point Arrhenius coefficients (fx.cuh), uint64 per reaction: log2 A 2^52, (b + 32) 2^57,
   // (Ea/R log2 e + 2^15) 2^46; fx: every reaction's fit their ranges
   int32_t fx = 0;
@@ -76,8 +76,9 @@ struct MechLayout {
   int64_t bytes = 0;
   // what kernels copy to shared memory: a prefix of the buffer -- through the base
   // arrays; also the list in pieces of the double-float gathers; also the FP32
-  // copies -- and, after it, the fixed-point segment [off_fA, off_fx_end): the
-  // Arrhenius coefficients and the gather list
+  // copies -- and, after it, the segment [off_lo, off_fx_end): the thermo
+  // coefficients, then (from off_fA) the fixed-point Arrhenius coefficients and
+  // the gather list
   int64_t bytes_base = 0, bytes_df = 0, bytes_f32 = 0, off_fx_end = 0;
 };
 

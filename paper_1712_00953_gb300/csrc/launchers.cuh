@@ -8,16 +8,53 @@ namespace rk {
 
 // Persistent ROK4E launch: as many cells per block as shared memory allows
 // (or a.cells_per_block), one wave of blocks sized to the device.
-template <int G, bool MIXED, bool TC>
-int launch_rok4e(const IntegrateLaunch& a) {
+template <int G, bool MIXED, bool TC, int THREADS>
+int launch_rok4e_kernel(const IntegrateLaunch& a) {
   IntegrateParams& P = *a.P;
   LaunchPlan plan;
-  const int rc = plan_for<G>(rok4e_integrate_kernel<G, MIXED, TC>, a.mech, P.S, a.cells_per_block, a.ncell, true,
-                             &plan, a.blocks_per_sm, a.static_bins, P.mech_copy + P.fx_copy + P.tc_bytes);
+  const int rc =
+      plan_for<G>(rok4e_integrate_kernel<G, MIXED, TC, THREADS>, a.mech, P.S, a.cells_per_block, a.ncell, true, &plan,
+                  a.blocks_per_sm, a.static_bins, P.mech_copy + P.fx_copy + P.tc_bytes, THREADS);
   if (rc) return rc;
   if (a.static_bins) P.subq = plan.cells_per_block % 4 == 0 ? 4 : (plan.cells_per_block % 2 == 0 ? 2 : 1);
-  rok4e_integrate_kernel<G, MIXED, TC><<<plan.blocks, plan.cells_per_block * G, plan.smem, a.stream>>>(P);
+  rok4e_integrate_kernel<G, MIXED, TC, THREADS>
+      <<<plan.blocks, plan.cells_per_block * G, plan.smem, a.stream>>>(P);
   return RK_OK;
+}
+template <int THREADS>
+int launch_rok4e_wide(const IntegrateLaunch& a) {
+  return launch_rok4e_kernel<32, false, false, THREADS>(a);
+}
+
+extern template int launch_rok4e_wide<384>(const IntegrateLaunch&);
+extern template int launch_rok4e_wide<512>(const IntegrateLaunch&);
+
+// FP64 cells one to a warp: an attempt is a chain of dependent instructions that
+// leaves its sub-partition idle a third of the time with two warps on it, so more
+// cells to an SM finish more of them, each with fewer registers (168 with up to
+// twelve warps, 128 with sixteen; 0 and 300 bytes of spills).  Which cells fit is
+// the mechanism's size.  With few cells for each SM the step lasts as long as its
+// slowest cells, which run fastest on eight warps.
+inline int rok4e_threads(const IntegrateLaunch& a) {
+  const IntegrateParams& P = *a.P;
+  int n_sm = 0;
+  size_t smem_max = 0;
+  if (device_props(&n_sm, &smem_max) != RK_OK) return MAX_BLOCK_THREADS;
+  const int64_t room = (int64_t)smem_max - 64 - EXP_TAB_BYTES - P.mech_copy - P.fx_copy;
+  int64_t cells = room / ((int64_t)P.S.stride * 8);
+  if (a.cells_per_block > 0 && a.cells_per_block < cells) cells = a.cells_per_block;
+  if (cells <= 8 || a.ncell < (int64_t)WIDE_MIN_CELLS_PER_SM * n_sm) return MAX_BLOCK_THREADS;
+  return cells <= 12 ? 384 : 512;
+}
+
+template <int G, bool MIXED, bool TC>
+int launch_rok4e(const IntegrateLaunch& a) {
+  if constexpr (G == 32 && !MIXED && !TC) {
+    const int threads = rok4e_threads(a);
+    if (threads == 384) return launch_rok4e_wide<384>(a);
+    if (threads == 512) return launch_rok4e_wide<512>(a);
+  }
+  return launch_rok4e_kernel<G, MIXED, TC, MAX_BLOCK_THREADS>(a);
 }
 
 // Persistent explicit Dormand-Prince launch, planned like ROK4E's.
@@ -26,7 +63,7 @@ int launch_rkdp(const IntegrateLaunch& a) {
   IntegrateParams& P = *a.P;
   LaunchPlan plan;
   const int rc = plan_for<G>(rkdp_integrate_kernel<G>, a.mech, P.S, a.cells_per_block, a.ncell, true, &plan,
-                             a.blocks_per_sm, a.static_bins, P.mech_copy + P.fx_copy);
+                             a.blocks_per_sm, a.static_bins, P.mech_copy + P.fx_copy, rkdp_threads(G));
   if (rc) return rc;
   if (a.static_bins) P.subq = plan.cells_per_block % 4 == 0 ? 4 : (plan.cells_per_block % 2 == 0 ? 2 : 1);
   rkdp_integrate_kernel<G><<<plan.blocks, plan.cells_per_block * G, plan.smem, a.stream>>>(P);

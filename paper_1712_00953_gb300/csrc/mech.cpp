@@ -329,10 +329,6 @@ bool pack_mechanism(const void* vdesc, HostMech* out, std::string* err) {
   L.off_W = take(8 * ns);
   L.off_invW = take(8 * ns);
   L.off_Tmid = take(8 * ns);
-  L.off_lo = take(8 * (int64_t)NCOEF * ns);
-  L.off_hi = take(8 * (int64_t)NCOEF * ns);
-  L.off_b = take(8 * (int64_t)nr);
-  L.off_EaR = take(8 * (int64_t)nr);
   L.off_eff = take(8 * (int64_t)L.ntb * ns);
   L.off_fo = take(8 * (int64_t)L.ntb * FO_STRIDE);
   L.off_slots = take(4 * (int64_t)nr);
@@ -340,7 +336,8 @@ bool pack_mechanism(const void* vdesc, HostMech* out, std::string* err) {
   // what only some kernels read comes last (internal.h): FP64 paths copy the base
   // arrays, the double-float gathers also the list in pieces with csr_nuf, the FP32
   // Jacobian-vector product the other FP32 copies; each adds the fixed-point
-  // segment; the rest is read from global memory
+  // segment of the thermo coefficients and the fixed-point form; the rest is read
+  // from global memory
   L.bytes_base = off;
   L.off_csr_j = take(4 * (int64_t)nnz);
   L.off_piece_ptr = take(4 * (int64_t)(npiece + 1));
@@ -353,6 +350,8 @@ bool pack_mechanism(const void* vdesc, HostMech* out, std::string* err) {
   L.off_EaRf = take(4 * (int64_t)nr);
   L.off_efff = take(4 * (int64_t)L.ntb * ns);
   L.bytes_f32 = off;
+  L.off_lo = take(8 * 7 * (int64_t)ns);
+  L.off_hi = take(8 * 7 * (int64_t)ns);
   L.off_fA = take(8 * (int64_t)nr);
   L.off_fb = take(8 * (int64_t)nr);
   L.off_fE = take(8 * (int64_t)nr);
@@ -360,6 +359,10 @@ bool pack_mechanism(const void* vdesc, HostMech* out, std::string* err) {
   L.off_gspec = take(4 * (int64_t)(2 * ns + 1));
   L.off_fx_end = off;
   L.off_lnA = take(8 * (int64_t)nr);
+  L.off_b = take(8 * (int64_t)nr);
+  L.off_EaR = take(8 * (int64_t)nr);
+  L.off_lo17 = take(8 * (int64_t)NCOEF * ns);
+  L.off_hi17 = take(8 * (int64_t)NCOEF * ns);
   L.off_csr_nu = take(8 * (int64_t)nnz);
   L.off_csr_ptr = take(4 * (int64_t)(ns + 1));
   L.off_perm = take(4 * (int64_t)nr);
@@ -401,7 +404,9 @@ bool pack_mechanism(const void* vdesc, HostMech* out, std::string* err) {
     D(L.off_Tmid)[k] = nk[1];
     for (int range = 0; range < 2; ++range) {
       const double* a = nk + 3 + 7 * range;
-      double* c = D(range == 0 ? L.off_lo : L.off_hi);
+      double* c = D(range == 0 ? L.off_lo17 : L.off_hi17);
+      double* c7 = D(range == 0 ? L.off_lo : L.off_hi);
+      for (int i = 0; i < 7; ++i) c7[(size_t)i * ns + k] = a[i];
       const double v[NCOEF] = {a[0],       a[1],       a[2],       a[3],       a[4],      a[1] / 2.0,
                                a[2] / 3.0, a[3] / 4.0, a[4] / 5.0, a[5],       a[2] / 2.0, a[3] / 3.0,
                                a[4] / 4.0, a[6],       2.0 * a[2], 3.0 * a[3], 4.0 * a[4]};

@@ -355,7 +355,8 @@ int integrate_impl(const rk_mech* mech, double* Y, const double* src, double* h_
   P.mech = mech->dev;
   P.L = mech->host.L;
   P.nx = nx;
-  P.S = make_slot(mech->host.L, Meff, mixed, nx, o.precision == 3, tc, o.precision == 6);
+  P.S = make_slot(mech->host.L, Meff, method == 1 ? SLOT_RKDP : SLOT_ROK4E, mixed, nx, o.precision == 3, tc,
+                  o.precision == 6, src || nx > 0 || (method == 0 && o.jv_mode == 1));
   P.precision = o.precision;
   P.Y = Y;
   P.src = src;
@@ -382,7 +383,7 @@ int integrate_impl(const rk_mech* mech, double* Y, const double* src, double* h_
     P.mech_copy = o.precision == 1 || o.precision == 3 ? L.bytes_df
                                                        : (o.precision == 2 ? L.bytes_f32 : L.bytes_base);
     P.tc_bytes = tc ? (int64_t)16 * 32 * L.nst * L.nrt : 0;
-    P.fx_copy = fixed_segment(L, P.mech_copy + P.tc_bytes + (int64_t)P.S.stride * 8);
+    P.fx_copy = segment_bytes(L, P.mech_copy + P.tc_bytes + (int64_t)P.S.stride * 8);
     int n_sm = 0;
     size_t smem_max = 0;
     if (tc && (rc = device_props(&n_sm, &smem_max))) return rc;
@@ -519,7 +520,7 @@ static int point_call(const rk_mech* mech, const double* Y, const double* src, c
   P.nx = nx;
   P.mech = mech->dev;
   P.L = mech->host.L;
-  P.S = make_slot(mech->host.L, 1, mode >= 3 && mode <= 5, nx, mode == 5, tc, mode == 8);
+  P.S = make_slot(mech->host.L, 1, SLOT_POINT, mode >= 3 && mode <= 5, nx, mode == 5, tc, mode == 8, true);
   P.Y = Y;
   P.src = src;
   P.V = V;
@@ -531,7 +532,7 @@ static int point_call(const rk_mech* mech, const double* Y, const double* src, c
     const MechLayout& L = mech->host.L;  // the arrays that the mode's precision reads
     P.mech_copy = mode == 3 || mode == 5 ? L.bytes_df : (mode == 4 ? L.bytes_f32 : L.bytes_base);
     P.tc_bytes = tc ? (int64_t)16 * 32 * L.nst * L.nrt : 0;
-    P.fx_copy = fixed_segment(L, P.mech_copy + P.tc_bytes + (int64_t)P.S.stride * 8);
+    P.fx_copy = segment_bytes(L, P.mech_copy + P.tc_bytes + (int64_t)P.S.stride * 8);
   }
   LaunchPlan plan;
   rc = plan_for<32>(chem_point_kernel<32>, mech, P.S, 8, ncell, false, &plan, 0, false,
@@ -1079,7 +1080,7 @@ int rk_rok4e_adjoint_ex(const rk_mech* mech, const double* checkpoints, const do
   if (G != 4 && G != 8 && G != 16 && G != 32)
     return set_error(RK_E_INVALID_ARGUMENT, "lanes_per_cell must be 0, 4, 8, 16 or 32");
   const MechLayout& L = mech->host.L;
-  const size_t smem = (size_t)(L.off_nuT - (L.off_fx_end - L.off_fA)) + EXP_TAB_BYTES;
+  const size_t smem = (size_t)(L.off_nuT - (L.off_fx_end - L.off_lo)) + EXP_TAB_BYTES;
   cudaError_t e = cudaSuccess;
   rc = G == 4 ? launch_adjoint<4>(P, smem, st)
               : (G == 8 ? launch_adjoint<8>(P, smem, st)
