@@ -80,6 +80,7 @@ constexpr int MAX_BLOCK_THREADS = 256;
 #endif
 constexpr int WIDE_MIN_CELLS_PER_SM = RK_WIDE_MIN;
 // the explicit integrator fits 128 registers with one warp per cell
+constexpr int POINT_BLOCK_THREADS = 512;
 constexpr int rkdp_threads(int G) { return G == 32 ? 512 : MAX_BLOCK_THREADS; }
 constexpr int EXP_TAB_BYTES = RK_FX_EXP2_N * 8;  // leads the dynamic shared memory
 
@@ -334,7 +335,8 @@ struct SlotLayout {
 // Arrays whose lives do not meet share storage, so that an SM holds more cells
 // (a warp each): with 19.2 kB at 53 species / 325 reactions instead of 22.7, and a
 // mechanism copy of 22 instead of 48 kB, ten instead of eight.
-enum SlotKind { SLOT_ROK4E, SLOT_RKDP, SLOT_POINT };
+// SLOT_RHS: one source term, no Jacobian caches or vectors.
+enum SlotKind { SLOT_ROK4E, SLOT_RKDP, SLOT_POINT, SLOT_RHS };
 inline SlotLayout make_slot(const MechLayout& L, int M, SlotKind kind, bool mixed, int nx, bool df, bool tc,
                             bool f32jv, bool src) {
   SlotLayout s;
@@ -352,15 +354,16 @@ inline SlotLayout make_slot(const MechLayout& L, int M, SlotKind kind, bool mixe
   const int N = s.N, ns1 = L.ns + 1;
   s.u = take(N);
   s.src = src ? take(N) : -1;
-  s.fn = take(N);
+  const bool rhs = kind == SLOT_RHS;
+  s.fn = rhs ? s.u : take(N);  // (not used)
   s.arg = take(N);
   // a stage's f may overwrite its argument, except in the auxiliary-temperature
   // system, whose T row reads the argument after the species rows are written
   s.fr = kind != SLOT_RKDP && nx > 0 ? take(N) : s.arg;
-  s.F = kind != SLOT_ROK4E ? take(N) : -1;  // RKDP: a stage vector; point kernel: V
-  s.w = take(N);
+  s.F = kind == SLOT_RKDP || kind == SLOT_POINT ? take(N) : -1;  // a stage vector; the point kernel's V
+  s.w = rhs ? s.u : take(N);
   const int Nq = (N + 1) & ~1;  // stride between Krylov / stage vectors
-  s.Q = take(Nq * M);
+  s.Q = rhs ? s.u : take(Nq * M);
   s.CE = take(ns1);
   // C is read beside CE only by third-body sums and the reduced-precision J v
   s.C = L.ntb > 0 || mixed || df || f32jv ? take(ns1) : s.CE;
@@ -372,15 +375,15 @@ inline SlotLayout make_slot(const MechLayout& L, int M, SlotKind kind, bool mixe
   s.om = s.gRT;  // w is kept (caching evaluation) when the Gibbs factors are done with
   // reactions, and entry nr: the zero rate that pads the gather's pieces
   s.q = take(L.nr + 1);
-  s.kc = take(L.nr + 1);
-  s.qT = take(L.nr + 1);
+  s.kc = rhs ? s.q : take(L.nr + 1);
+  s.qT = rhs ? s.q : take(L.nr + 1);
   s.krc = take(L.nr + 1);
   // The stage vectors K live only inside an attempt; the J v caches kc, qT
   // (contiguous) only from the caching right-hand side to the end of the
   // Arnoldi process that precedes the attempts.  K shares their storage when
   // it fits there (not krc's, which holds the low words of the gather's rates).
   const int nr_even = (L.nr + 2) & ~1;
-  s.K = (4 * Nq <= 2 * nr_even) ? s.kc : take(4 * Nq);
+  s.K = rhs || 4 * Nq <= 2 * nr_even ? s.kc : take(4 * Nq);
   s.tb = take(4 * (L.ntb > 0 ? L.ntb : 1));
   s.tro = take(11 * (L.ntroe > 0 ? L.ntroe : 1));
   // the gather's pieces ((hi, lo) words in fixed point); LU and its pivots, used
@@ -2778,22 +2781,13 @@ template <int G>
 __global__ void __launch_bounds__(128) rok4e_adjoint_kernel(AdjointParams P) {
   extern __shared__ __align__(16) unsigned char smem[];
   load_exp_table(reinterpret_cast<uint64_t*>(smem));
-  // everything before the nu^T tiles but the integrators' segment
+  // everything before the integrators' segment
   unsigned char* base = smem + EXP_TAB_BYTES;
-  load_mech(base, P.mech, P.L.bytes_f32);
-  load_mech(base + P.L.bytes_f32, P.mech + P.L.off_fx_end, P.L.off_nuT - P.L.off_fx_end);
+  load_mech(base, P.mech, P.L.off_lo);
   __syncthreads();
-  MechView m = make_view(base, P.mech, P.L, P.L.bytes_f32, false);
-  const unsigned char* tail = base + P.L.bytes_f32 - P.L.off_fx_end;
-  m.lnA = reinterpret_cast<const double*>(tail + P.L.off_lnA);
-  m.bexp = reinterpret_cast<const double*>(tail + P.L.off_b);
-  m.EaR = reinterpret_cast<const double*>(tail + P.L.off_EaR);
-  m.lo = reinterpret_cast<const double*>(tail + P.L.off_lo17);
-  m.hi = reinterpret_cast<const double*>(tail + P.L.off_hi17);
-  m.csr_nu = reinterpret_cast<const double*>(tail + P.L.off_csr_nu);
-  m.csr_ptr = reinterpret_cast<const int32_t*>(tail + P.L.off_csr_ptr);
-  m.role_ptr = reinterpret_cast<const int32_t*>(tail + P.L.off_role_ptr);
-  m.role = reinterpret_cast<const int32_t*>(tail + P.L.off_role);
+  MechView m = make_view(base, base, P.L, P.L.off_lo, false);
+  m.lo = reinterpret_cast<const double*>(base + P.L.off_lo17);
+  m.hi = reinterpret_cast<const double*>(base + P.L.off_hi17);
   m.etab = reinterpret_cast<const uint64_t*>(smem);
   const Grp<G> g;
   const int gpb = blockDim.x / G;
@@ -2837,7 +2831,7 @@ struct PointParams {
 };
 
 template <int G>
-__global__ void __launch_bounds__(MAX_BLOCK_THREADS) chem_point_kernel(PointParams P) {
+__global__ void __launch_bounds__(POINT_BLOCK_THREADS, 1) chem_point_kernel(PointParams P) {
   extern __shared__ __align__(16) unsigned char smem[];
   load_exp_table(reinterpret_cast<uint64_t*>(smem));
   load_mech(smem + EXP_TAB_BYTES, P.mech, P.mech_copy);
@@ -2863,7 +2857,7 @@ __global__ void __launch_bounds__(MAX_BLOCK_THREADS) chem_point_kernel(PointPara
   for (int e = g.lane; e < N; e += G) {
     s.u[e] = P.Y[cell * N + e];
     s.src[e] = P.src ? P.src[cell * N + e] : 0.0;
-    if (P.V) s.F[e] = P.V[cell * N + e];
+    if (P.V && P.S.F >= 0) s.F[e] = P.V[cell * N + e];
   }
   g.sync();
   const double pr = P.rho_cell ? -P.rho_cell[cell] : P.p;

@@ -278,30 +278,33 @@ bool pack_mechanism(const void* vdesc, HostMech* out, std::string* err) {
   gpieces.resize(gnpp);
   // The sums are exact, so a piece's entries may come in any order: at each step the
   // 16 lanes of a half-warp take entries of different 8-byte shared-memory banks
-  // (index mod 16) where they can, lanes with the most entries left first.
+  // (index mod 16) where they can.
   const int gbat = (glen + 7) / 8;
   std::vector<uint16_t> gidx((size_t)gbat * 8 * gnpp, (uint16_t)(8 * nr));
   if (nr < 8191) {
-    std::vector<std::vector<int>> left = gpieces;
+    std::vector<int> done(gnpp, 0);  // entries already placed stand first in their piece
     for (int p0 = 0; p0 < gnpp; p0 += 16)
       for (int i = 0; i < glen; ++i) {
         int bank[16];
         for (int& b : bank) b = -1;
-        std::vector<int> lanes;
-        for (int p = p0; p < p0 + 16; ++p) lanes.push_back(p);
-        std::stable_sort(lanes.begin(), lanes.end(), [&](int a, int b) { return left[a].size() > left[b].size(); });
-        for (int p : lanes) {
-          auto& l = left[p];
-          size_t at = l.size();
-          for (size_t t = 0; t < l.size() && at == l.size(); ++t)
-            if (bank[l[t] & 15] < 0 || bank[l[t] & 15] == l[t]) at = t;
-          if (at == l.size()) {
-            if ((int)l.size() < glen - i) continue;  // padding for now; its entries still fit
-            at = 0;
+        for (int u = 0; u < 16; ++u) {
+          const int p = p0 + (u + i) % 16;  // the lane that chooses first goes round
+          auto& l = gpieces[p];
+          const int n = (int)l.size();
+          int at = n;
+          for (int t = done[p]; t < n; ++t)
+            if (bank[l[t] & 15] < 0 || bank[l[t] & 15] == l[t]) {
+              at = t;
+              break;
+            }
+          if (at == n) {
+            if (n - done[p] < glen - i) continue;  // padding for now; its entries still fit
+            at = done[p];
           }
-          bank[l[at] & 15] = l[at];
-          gidx[((size_t)(i / 8) * gnpp + p) * 8 + i % 8] = (uint16_t)(8 * l[at]);
-          l.erase(l.begin() + at);
+          const int j = l[at];
+          std::swap(l[at], l[done[p]++]);
+          bank[j & 15] = j;
+          gidx[((size_t)(i / 8) * gnpp + p) * 8 + i % 8] = (uint16_t)(8 * j);
         }
       }
   }
@@ -350,14 +353,6 @@ bool pack_mechanism(const void* vdesc, HostMech* out, std::string* err) {
   L.off_EaRf = take(4 * (int64_t)nr);
   L.off_efff = take(4 * (int64_t)L.ntb * ns);
   L.bytes_f32 = off;
-  L.off_lo = take(8 * 7 * (int64_t)ns);
-  L.off_hi = take(8 * 7 * (int64_t)ns);
-  L.off_fA = take(8 * (int64_t)nr);
-  L.off_fb = take(8 * (int64_t)nr);
-  L.off_fE = take(8 * (int64_t)nr);
-  L.off_gidx = take(16 * (int64_t)gbat * gnpp);
-  L.off_gspec = take(4 * (int64_t)(2 * ns + 1));
-  L.off_fx_end = off;
   L.off_lnA = take(8 * (int64_t)nr);
   L.off_b = take(8 * (int64_t)nr);
   L.off_EaR = take(8 * (int64_t)nr);
@@ -386,6 +381,14 @@ bool pack_mechanism(const void* vdesc, HostMech* out, std::string* err) {
   for (auto& v : roles) L.nrole += (int32_t)v.size();
   L.off_role_ptr = take(4 * (int64_t)(ns + 1));
   L.off_role = take(4 * (int64_t)(L.nrole > 0 ? L.nrole : 1));
+  L.off_lo = take(8 * 7 * (int64_t)ns);
+  L.off_hi = take(8 * 7 * (int64_t)ns);
+  L.off_fA = take(8 * (int64_t)nr);
+  L.off_fb = take(8 * (int64_t)nr);
+  L.off_fE = take(8 * (int64_t)nr);
+  L.off_gidx = take(16 * (int64_t)gbat * gnpp);
+  L.off_gspec = take(4 * (int64_t)(2 * ns + 1));
+  L.off_fx_end = off;
   L.nst = (ns + 15) / 16;
   L.nrt = (nr + 15) / 16;
   L.off_nuT = take(16 * 32 * (int64_t)L.nst * L.nrt);

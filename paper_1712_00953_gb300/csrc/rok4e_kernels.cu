@@ -520,7 +520,7 @@ static int point_call(const rk_mech* mech, const double* Y, const double* src, c
   P.nx = nx;
   P.mech = mech->dev;
   P.L = mech->host.L;
-  P.S = make_slot(mech->host.L, 1, SLOT_POINT, mode >= 3 && mode <= 5, nx, mode == 5, tc, mode == 8, true);
+  P.S = make_slot(mech->host.L, 1, needs_v ? SLOT_POINT : SLOT_RHS, mode >= 3 && mode <= 5, nx, mode == 5, tc, mode == 8, true);
   P.Y = Y;
   P.src = src;
   P.V = V;
@@ -535,8 +535,15 @@ static int point_call(const rk_mech* mech, const double* Y, const double* src, c
     P.fx_copy = segment_bytes(L, P.mech_copy + P.tc_bytes + (int64_t)P.S.stride * 8);
   }
   LaunchPlan plan;
-  rc = plan_for<32>(chem_point_kernel<32>, mech, P.S, 8, ncell, false, &plan, 0, false,
-                    P.mech_copy + P.fx_copy + P.tc_bytes);
+  // as many cells a block as fit (up to 16 warps of 128 registers; the block's copy of
+  // the mechanism serves them all), fewer where that would leave SMs without a block
+  int n_sm = 0;
+  size_t smem_max = 0;
+  if ((rc = device_props(&n_sm, &smem_max))) return rc;
+  const int64_t share = (ncell + n_sm - 1) / n_sm;
+  const int cells = (int)(share < POINT_BLOCK_THREADS / 32 ? share : POINT_BLOCK_THREADS / 32);
+  rc = plan_for<32>(chem_point_kernel<32>, mech, P.S, cells, ncell, false, &plan, 0, false,
+                    P.mech_copy + P.fx_copy + P.tc_bytes, POINT_BLOCK_THREADS);
   if (rc) return rc;
   chem_point_kernel<32><<<plan.blocks, plan.cells_per_block * 32, plan.smem, (cudaStream_t)stream>>>(P);
   cudaError_t e = cudaGetLastError();
@@ -1080,7 +1087,7 @@ int rk_rok4e_adjoint_ex(const rk_mech* mech, const double* checkpoints, const do
   if (G != 4 && G != 8 && G != 16 && G != 32)
     return set_error(RK_E_INVALID_ARGUMENT, "lanes_per_cell must be 0, 4, 8, 16 or 32");
   const MechLayout& L = mech->host.L;
-  const size_t smem = (size_t)(L.off_nuT - (L.off_fx_end - L.off_lo)) + EXP_TAB_BYTES;
+  const size_t smem = (size_t)L.off_lo + EXP_TAB_BYTES;
   cudaError_t e = cudaSuccess;
   rc = G == 4 ? launch_adjoint<4>(P, smem, st)
               : (G == 8 ? launch_adjoint<8>(P, smem, st)
