@@ -2026,7 +2026,7 @@ __device__ int arnoldi(const MechView& m, const SlotPtrs& s, const CellScalars& 
     // (only the breakdown threshold reads ||J q_j||^2: FP32 is enough there)
     double w02 = 0.0;
     if (MIXED) w02 = (double)group_dot_f<G>(g, s.w, s.w, N);
-    else if (M > 4) w02 = group_dot<G>(g, s.w, s.w, N);
+    else if (M > 6) w02 = group_dot<G>(g, s.w, s.w, N);
     double hcol = 0.0;  // lane i: h_ij
     for (int pass = 0; pass < 2; ++pass) {
       double hpass;
@@ -2054,14 +2054,16 @@ __device__ int arnoldi(const MechView& m, const SlotPtrs& s, const CellScalars& 
         hpass = hp[0];
 #pragma unroll
         for (int i = 1; i < MAXM; ++i) hpass = g.lane == i ? hp[i] : hpass;
-      } else if (M <= 4) {
-        const bool first = !MIXED && pass == 0;
+      } else if (M <= 6) {
+        const bool first = !MIXED && pass == 0 && j + 1 < M;  // (the last column has no breakdown test to feed)
         // the common Krylov dimensions: column j + 1 known at compile time
         switch (j) {
           case 0: hpass = first ? cgs_pass<G, 1, true>(s, N, 1, &w02) : cgs_pass<G, 1>(s, N, 1); break;
           case 1: hpass = first ? cgs_pass<G, 2, true>(s, N, 2, &w02) : cgs_pass<G, 2>(s, N, 2); break;
           case 2: hpass = first ? cgs_pass<G, 3, true>(s, N, 3, &w02) : cgs_pass<G, 3>(s, N, 3); break;
-          default: hpass = cgs_pass<G, 4>(s, N, 4); break;  // (the last column has no breakdown test to feed)
+          case 3: hpass = first ? cgs_pass<G, 4, true>(s, N, 4, &w02) : cgs_pass<G, 4>(s, N, 4); break;
+          case 4: hpass = first ? cgs_pass<G, 5, true>(s, N, 5, &w02) : cgs_pass<G, 5>(s, N, 5); break;
+          default: hpass = cgs_pass<G, 6>(s, N, 6); break;
         }
       } else {
         hpass = cgs_pass<G, 0>(s, N, j + 1);
@@ -2141,6 +2143,54 @@ __device__ __forceinline__ void factor_four(const SlotPtrs& s, double h) {
     v = r == p ? row : fma(-f, row, v);
   }
   if (c >= 4) s.Bm[r * MAXM + c - 4] = (c - 4 == r ? 1.0 : 0.0) - v;
+  __syncwarp();
+}
+
+// The same for m = 5 and 6, one column of [I - h gamma H | I] a lane (lanes past
+// 2 m repeat the last): a pivot column goes round by shuffles and every lane
+// eliminates its own column, m + 5 FP64 instructions a pivot.
+template <int M>
+__device__ __forceinline__ void factor_columns(const SlotPtrs& s, double h) {
+  const int lane = threadIdx.x & 31, c = min(lane, 2 * M - 1);
+  const unsigned all = 0xffffffffu;
+  const double hg = h * GAM;
+  double v[M];
+#pragma unroll
+  for (int r = 0; r < M; ++r) {
+    const double a = fma(-hg, s.H[r * MAXM + min(c, M - 1)], r == c ? 1.0 : 0.0);
+    v[r] = c < M ? a : (c - M == r ? 1.0 : 0.0);
+  }
+#pragma unroll
+  for (int p = 0; p < M; ++p) {
+    double f[M];
+#pragma unroll
+    for (int r = 0; r < M; ++r) f[r] = __shfl_sync(all, v[r], p);
+    int pr = p;
+    long long best = __double_as_longlong(f[p]) & 0x7fffffffffffffffll;
+#pragma unroll
+    for (int r = p + 1; r < M; ++r) {
+      const long long cand = __double_as_longlong(f[r]) & 0x7fffffffffffffffll;
+      pr = cand > best ? r : pr;
+      best = cand > best ? cand : best;
+    }
+#pragma unroll
+    for (int r = p + 1; r < M; ++r) {  // rows p and pr exchanged
+      const bool x = pr == r;
+      const double fp = f[p], vp = v[p];
+      f[p] = x ? f[r] : fp;
+      f[r] = x ? fp : f[r];
+      v[p] = x ? v[r] : vp;
+      v[r] = x ? vp : v[r];
+    }
+    v[p] *= rcp_any(f[p]);
+#pragma unroll
+    for (int r = 0; r < M; ++r)
+      if (r != p) v[r] = fma(-f[r], v[p], v[r]);
+  }
+  if (lane >= M && lane < 2 * M) {
+#pragma unroll
+    for (int r = 0; r < M; ++r) s.Bm[r * MAXM + lane - M] = (r == lane - M ? 1.0 : 0.0) - v[r];
+  }
   __syncwarp();
 }
 
@@ -2264,6 +2314,17 @@ __device__ __forceinline__ void stage_solve(const SlotPtrs& s, int N, int i, int
 }
 
 
+template <int G, int MD>
+__device__ __forceinline__ void stage_of(const SlotPtrs& s, int N, int i, const double* fi, double (&part)[MAXM]) {
+  switch (i) {
+    case 0: stage_rhs<G, MD, 0>(s, N, 0, MD, fi, part); break;
+    case 1: stage_rhs<G, MD, 1>(s, N, 1, MD, fi, part); break;
+    case 2: stage_rhs<G, MD, 2>(s, N, 2, MD, fi, part); break;
+    default: stage_rhs<G, MD, 3>(s, N, 3, MD, fi, part); break;
+  }
+  stage_solve<G, MD>(s, N, i, MD, fi, part);
+}
+
 // ------------------------------------------------ cost-ordered work queue
 // Cells are handed out longest-expected-first: the expected substep count of
 // a cell is dt / h with h its carried step (h_cell), binned on a quarter-octave
@@ -2358,6 +2419,8 @@ __device__ void integrate_cell(const MechView& m, const SlotPtrs& s, const Integ
     }
     if (!fixed && __double_as_longlong(left) < __double_as_longlong(h)) h = left;  // both positive
     if (G == 32 && mdim == 4) factor_four(s, h);
+    else if (G == 32 && mdim == 5) factor_columns<5>(s, h);
+    else if (G == 32 && mdim == 6) factor_columns<6>(s, h);
     else factor_small<G>(s, mdim, h);
     // ---- four stages (Algorithm 1); f is evaluated at stages 2 and 3 only
     for (int i = 0; i < 4; ++i) {
@@ -2377,14 +2440,12 @@ __device__ void integrate_cell(const MechView& m, const SlotPtrs& s, const Integ
         fi = s.fr;  // alpha_4j = alpha_3j: same argument as stage 3
       }
       double part[MAXM];
-      if (mdim == 4) {  // the common Krylov dimension: stage and dimension known at compile time
-        switch (i) {
-          case 0: stage_rhs<G, 4, 0>(s, N, 0, 4, fi, part); break;
-          case 1: stage_rhs<G, 4, 1>(s, N, 1, 4, fi, part); break;
-          case 2: stage_rhs<G, 4, 2>(s, N, 2, 4, fi, part); break;
-          default: stage_rhs<G, 4, 3>(s, N, 3, 4, fi, part); break;
-        }
-        stage_solve<G, 4>(s, N, i, 4, fi, part);
+      if (mdim == 4) {  // the common Krylov dimensions: stage and dimension known at compile time
+        stage_of<G, 4>(s, N, i, fi, part);
+      } else if (G == 32 && mdim == 5) {
+        stage_of<G, 5>(s, N, i, fi, part);
+      } else if (G == 32 && mdim == 6) {
+        stage_of<G, 6>(s, N, i, fi, part);
       } else {
         stage_rhs<G, 0, -1>(s, N, i, mdim, fi, part);
         stage_solve<G, 0>(s, N, i, mdim, fi, part);
