@@ -1,0 +1,129 @@
+"""The fixed-point form of the reactions and of the species gather, where it can
+go wrong: the ends of its temperature range, Gibbs factors and Arrhenius
+coefficients that send a cell to the direct form, zero, tiny and negative mass
+fractions, few and many cells to a block.  Bars as in the parity tests: the
+source term and J v within 1e-11 of the row scale of the FP64 oracle; the
+launch shape never changes a bit."""
+
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+P = 101325.0
+
+
+@pytest.fixture(scope="module")
+def rk():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1712_00953_gb300 as rk
+
+    return rk
+
+
+def _mech(name):
+    from synth.fields import WORKLOADS, mechanism_for
+
+    return mechanism_for(WORKLOADS[name])
+
+
+def _check(rk, mech, U, bar=1e-11):
+    from oracle.kinetics import Kinetics
+
+    kin = Kinetics(mech)
+    m = rk.mech_load(mech)
+    V = np.random.default_rng(5).normal(size=U.shape)
+    Ug, Vg = torch.tensor(U, device="cuda"), torch.tensor(V, device="cuda")
+    for got, ref in ((rk.chem_rhs(m, Ug, P), [kin.rhs(u, P) for u in U]),
+                     (rk.chem_jvp(m, Ug, Vg, P), [kin.jvp(u, P, v) for u, v in zip(U, V)])):
+        got, ref = got.cpu().numpy(), np.array(ref)
+        scale = np.max(np.abs(ref), axis=1, keepdims=True)
+        assert np.all(np.isfinite(got))
+        assert np.all(np.abs(got - ref) <= bar * scale)  # (a species alone does not react: both zero)
+
+
+@pytest.mark.parametrize("name", ["small", "flame1d", "batched"])
+def test_temperatures_around_the_range(rk, name):
+    """250 K is the lower end of the fixed-point form; below it the direct form runs."""
+    mech = _mech(name)
+    T = np.array([120.0, 249.0, np.nextafter(250.0, 0), 250.0, np.nextafter(250.0, 251), 256.0, 511.9999, 1024.0, 4000.0])
+    U = np.concatenate([np.random.default_rng(1).dirichlet(np.full(mech.n_species, 0.5), len(T)), T[:, None]], 1)
+    _check(rk, mech, U)
+
+
+@pytest.mark.parametrize("name", ["small", "flame1d", "batched"])
+def test_zero_tiny_and_negative_mass_fractions(rk, name):
+    mech = _mech(name)
+    rng = np.random.default_rng(2)
+    Y = rng.dirichlet(np.full(mech.n_species, 0.5), 8)
+    Y[0, ::2] = 0.0
+    Y[1, 1:] = 0.0
+    Y[2, ::3] = 1e-300
+    Y[3, ::3] = 5e-324
+    Y[4, ::4] = -1e-9
+    Y[5] = 10.0 ** rng.uniform(-150, 0, mech.n_species)
+    Y[6, :] = 0.0
+    Y[6, 3] = 1.0
+    _check(rk, mech, np.concatenate([Y, rng.uniform(400.0, 2500.0, (8, 1))], 1))
+
+
+@pytest.mark.parametrize("name", ["small", "flame1d"])
+def test_large_gibbs_factors_take_the_direct_form(rk, name):
+    """An element-additive shift of the enthalpies cancels from every reaction but
+    carries |g/RT| past 170 in the cold cells."""
+    mech = _mech(name)
+    mech.nasa[:, 8] -= 60000.0 * mech.elem[:, 1]
+    mech.nasa[:, 15] -= 60000.0 * mech.elem[:, 1]
+    T = np.linspace(300.0, 2500.0, 9)
+    U = np.concatenate([np.random.default_rng(3).dirichlet(np.full(mech.n_species, 0.5), len(T)), T[:, None]], 1)
+    _check(rk, mech, U)
+
+
+@pytest.mark.parametrize("change", ["b", "A", "Ea"])
+def test_coefficients_outside_the_fixed_point_range(rk, change):
+    mech = _mech("small")
+    if change == "b":
+        mech.arrh[3, 1] = 20.0
+        mech.arrh[3, 0] *= 1e-60
+    elif change == "A":
+        mech.arrh[3, 0] = 1e-140
+    else:
+        mech.arrh[3, 2] = 2.0e6
+    T = np.linspace(300.0, 2500.0, 7)
+    U = np.concatenate([np.random.default_rng(4).dirichlet(np.full(mech.n_species, 0.5), len(T)), T[:, None]], 1)
+    _check(rk, mech, U)
+
+
+def test_non_finite_states_give_non_finite_rates(rk):
+    mech = _mech("batched")
+    m = rk.mech_load(mech)
+    U = np.concatenate([np.random.default_rng(6).dirichlet(np.full(mech.n_species, 0.5), 4), np.full((4, 1), 900.0)], 1)
+    U[0, 5] = np.nan
+    U[1, -1] = np.nan
+    U[2, 7] = np.inf
+    out = rk.chem_rhs(m, torch.tensor(U, device="cuda"), P).cpu().numpy()
+    assert not np.isfinite(out[:3, -1]).any() and np.isfinite(out[3]).all()
+
+
+@pytest.mark.parametrize("name,precision", [("small", 0), ("flame1d", 0), ("batched", 0), ("batched", 6)])
+def test_cells_per_block_never_change_a_bit(rk, name, precision):
+    """One, eight (256 threads), ten (384) and sixteen cells a block (512 where they
+    fit), more cells than the device holds at once."""
+    mech = _mech(name)
+    m = rk.mech_load(mech)
+    n = 8 * torch.cuda.get_device_properties(0).multi_processor_count + 37
+    rng = np.random.default_rng(7)
+    U = np.concatenate([rng.dirichlet(np.full(mech.n_species, 0.5), n), rng.uniform(900.0, 1500.0, (n, 1))], 1)
+    ref = None
+    for cells in (0, 1, 8, 10, 16):
+        Y = torch.tensor(U, device="cuda")
+        h = torch.zeros(n, dtype=torch.float64, device="cuda")
+        stats = torch.zeros(n, 4, dtype=torch.int32, device="cuda")
+        for _ in range(2):
+            rk.rok4e_integrate(m, Y, 2e-8, 1e-6, 1e-10, 4, h_cell=h, stats=stats,
+                               opts=rk.Opts(cells_per_block=cells, precision=precision))
+        got = (Y, h, stats)
+        ref = ref or got
+        assert all(torch.equal(a, b) for a, b in zip(got, ref)), cells
