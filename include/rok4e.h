@@ -157,10 +157,9 @@ int rk_chem_jvp_cv(const rk_mech* mech, const double* Y, const double* V, const 
 /* Mixed-precision source term (the right-hand side of precision levels 1 and
  * 2): as rk_chem_rhs, with w = nu^T q gathered on the FP32 pipe in
  * double-float (FP32 pairs, ~44-bit significands; the small-integer net
- * coefficients are exact in FP32) and the rate-coefficient exponentials'
- * polynomial tails in FP32 (~1e-13 relative), while the Gibbs factors, 1/Kc, the
- * rates of progress q = m (k prod C - k/Kc prod C) and the assembly of f stay
- * FP64.  Needs |q_j| below the FP32 range (3.4e38 mol/m^3/s); rates below
+ * coefficients are exact in FP32), while the rate coefficients, the Gibbs
+ * factors, 1/Kc, the rates of progress q = m (k prod C - k/Kc prod C) and the
+ * assembly of f stay FP64.  Needs |q_j| below the FP32 range (3.4e38 mol/m^3/s); rates below
  * 1.2e-38 drop out of w. */
 int rk_chem_rhs_mixed(const rk_mech* mech, const double* Y, const double* src, double p,
                       double* dYdt, int64_t ncell, void* stream);
@@ -185,12 +184,13 @@ typedef struct rk_opts {
   int32_t max_attempts;   /* per-cell cap on attempted steps; <= 0: 100000 */
   int32_t lanes_per_cell; /* 0 auto; 8, 16 or 32 lanes of a warp share one cell */
   int32_t cells_per_block;/* 0 auto: as many as shared memory allows, at most
-                             256 threads per block (8 cells of 32 lanes) */
+                             16 cells of 32 lanes (FP64, level 5 and 6 with at
+                             least 8 cells to an SM), else 256 threads per block */
   double h0;              /* first step when h_cell is NULL or holds <= 0; <= 0: dt */
   double fixed_h;         /* > 0: fixed steps of this size, no error control */
   int32_t trace_cap;      /* attempts recorded per cell into trace (0: none) */
   int32_t precision;      /* 0: FP64 throughout (default).  Every level keeps in
-                             FP64 the equilibrium-constant exponentials, 1/Kc,
+                             FP64 every exponential, 1/Kc,
                              the rates of progress (forward minus reverse), the
                              stage solves, the error norm and the state update,
                              and meets the library's bar against the FP64
@@ -199,24 +199,20 @@ typedef struct rk_opts {
                              Jacobian-vector product) gathered in double-float
                              on the FP32 pipe, the first Gram-Schmidt pass of
                              Arnoldi with FP32 inner products (the
-                             reorthogonalisation pass and the norms FP64), the
-                             rate-coefficient exponentials' polynomial tails in
-                             FP32 (~1e-13 relative).
+                             reorthogonalisation pass and the norms FP64).
                              2: as 1 with the Jacobian-vector products in FP32
                              (~1e-5 relative; the Krylov basis tolerates it).
-                             3: FP64 Arnoldi; the rate-coefficient exponentials'
-                             polynomial tails in FP32; the Jacobian-vector
+                             3: FP64 Arnoldi; the Jacobian-vector
                              product's reaction-level core (d(C_a C_b), dq,
                              nu^T dq) in double-float on the FP32 pipe.
                              4: FP64 throughout except w = nu^T q (in the
                              right-hand side and the Jacobian-vector product),
                              which is formed on the tensor cores as in
                              rk_chem_rhs_tc; needs lanes_per_cell 0 or 32.
-                             5: FP64 throughout except the rate-coefficient
-                             exponentials' polynomial tails (FP32): the FP64
-                             kernel's layout and occupancy, three FP64
-                             instructions fewer per reaction and evaluation.
-                             6: as 5 with the Jacobian-vector products in FP32
+                             5: as 0 (it had the rate-coefficient exponentials'
+                             polynomial tails in FP32; on the integer pipes
+                             they cost the same at full precision).
+                             6: as 0 with the Jacobian-vector products in FP32
                              arithmetic on FP32 copies of their caches, which
                              the caching right-hand side writes into the FP64
                              caches' own storage (the FP64 kernel's occupancy;
@@ -500,14 +496,11 @@ int rk_rok4e_adjoint_ex(const rk_mech* mech, const double* checkpoints, const do
 int rk_probe_throughput(int32_t kind, double* ops_per_s);
 
 /* The kernels' own elementary functions on a device array (for testing them
- * against the CUDA math library): which 0: y = exp(x); 1: exp(x) and 2:
- * exp(-x) from the shared-reduction pair; 3, 4, 5: the same three in the
- * mixed-precision form (polynomial's small term in FP32, relative error
- * ~1e-13; 3 is the rate-coefficient exponential of precision levels 1, 2, 3,
- * 5 and 6, while the pair 4, 5 is no longer used by any level, whose
- * equilibrium-constant exponentials stay FP64); 6: y = ln x; 7: y = 1/x.
+ * against the CUDA math library): which 0, 1, 3, 4: y = exp(x); 2, 5:
+ * y = exp(-x) (1 and 2 were a pair with a shared reduction, 3 to 5 a form with
+ * an FP32 polynomial; one function serves all now); 6: y = ln x; 7: y = 1/x.
  * Methods: Tang, ACM TOMS 15(2), 1989 (exp: a 256-entry table of 2^(j/256)
- * and a degree-4 polynomial) and 16(4), 1990 (ln: a 128-entry table and a
+ * and a degree-5 polynomial, in 64-bit integers) and 16(4), 1990 (ln: a 128-entry table and a
  * degree-7 polynomial); 1/x by two Newton steps from an FP32 estimate where
  * x and 1/x are FP32-normal, a division elsewhere.  The paper itself delegates
  * kinetics to Cantera and prints none of these.  x, y: n doubles in device

@@ -138,10 +138,9 @@ class Opts:
         self.trace = trace  # CUDA float64 tensor [ncell, cap] or None
         self.events = events  # (begin, end) torch.cuda.Event pair around the integration kernel
         # rk_opts.precision: 0 FP64; 1 double-float nu^T q, FP32 first
-        # Gram-Schmidt products and rate-coefficient exp tails; 2 as 1 with an
-        # FP32 J v; 3 FP64 Krylov path, double-float J v core, FP32 exp tails;
-        # 4 nu^T q on the tensor cores; 5 FP32 rate-coefficient exp tails only;
-        # 6 as 5 with an FP32 J v on FP32 copies of its caches
+        # Gram-Schmidt products; 2 as 1 with an FP32 J v; 3 FP64 Krylov path,
+        # double-float J v core; 4 nu^T q on the tensor cores; 5 as 0; 6 as 0
+        # with an FP32 J v on FP32 copies of its caches
         self.precision = precision
         self.queue_order, self.blocks_per_sm = queue_order, blocks_per_sm
         self.rho_cell = rho_cell  # CUDA float64 [ncell]: constant-volume cells of these densities
@@ -490,8 +489,8 @@ def simpler_split_step_sharded(m: Mechanism, Uext, dt, D, dx, rtol, atol, krylov
 
 
 def eval_exp(x, which=0, out=None, stream=None):
-    """The kernels' own elementary functions on a CUDA float64 tensor (0: exp(x), 1/2: exp(+-x)
-    pair; 3/4/5: the same in the mixed-precision form; 6: ln x; 7: 1/x)."""
+    """The kernels' own elementary functions on a CUDA float64 tensor (0, 1, 3, 4: exp(x);
+    2, 5: exp(-x); 6: ln x; 7: 1/x)."""
     out = torch.empty_like(x) if out is None else out
     _check(_L().rk_eval_exp(_dptr(x, "x"), _dptr(out, "out", x.numel()), x.numel(), int(which),
                             _stream_ptr(stream)), "rk_eval_exp")

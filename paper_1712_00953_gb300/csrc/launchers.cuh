@@ -32,8 +32,9 @@ extern template int launch_rok4e_wide<512>(const IntegrateLaunch&);
 // FP64 cells one to a warp: an attempt is a chain of dependent instructions that
 // leaves its sub-partition idle a third of the time with two warps on it, so more
 // cells to an SM finish more of them, each with fewer registers (168 with up to
-// twelve warps, 128 with sixteen; 0 and 300 bytes of spills).  Which cells fit is
-// the mechanism's size.  With few cells for each SM the step lasts as long as its
+// twelve warps, 128 with sixteen; 0 and 400 bytes of spills).  How many fit is the
+// mechanism's size: ten at 53 species / 325 reactions (12288 cells, two steps: 177
+// ms with eight, 165 with ten), sixteen at 10 / 24 (20001 cells: 287 and 210 ms).  With few cells for each SM the step lasts as long as its
 // slowest cells, which run fastest on eight warps.
 inline int rok4e_threads(const IntegrateLaunch& a) {
   const IntegrateParams& P = *a.P;
