@@ -21,17 +21,18 @@
 // way cells needing 1 or 200 substeps share one launch without a tail of
 // idle blocks.
 //
-// Arithmetic.  FP64 throughout.  Three restatements differ from a literal
-// transcription of the kinetics while computing the same quantities:
-//  * 1/Kc_j = exp(Delta G_j/RT) (RT/p_ref)^dnu_j is formed as a product of the
-//    per-species factors E_k = exp(g_k/RT) (RT/p_ref) over the products and
-//    1/E_k over the reactants (2 exponentials per species instead of one per
-//    reaction, the pressure factor folded in), falling back to one
-//    exponential per reaction when some |g/RT + ln(RT/p_ref)| > 170 (where a
-//    product of four factors could overflow);
-//  * q_j = m_j k_j (prod C^nu' - prod C^nu''/Kc_j), the second product formed
-//    from the per-species C_k E_k and the reactants' 1/E_k;
-//  * w = nu^T q is a gather over a species-major list (deterministic order).
+// Arithmetic.  FP64 accuracy throughout, on two kinds of pipe: a warp's FP64
+// instruction holds its sub-partition's FP64 unit for 64 cycles, an integer one
+// its pipe for 2 to 4, so what can be formed from 64-bit integers without loss is
+// (fx.cuh), and FP64 instructions are kept for the rest.  Restatements that differ
+// from a literal transcription of the kinetics while computing the same quantities:
+//  * with E_k = exp(g_k/RT) (RT/p_ref) and z_k = C_k E_k, 1/Kc is a product of E
+//    over the products divided by one over the reactants and q_j = m_j kappa_j
+//    (z_ra z_rb - z_pa z_pb), ln kappa = ln k - ln E_ra - ln E_rb: one exponential
+//    per reaction and one per species.  Cells outside its range (reactions_direct)
+//    take 1/Kc from an exponential of its own;
+//  * w = nu^T q is a gather over a species-major list, exact in 128-bit fixed point
+//    for all but the smallest mechanisms.
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -75,10 +76,10 @@ constexpr int MAXM = RK_MAX_KRYLOV;
 // up to 255 registers (one such block fills an SM's register file, which the
 // cells' shared-memory slots limit the SM to anyway).
 constexpr int MAX_BLOCK_THREADS = 256;
-#ifndef RK_WIDE_MIN
-#define RK_WIDE_MIN 8
-#endif
-constexpr int WIDE_MIN_CELLS_PER_SM = RK_WIDE_MIN;
+// Cells for each SM from which the integrator's wider blocks are taken: with eight
+// or fewer they change nothing (1216 cells on 152 SMs: 24.2 ms on eight warps, 24.9
+// on sixteen), with sixteen they gain (2500 cells: 34.8 and 28.1 ms).
+constexpr int WIDE_MIN_CELLS_PER_SM = 8;
 // the explicit integrator fits 128 registers with one warp per cell
 constexpr int POINT_BLOCK_THREADS = 512;
 constexpr int rkdp_threads(int G) { return G == 32 ? 512 : MAX_BLOCK_THREADS; }
@@ -238,6 +239,7 @@ struct MechView {
   const double *W, *invW, *Tmid, *lo, *hi, *lnA, *bexp, *EaR, *eff, *fo, *csr_nu;
   const uint64_t *fA, *fb, *fE;  // fixed-point Arrhenius coefficients (fx.cuh)
   bool fx;                       // every coefficient fits that form
+  bool seg;                      // the gather's list is in shared memory
   const uint32_t* slots;
   const int32_t *meta, *csr_ptr, *csr_j;
   const int32_t* gcsr_j;  // csr_j in global memory
@@ -277,6 +279,7 @@ __host__ __device__ inline MechView make_view(const unsigned char* base, const u
   m.fb = reinterpret_cast<const uint64_t*>(fbase + L.off_fb);
   m.fE = reinterpret_cast<const uint64_t*>(fbase + L.off_fE);
   m.fx = fxseg && L.fx != 0;
+  m.seg = fxseg && L.nr < 8191;
   m.gcsr_j = reinterpret_cast<const int32_t*>(gbase + L.off_csr_j);
   m.bexp = reinterpret_cast<const double*>(gbase + L.off_b);
   m.EaR = reinterpret_cast<const double*>(gbase + L.off_EaR);
@@ -538,7 +541,7 @@ struct CellScalars {
   double TSh, irc;  // T Sh, 1 / (rho cb)
   double Hs, Ds;    // sum (cp_k/R - h_k/RT) w_k / T, sum Y_k d(cp_k/R)/dT / W_k
   double pinv;  // 1 / p (constant pressure) or 1 / rho (constant volume): set by the caller
-  int prec;     // precision level (3: mixed exp in the RHS, double-float J v core): set by the caller
+  int prec;     // precision level (3: double-float J v core, 6: FP32 J v): set by the caller
   // auxiliary-temperature system: sum_k (cp_k/R - 1) F_k / W_k, the T row
   // without its own source, 1 / rho and the velocity
   double B, fT, irho_c, vel[3];
@@ -624,10 +627,10 @@ __device__ inline SlotPtrs slot_ptrs(double* b, const SlotLayout& s) {
   return p;
 }
 
-// w = nu^T q by rows of the species-major list in FP64, into part[0..ns): cells in
-// the direct form, rates that are not finite (their rows alone become so).
+// w = nu^T q by rows of the species-major list in FP64, into part[0..ns), for
+// mechanisms whose gather list does not fit in shared memory.
 template <int G>
-__device__ __noinline__ void gather_rows(const MechView& m, const SlotPtrs& s) {
+__device__ __noinline__ int gather_rows(const MechView& m, const SlotPtrs& s) {
   const Grp<G> g;
   for (int k = g.lane; k < m.ns; k += G) {
     double acc = 0.0;
@@ -635,6 +638,7 @@ __device__ __noinline__ void gather_rows(const MechView& m, const SlotPtrs& s) {
     s.part[k] = acc;
   }
   g.sync();
+  return -1;
 }
 // The gather in 128-bit fixed point (fx.cuh): the rates in s.q go onto one grid
 // below their largest (high words in place, low words in krc's storage), each lane
@@ -709,6 +713,12 @@ __device__ __forceinline__ int gather_listed(const MechView& m, const SlotPtrs& 
   }
   g.sync();
   return -2;
+}
+// (for cells in the direct form, and rates that are not finite: their rows alone
+// become so)
+template <int G>
+__device__ __noinline__ int gather_listed_call(const MechView& m, const SlotPtrs& s) {
+  return gather_listed<G>(m, s);
 }
 // nu^T q of species k after gather_fixed (em >= 0), gather_listed (-2) or gather_rows (-1)
 __device__ __forceinline__ double gathered_row(const MechView& m, const SlotPtrs& s, int k, int em) {
@@ -1296,7 +1306,7 @@ __device__ __forceinline__ void rhs_eval(const MechView& m, const SlotPtrs& s, c
     g.sync();
   } else if (!tc_om) {
     if (zf && !(cache && cs->prec == 3)) em = m.gfix ? gather_fixed<G>(m, s, qe) : gather_listed<G>(m, s);
-    if (em == -1) gather_rows<G>(m, s);
+    if (em == -1) em = m.seg ? gather_listed_call<G>(m, s) : gather_rows<G>(m, s);
   }
   for (int k = g.lane; k < ns; k += G) {
     double om;
@@ -1573,7 +1583,7 @@ __device__ __forceinline__ void jvp_eval(const MechView& m, const SlotPtrs& s, c
     g.sync();
   } else if (!tc_om) {
     if (zf) em = m.gfix ? gather_fixed<G>(m, s, qe) : gather_listed<G>(m, s);
-    if (em == -1) gather_rows<G>(m, s);
+    if (em == -1) em = m.seg ? gather_listed_call<G>(m, s) : gather_rows<G>(m, s);
   }
   double dSh = 0.0, dcb = 0.0;
   for (int k = g.lane; k < ns; k += G) {
