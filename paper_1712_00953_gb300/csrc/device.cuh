@@ -999,7 +999,7 @@ __device__ __forceinline__ void reactions_scaled(const MechView& m, const SlotPt
 
 // Every reaction with 1/Kc from one exponential of its own: the form for cells
 // the scaled one does not hold for (a Gibbs factor past e^170, T outside
-// [250, 16000) K, coefficients outside the fixed-point range, NaN).
+// [150, 16000) K, coefficients outside the fixed-point range, NaN).
 template <int G, bool MIXED>
 __device__ __noinline__ void reactions_direct(const MechView& m, const SlotPtrs& s, double T, double invT, double lnT,
                                               double lnRTp, bool coop_tb, bool cache, CellScalars* cs) {

@@ -222,10 +222,11 @@ RK_FX double from_grid(Wide a, int em, int hb) {
 // The fixed-point Arrhenius form: log2 k = log2 A + b log2 T - (Ea / R) log2 e / T.
 // Coefficients are stored shifted to be non-negative (b + 32 scaled by 2^57, Ea/R
 // log2 e + 2^15 scaled by 2^46), the shifts taken out once per cell.
-// Valid for |b| <= 16, Ea/R log2 e in [-2^15, 2^18 - 2^15), |log2 A| <= 200 and T in
-// [T_LO, T_HI): a rate constant's logarithm and those of two Gibbs factors
-// (each below 246) then stay inside (-2048, 946).
-constexpr double T_LO = 250.0, T_HI = 16000.0;
+// Valid for |b| <= 16, Ea/R log2 e in [-2^13, 130000), |log2 A| <= 150 and T in
+// [T_LO, T_HI): a rate constant's logarithm (between -1242 and 429) and those of two
+// Gibbs factors (each below 246 in magnitude) then stay inside (-1735, 922), which
+// neither wraps nor overflows a double.
+constexpr double T_LO = 150.0, T_HI = 16000.0;
 struct Temp {
   uint64_t lgT, iT, c;  // log2 T 2^59, 2^70 / T, and the shifts' share
 };

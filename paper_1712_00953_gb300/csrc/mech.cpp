@@ -74,8 +74,8 @@ FxArrhenius fx_arrhenius(double A, int order, double b, double EaR) {
   const int64_t lg = (int64_t)e * ((int64_t)1 << 52) + (int64_t)llrint(ldexp(log2(m), 52)) +
                      (int64_t)(order - 1) * RK_FX_LOG2_1EM6;
   const double El = EaR * 1.4426950408889634;
-  f.ok = A < 1e150 && A > 1e-150 && llabs(lg) <= (int64_t)200 << 52 && fabs(b) <= 16.0 && El >= -32768.0 &&
-         El < 229375.0;
+  f.ok = A < 1e150 && A > 1e-150 && llabs(lg) <= (int64_t)150 << 52 && fabs(b) <= 16.0 && El >= -8192.0 &&
+         El < 130000.0;
   if (!f.ok) return f;
   f.A = (uint64_t)lg;
   f.b = (uint64_t)((int64_t)llrint(ldexp(b, 57)) + ((int64_t)32 << 57));
