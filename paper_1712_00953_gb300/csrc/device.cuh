@@ -256,9 +256,11 @@ struct MechView {
   const int32_t *role_ptr, *role;  // species-major reaction slots (r << 2 | role)
 };
 
-// The view of a block that copied the buffer's first `prefix` bytes to base and,
-// the segment after them (fxseg: its fixed-point part too); lnA, b, Ea/R, csr_ptr and csr_nu are read
-// from the whole buffer in global memory, gbase.
+// The view of a block that copied the buffer's first `prefix` bytes to base and
+// after them the segment: all of it (fxseg), or its thermo coefficients alone.  Then
+// fA, fb, fE, gidx and gspec are not in shared memory, m.fx and m.seg say so, and
+// nothing may read them; the rows of the species-major list (csr_ptr, csr_nu,
+// gcsr_j), lnA, b and Ea/R are read from the whole buffer in global memory, gbase.
 __host__ __device__ inline MechView make_view(const unsigned char* base, const unsigned char* gbase,
                                               const MechLayout& L, int64_t prefix, bool fxseg) {
   const unsigned char* fbase = base + prefix - L.off_lo;  // the segment's arrays sit at fbase + their offset
@@ -639,6 +641,18 @@ __device__ __noinline__ int gather_rows(const MechView& m, const SlotPtrs& s) {
   }
   g.sync();
   return -1;
+}
+// The same in FP32 (the J v of precision 6).
+template <int G>
+__device__ __noinline__ void gather_rows_f32(const MechView& m, const float* q, float* part) {
+  const Grp<G> g;
+  for (int k = g.lane; k < m.ns; k += G) {
+    float acc = 0.f;
+    for (int e = m.csr_ptr[k]; e < m.csr_ptr[k + 1]; ++e)
+      acc = fmaf(__double2float_rn(m.csr_nu[e]), q[m.gcsr_j[e]], acc);
+    part[k] = acc;
+  }
+  g.sync();
 }
 // The gather in 128-bit fixed point (fx.cuh): the rates in s.q go onto one grid
 // below their largest (high words in place, low words in krc's storage), each lane
@@ -1883,18 +1897,26 @@ __device__ __forceinline__ void jvp_eval_f32x(const MechView& m, const SlotPtrs&
     fq[j] = dq;
   }
   g.sync();
-  for (int p = g.lane; p < m.gnpp; p += G) {  // d w = nu^T dq, in the fixed-point gather's pieces
-    float acc = 0.f;
-    for (int i = 0; i < m.glen; ++i) acc += fq[m.gidx[((i >> 3) * m.gnpp + p) * 8 + (i & 7)] >> 3];
-    fpart[p] = acc;
+  if (m.seg) {  // d w = nu^T dq, in the fixed-point gather's pieces
+    for (int p = g.lane; p < m.gnpp; p += G) {
+      float acc = 0.f;
+      for (int i = 0; i < m.glen; ++i) acc += fq[m.gidx[((i >> 3) * m.gnpp + p) * 8 + (i & 7)] >> 3];
+      fpart[p] = acc;
+    }
+    g.sync();
+  } else {
+    gather_rows_f32<G>(m, fq, fpart);
   }
-  g.sync();
   float dSh = 0.f, dcb = 0.f;
   for (int k = g.lane; k < ns; k += G) {
     float dom = 0.f;
-    int p = m.gspec[2 * k];
-    for (; p < m.gspec[2 * k + 1]; ++p) dom += fpart[p];
-    for (; p < m.gspec[2 * k + 2]; ++p) dom -= fpart[p];
+    if (m.seg) {
+      int p = m.gspec[2 * k];
+      for (; p < m.gspec[2 * k + 1]; ++p) dom += fpart[p];
+      for (; p < m.gspec[2 * k + 2]; ++p) dom -= fpart[p];
+    } else {
+      dom = fpart[k];
+    }
     out[k] = (double)(s.xEinv[k] * fmaf(-s.xom[k], drr, dom));  // xEinv: W_k / rho
     dSh = fmaf(s.xg[k], dom, dSh);
     dcb = fmaf(s.xcp[k], f(v[k]), dcb);
