@@ -111,10 +111,10 @@ __device__ __forceinline__ bool below(double a, double b) {
 // 1/x by Newton's iteration for the reciprocal, r <- r + r (1 - x r), from
 // an FP32 estimate: two steps square the estimate's relative error twice
 // ((2e-7)^4), leaving the last rounding.  Four FP64 operations instead of a
-// full-precision division; for normal x inside the FP32 range (the
-// temperature and the mixture sums of a cell).  The conversions to FP32
-// (truncated) and back are integer moves: a conversion instruction takes the FP64
-// unit as long as an FP64 operation.
+// full-precision division; only for x whose reciprocal and itself are FP32-normal
+// (|x| in [2^-125, 2^125): anything else, 0 and NaN too, wraps to a finite wrong
+// value).  The conversions to FP32 (truncated) and back are integer moves: a
+// conversion instruction takes the FP64 unit as long as an FP64 operation.
 __device__ __forceinline__ double rcp_newton(double x) {
   const int hi = __double2hiint(x), sign = hi & (int)0x80000000;
   const float f = __int_as_float((((hi & 0x7fffffff) - (896 << 20)) << 3) | (int)((unsigned)__double2loint(x) >> 29));
@@ -134,6 +134,20 @@ __device__ __forceinline__ double rcp_newton(double x) {
 __device__ __forceinline__ double rcp_any(double x) {
   const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
   return ex - 898u < 250u ? rcp_newton(x) : 1.0 / x;
+}
+
+// 1/x for the temperature and the mixture sums of a cell.  What is no state any more
+// stays visible: 0 (a cell whose mass fractions are all zero, T = 0), NaN, infinities
+// and |x| below 2^-128 give NaN, |x| from 2^128 zero, through rounding conversions;
+// one integer test on the main path.
+static __device__ __noinline__ double rcp_beyond(double x) {
+  double r = (double)__frcp_rn(__double2float_rn(x));
+  r = fma(r, fma(-x, r, 1.0), r);
+  return fma(r, fma(-x, r, 1.0), r);
+}
+__device__ __forceinline__ double rcp_state(double x) {
+  const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
+  return ex - 898u < 250u ? rcp_newton(x) : rcp_beyond(x);
 }
 
 // 1/sqrt(x) for positive, finite, normal x: FP32 estimate of the significand with
@@ -1092,7 +1106,7 @@ __device__ __forceinline__ void rhs_eval(const MechView& m, const SlotPtrs& s, c
   const Grp<G> g;
   const int ns = m.ns;
   const double T = uu[ns];
-  const double invT = rcp_newton(T);
+  const double invT = rcp_state(T);
   // log2 T in fixed point gives ln T (0.6 ulp) and the rate constants' T^b
   const bool t_fx = below(T, fx::T_HI) && !below(T, fx::T_LO);
   uint64_t lgT = 0;
@@ -1162,7 +1176,7 @@ __device__ __forceinline__ void rhs_eval(const MechView& m, const SlotPtrs& s, c
   // the constant-volume arithmetic with unit density
   const bool aux = m.nx > 0;
   const bool cv = __double2hiint(p) < 0 || aux;  // p < 0 (never -0 or NaN)
-  const double invS = rcp_newton(S);
+  const double invS = rcp_state(S);
   // rho = p / (R T S), 1/rho = R T S / p, with 1/p (or 1/rho) from the caller
   const double rho = aux ? 1.0 : (cv ? -p : p * invT * invS * INV_R);
   const double invrho = aux ? 1.0 : (cv ? cs->pinv : R_GAS * T * S * cs->pinv);
@@ -1393,7 +1407,7 @@ __device__ __forceinline__ void rhs_eval(const MechView& m, const SlotPtrs& s, c
     Sh = t2[0];
     cb = t2[1];
   }
-  const double invcb = rcp_newton(cb);
+  const double invcb = rcp_state(cb);
   double fT = 0.0;
   if (aux) {
     // Eq. aux_t_equation with specific internal energies e_k = (u_k/RT) R T / W_k

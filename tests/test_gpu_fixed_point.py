@@ -130,3 +130,34 @@ def test_cells_per_block_never_change_a_bit(rk, name, precision):
         got = (Y, h, stats)
         ref = ref or got
         assert all(torch.equal(a, b) for a, b in zip(got, ref)), cells
+
+
+def test_cells_that_are_no_state_are_not_finite_and_fail(rk):
+    """All mass fractions zero or tiny (an unset cell; sum Y/W at or below the smallest
+    number whose reciprocal the right-hand side forms), a zero temperature: the source term
+    is not finite, the integrators say so and touch no other cell."""
+    for name in ("small", "batched"):
+        mech = _mech(name)
+        m = rk.mech_load(mech)
+        ns = mech.n_species
+        U = np.concatenate([np.random.default_rng(11).dirichlet(np.full(ns, 0.5), 6), np.full((6, 1), 1100.0)], 1)
+        U[0, :-1] = 0.0
+        U[1, :-1] = 1e-60
+        U[2, -1] = 0.0
+        U[3, :-1] = -0.0
+        U[4, :-1] = 5e-324
+        Ug = torch.tensor(U, device="cuda")
+        out = rk.chem_rhs(m, Ug, P).cpu().numpy()
+        assert not np.isfinite(out[:5, -1]).any() and np.isfinite(out[5]).all()
+        rho = torch.full((6,), 0.2, dtype=torch.float64, device="cuda")
+        out = rk.chem_rhs_cv(m, Ug, rho).cpu().numpy()  # (fixed density: the mixture's heat capacity is what is zero)
+        assert not np.isfinite(out[:5, -1]).any() and np.isfinite(out[5]).all()
+        for run in (lambda y, st: rk.rok4e_integrate(m, y, 1e-8, 1e-6, 1e-10, 4, stats=st),
+                    lambda y, st: rk.rkdp_integrate(m, y, 1e-8, 1e-6, 1e-10, stats=st)):
+            Y, stats = Ug.clone(), torch.zeros(6, 4, dtype=torch.int32, device="cuda")
+            run(Y, stats)
+            alone, one = Ug[5:].clone(), torch.zeros(1, 4, dtype=torch.int32, device="cuda")
+            run(alone, one)
+            st = stats.cpu().numpy()
+            assert (st[:5, 3] != 0).all() and st[5, 3] == 0
+            assert torch.equal(Y[5:], alone)
