@@ -31,8 +31,8 @@
 //    (z_ra z_rb - z_pa z_pb), ln kappa = ln k - ln E_ra - ln E_rb: one exponential
 //    per reaction and one per species.  Cells outside its range (reactions_direct)
 //    take 1/Kc from an exponential of its own;
-//  * w = nu^T q is a gather over a species-major list, exact in 128-bit fixed point
-//    for all but the smallest mechanisms.
+//  * w = nu^T q is a gather over a species-major list, for all but the smallest
+//    mechanisms in 128-bit fixed point wherever every row keeps FP64's bits there.
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -261,7 +261,7 @@ struct MechView {
   int npiece;
   const uint16_t* gidx;  // fixed-point gather: [glen][gnpp] reactions, pieces of each species
   const int32_t* gspec;
-  int glen, gnpp, ghb;
+  int glen, gnpp, ghb, gdeep;
   bool gfix;  // gather in fixed point
   const float *Wf, *invWf, *bf, *EaRf, *efff, *csr_nuf;  // FP32 copies
   const int32_t* perm;  // input index of each packed reaction
@@ -314,6 +314,7 @@ __host__ __device__ inline MechView make_view(const unsigned char* base, const u
   m.glen = L.glen;
   m.gnpp = L.gnpp;
   m.ghb = L.ghb;
+  m.gdeep = 73 - 2 * L.ghb;
   m.gfix = L.gfix != 0;
   m.Wf = reinterpret_cast<const float*>(base + L.off_Wf);
   m.invWf = reinterpret_cast<const float*>(base + L.off_invWf);
@@ -485,6 +486,12 @@ struct Grp {
     for (int o = G / 2; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(mask, v, o, G));
     return v;
   }
+  __device__ __forceinline__ unsigned umin(unsigned v) const {
+    if constexpr (G == 32) return __reduce_min_sync(0xffffffffu, v);
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) v = ::min(v, __shfl_xor_sync(mask, v, o, G));
+    return v;
+  }
   __device__ __forceinline__ int imax(int v) const {
     if constexpr (G == 32) return __reduce_max_sync(0xffffffffu, v);
 #pragma unroll
@@ -643,10 +650,13 @@ __device__ inline SlotPtrs slot_ptrs(double* b, const SlotLayout& s) {
   return p;
 }
 
+// Where a gather left w = nu^T q: nowhere yet; pieces, or a species' sum each, in
+// part; a species' sum each in the rates' place.
+enum Gathered { NOT_GATHERED, PIECES_IN_PART, ROWS_IN_PART, ROWS_IN_Q };
 // w = nu^T q by rows of the species-major list in FP64, into part[0..ns), for
 // mechanisms whose gather list does not fit in shared memory.
 template <int G>
-__device__ __noinline__ int gather_rows(const MechView& m, const SlotPtrs& s) {
+__device__ __noinline__ Gathered gather_rows(const MechView& m, const SlotPtrs& s) {
   const Grp<G> g;
   for (int k = g.lane; k < m.ns; k += G) {
     double acc = 0.0;
@@ -654,7 +664,7 @@ __device__ __noinline__ int gather_rows(const MechView& m, const SlotPtrs& s) {
     s.part[k] = acc;
   }
   g.sync();
-  return -1;
+  return ROWS_IN_PART;
 }
 // The same in FP32 (the J v of precision 6).
 template <int G>
@@ -668,20 +678,43 @@ __device__ __noinline__ void gather_rows_f32(const MechView& m, const float* q, 
   }
   g.sync();
 }
+// High words without signs of a lane's rates: the largest, and the smallest that is
+// not zero, less one (a zero wraps to the top).
+struct RateRange {
+  uint32_t top = 0u, low = 0xffffffffu;
+  __device__ __forceinline__ void take(double q) {
+    const uint32_t w = (uint32_t)__double2hiint(q) & 0x7fffffffu;
+    top = ::max(top, w);
+    low = ::min(low, w - 1u);
+  }
+};
+constexpr int DEPTH_FP64 = 80;
 // The gather in 128-bit fixed point (fx.cuh): the rates in s.q go onto one grid
 // below their largest (high words in place, low words in krc's storage), each lane
 // adds up whole pieces with integer adds, and a species adds and subtracts its
-// pieces and rounds once.  Exact sums, whatever the order, so the pieces' entries
-// are ordered to meet no shared-memory bank conflicts and no coefficient is
+// pieces and rounds once.  The sums do not depend on their order, so the pieces'
+// entries are ordered to meet no shared-memory bank conflicts and no coefficient is
 // loaded or multiplied.  An FP64 term took 64 cycles of the FP64 unit, here ~20 of
-// the integer pipes and ~5 shared-memory wavefronts.  Returns the largest biased
-// exponent, or -1 with nothing done when a rate is infinite or NaN.
-// em: the largest (high word >> 20) & 0x7ff over the lane's rates.
+// the integer pipes and ~5 shared-memory wavefronts.
+// The grid ends 2^-(126 - ghb) below the cell's largest rate, and a row of up to
+// 2^(ghb - 1) terms may lose a unit with each: a row whose sum is 2^(53 + ghb) units or
+// more, 2^-gdeep of the largest, keeps it to 2^-54, half a rounding of FP64.  Where some
+// rate that is not zero lies below that and a row's sum too (a cold mixture with few
+// species present: the first radicals' rates are tens of orders of magnitude below the
+// others'), the caller forms the rates again and sums them in FP64.  Where the rates
+// reach down 2^-80 that is likely (53 species, 300 to 2000 K: 5 % of the cells at 2^-60
+// to 2^-70, 71 % at 2^-80 to 2^-90) and FP64 is taken at once: its gather costs a
+// right-hand side a tenth more, forming the rates again two thirds.
+// NOT_GATHERED, with nothing done, for these and when a rate is infinite or NaN;
+// *again: a row out of reach.
 template <int G>
-__device__ __forceinline__ int gather_fixed(const MechView& m, const SlotPtrs& s, int em) {
+__device__ __forceinline__ Gathered gather_fixed(const MechView& m, const SlotPtrs& s, const RateRange& lane_range,
+                                                 bool* again) {
   const Grp<G> g;
-  em = g.imax(em);
-  if (em == 0x7ff) return -1;
+  const int em = g.imax((int)lane_range.top) >> 20;
+  const uint32_t least = g.umin(lane_range.low);
+  const int depth = least == 0xffffffffu ? 0 : em - (int)((least + 1u) >> 20);
+  if (em == 0x7ff || depth > DEPTH_FP64) return NOT_GATHERED;
   uint64_t* qh = reinterpret_cast<uint64_t*>(s.q);
   uint64_t* ql = reinterpret_cast<uint64_t*>(s.krc);
   constexpr int U = 4;
@@ -721,12 +754,26 @@ __device__ __forceinline__ int gather_fixed(const MechView& m, const SlotPtrs& s
     part[m.gnpp + p] = a.lo;
   }
   g.sync();
-  return em;
+  bool out = false;
+  for (int k = g.lane; k < m.ns; k += G) {
+    const int p0 = m.gspec[2 * k], p1 = m.gspec[2 * k + 1], p2 = m.gspec[2 * k + 2];
+    int p = p0;
+    fx::Wide a = {0ull, 0ull};
+#pragma unroll 2
+    for (; p < p1; ++p) fx::add(a, part[p], part[m.gnpp + p]);
+#pragma unroll 2
+    for (; p < p2; ++p) fx::sub(a, part[p], part[m.gnpp + p]);
+    const double r = fx::from_grid(a, em, m.ghb);
+    s.q[k] = r;
+    out |= p0 != p2 && ((__double2hiint(r) >> 20) & 0x7ff) + m.gdeep < em;
+  }
+  *again = depth > m.gdeep && g.any(out);
+  return ROWS_IN_Q;
 }
 // The same pieces in FP64, for mechanisms of few entries (gfix false), where the
 // conversions to the grid and back would cost more than the additions they save.
 template <int G>
-__device__ __forceinline__ int gather_listed(const MechView& m, const SlotPtrs& s) {
+__device__ __forceinline__ Gathered gather_listed(const MechView& m, const SlotPtrs& s) {
   const Grp<G> g;
   if (g.lane == 0) s.q[m.nr] = 0.0;
   g.sync();
@@ -740,34 +787,27 @@ __device__ __forceinline__ int gather_listed(const MechView& m, const SlotPtrs& 
     s.part[p] = a;
   }
   g.sync();
-  return -2;
+  return PIECES_IN_PART;
 }
 // (for cells in the direct form, and rates that are not finite: their rows alone
 // become so)
 template <int G>
-__device__ __noinline__ int gather_listed_call(const MechView& m, const SlotPtrs& s) {
+__device__ __noinline__ Gathered gather_listed_call(const MechView& m, const SlotPtrs& s) {
   return gather_listed<G>(m, s);
 }
-// nu^T q of species k after gather_fixed (em >= 0), gather_listed (-2) or gather_rows (-1)
-__device__ __forceinline__ double gathered_row(const MechView& m, const SlotPtrs& s, int k, int em) {
-  if (em == -1) return s.part[k];
+// nu^T q of species k after gather_fixed, gather_listed or gather_rows
+__device__ __forceinline__ double gathered_row(const MechView& m, const SlotPtrs& s, int k,
+                                               Gathered how) {
+  if (how == ROWS_IN_Q) return s.q[k];
+  if (how == ROWS_IN_PART) return s.part[k];
   const int p1 = m.gspec[2 * k + 1], p2 = m.gspec[2 * k + 2];
   int p = m.gspec[2 * k];
-  if (em < 0) {
-    double a = 0.0, b = 0.0;
-    if (p < p1) a = s.part[p++];
-    for (; p < p1; ++p) a += s.part[p];
-    if (p < p2) b = s.part[p++];
-    for (; p < p2; ++p) b += s.part[p];
-    return a - b;
-  }
-  const uint64_t* part = reinterpret_cast<const uint64_t*>(s.part);
-  fx::Wide a = {0ull, 0ull};
-#pragma unroll 2
-  for (; p < p1; ++p) fx::add(a, part[p], part[m.gnpp + p]);
-#pragma unroll 2
-  for (; p < p2; ++p) fx::sub(a, part[p], part[m.gnpp + p]);
-  return fx::from_grid(a, em, m.ghb);
+  double a = 0.0, b = 0.0;
+  if (p < p1) a = s.part[p++];
+  for (; p < p1; ++p) a += s.part[p];
+  if (p < p2) b = s.part[p++];
+  for (; p < p2; ++p) b += s.part[p];
+  return a - b;
 }
 
 // The gather in double-float (FP32 pairs, ~44-bit significands, on the FP32
@@ -1004,7 +1044,7 @@ __device__ __forceinline__ void cache_scaled(const MechView& m, const SlotPtrs& 
 template <int G, bool MIXED, bool PRESSURE>
 __device__ __forceinline__ void reactions_scaled(const MechView& m, const SlotPtrs& s, const fx::Temp& ft, double T,
                                                  double invT, bool coop_tb, bool cache, CellScalars* cs, int j0,
-                                                 int lane, int* qe) {
+                                                 int lane, RateRange* range) {
   const int j = min(j0 + lane, m.nr - 1);
   const uint32_t sl = m.slots[j];
   const int meta = m.meta[j], kind = PRESSURE ? meta & 3 : 0;
@@ -1017,7 +1057,7 @@ __device__ __forceinline__ void reactions_scaled(const MechView& m, const SlotPt
     Dm = __dmul_rn(Dm, mult);
   }
   const double q = fx::mul_sig(r.ks, r.kn, Dm);
-  *qe = max(*qe, (__double2hiint(q) >> 20) & 0x7ff);
+  range->take(q);
   if (j0 + lane < m.nr) {
     if (MIXED) reinterpret_cast<df2*>(s.q)[j] = df_from(q);  // double-float copy for the gather
     else s.q[j] = q;
@@ -1025,6 +1065,19 @@ __device__ __forceinline__ void reactions_scaled(const MechView& m, const SlotPt
   }
 }
 
+// The rates again (their caches are kept) and their rows in FP64, for cells with a row
+// out of the grid's reach.
+template <int G>
+__device__ __noinline__ Gathered rates_listed_call(const MechView& m, const SlotPtrs& s, uint64_t lgT, double T,
+                                                   double invT, bool coop_tb) {
+  const Grp<G> g;
+  const fx::Temp ft = fx::temperature(lgT, fx::recip_fixed70(T, invT));
+  RateRange range;
+  for (int j0 = 0; j0 < m.nr; j0 += G)
+    reactions_scaled<G, false, true>(m, s, ft, T, invT, coop_tb, false, nullptr, j0, g.lane, &range);
+  g.sync();
+  return gather_listed<G>(m, s);
+}
 // Every reaction with 1/Kc from one exponential of its own: the form for cells
 // the scaled one does not hold for (a Gibbs factor past e^170, T outside
 // [150, 16000) K, coefficients outside the fixed-point range, NaN).
@@ -1308,13 +1361,14 @@ __device__ __forceinline__ void rhs_eval(const MechView& m, const SlotPtrs& s, c
     g.sync();
   }
   // reactions: rate coefficients and rates of progress
-  int qe = 0;  // largest exponent of the lane's rates
+  RateRange range;
   if (zf) {
     const fx::Temp ft = fx::temperature(lgT, fx::recip_fixed70(T, invT));
     int j0 = 0;
-    for (; j0 < m.ntb; j0 += G) reactions_scaled<G, MIXED, true>(m, s, ft, T, invT, coop_tb, cache, cs, j0, g.lane, &qe);
+    for (; j0 < m.ntb; j0 += G)
+      reactions_scaled<G, MIXED, true>(m, s, ft, T, invT, coop_tb, cache, cs, j0, g.lane, &range);
     for (; j0 < m.nr; j0 += G)
-      reactions_scaled<G, MIXED, false>(m, s, ft, T, invT, coop_tb, cache, cs, j0, g.lane, &qe);
+      reactions_scaled<G, MIXED, false>(m, s, ft, T, invT, coop_tb, cache, cs, j0, g.lane, &range);
   } else {
     reactions_direct<G, MIXED>(m, s, T, invT, lnT, lnRTp, coop_tb, cache, cs);
   }
@@ -1327,14 +1381,17 @@ __device__ __forceinline__ void rhs_eval(const MechView& m, const SlotPtrs& s, c
   bool tc_om = false;  // w already in part[0..ns) from the tensor cores
   if constexpr (TC) tc_om = gather_tc<G>(m, s, s.q, s.part);
   // in fixed point, except where krc's storage is taken (by the caches of the
-  // direct form and of precision 3) or a rate is not finite
-  int em = -1;
+  // direct form and of precision 3), a rate is not finite or a row is out of reach
+  Gathered how = ROWS_IN_PART;
   if (MIXED) {
     gather_pieces_df<G>(m, g.lane, reinterpret_cast<const df2*>(s.q), reinterpret_cast<df2*>(s.part));
     g.sync();
   } else if (!tc_om) {
-    if (zf && !(cache && cs->prec == 3)) em = m.gfix ? gather_fixed<G>(m, s, qe) : gather_listed<G>(m, s);
-    if (em == -1) em = m.seg ? gather_listed_call<G>(m, s) : gather_rows<G>(m, s);
+    bool again = false;
+    how = NOT_GATHERED;
+    if (zf && !(cache && cs->prec == 3)) how = m.gfix ? gather_fixed<G>(m, s, range, &again) : gather_listed<G>(m, s);
+    if (again) how = rates_listed_call<G>(m, s, lgT, T, invT, coop_tb);
+    if (how == NOT_GATHERED) how = m.seg ? gather_listed_call<G>(m, s) : gather_rows<G>(m, s);
   }
   for (int k = g.lane; k < ns; k += G) {
     double om;
@@ -1342,7 +1399,7 @@ __device__ __forceinline__ void rhs_eval(const MechView& m, const SlotPtrs& s, c
       om = piece_sum_df(m, reinterpret_cast<const df2*>(s.part), k);
       if (cache) s.fom[k] = __double2float_rn(om);
     } else {
-      om = gathered_row(m, s, k, em);
+      om = gathered_row(m, s, k, how);
     }
     if (cache) s.om[k] = om;
     const double r = __dmul_rn(__dmul_rn(m.W[k], om), invrho);
@@ -1498,7 +1555,7 @@ __device__ __forceinline__ double third_body_rate(const MechView& m, const doubl
 // j0 + lane (as reactions_scaled): six FP64 instructions.
 template <int G, bool PRESSURE>
 __device__ __forceinline__ void jvp_scaled(const MechView& m, const SlotPtrs& s, double vTT, bool coop_tb,
-                                           const double (&mp)[MAXM], int j0, int lane, int* qe) {
+                                           const double (&mp)[MAXM], int j0, int lane, RateRange* range) {
   const int j = min(j0 + lane, m.nr - 1);
   const uint32_t sl = m.slots[j];
   const int ra = sl & 255, rb = (sl >> 8) & 255, pa = (sl >> 16) & 255, pb = sl >> 24;
@@ -1517,10 +1574,20 @@ __device__ __forceinline__ void jvp_scaled(const MechView& m, const SlotPtrs& s,
     const double dM = third_body_rate<G>(m, s.arg, slot, coop_tb, mp);
     dq = (meta & 3) == 1 ? t[0] * dq + dM * (kap * D) : dq + t[1] * dM * D;
   }
-  *qe = max(*qe, (__double2hiint(dq) >> 20) & 0x7ff);
+  range->take(dq);
   if (j0 + lane < m.nr) s.q[j] = dq;
 }
 
+// The same again and their rows in FP64 (as rates_listed_call).
+template <int G>
+__device__ __noinline__ Gathered products_listed_call(const MechView& m, const SlotPtrs& s, double vTT, bool coop_tb,
+                                                      const double (&mp)[MAXM]) {
+  const Grp<G> g;
+  RateRange range;
+  for (int j0 = 0; j0 < m.nr; j0 += G) jvp_scaled<G, true>(m, s, vTT, coop_tb, mp, j0, g.lane, &range);
+  g.sync();
+  return gather_listed<G>(m, s);
+}
 // The reaction rates' derivatives from k and k/Kc (caches not in the scaled form).
 template <int G, bool DFG>
 __device__ __forceinline__ void jvp_reactions(const MechView& m, const SlotPtrs& s, double vTT, bool coop_tb,
@@ -1572,7 +1639,6 @@ __device__ __forceinline__ void jvp_eval(const MechView& m, const SlotPtrs& s, c
   const double drr = cs.cv ? 0.0 : -fma(a, cs.invS, vTT);  // d rho / rho (0 at fixed volume)
   const bool coop_tb = m.ntb > 0 && m.ntb <= MAXM;
   const bool zf = !DFG && cs.zf;
-  int qe = 0;  // largest exponent of the lane's dq
   double mp[MAXM];
 #pragma unroll
   for (int t = 0; t < MAXM; ++t) mp[t] = 0.0;
@@ -1593,10 +1659,11 @@ __device__ __forceinline__ void jvp_eval(const MechView& m, const SlotPtrs& s, c
   }
   if (coop_tb) sum_first<G>(g, mp, m.ntb);  // d[M]_t, identical on every lane
   g.sync();
+  RateRange range;
   if (zf) {
     int j0 = 0;
-    for (; j0 < m.ntb; j0 += G) jvp_scaled<G, true>(m, s, vTT, coop_tb, mp, j0, g.lane, &qe);
-    for (; j0 < m.nr; j0 += G) jvp_scaled<G, false>(m, s, vTT, coop_tb, mp, j0, g.lane, &qe);
+    for (; j0 < m.ntb; j0 += G) jvp_scaled<G, true>(m, s, vTT, coop_tb, mp, j0, g.lane, &range);
+    for (; j0 < m.nr; j0 += G) jvp_scaled<G, false>(m, s, vTT, coop_tb, mp, j0, g.lane, &range);
   } else if constexpr (DFG) {
     jvp_reactions<G, true>(m, s, vTT, coop_tb, mp);
   } else {
@@ -1605,18 +1672,21 @@ __device__ __forceinline__ void jvp_eval(const MechView& m, const SlotPtrs& s, c
   g.sync();
   bool tc_om = false;  // d w already in part[0..ns) from the tensor cores
   if constexpr (TC) tc_om = gather_tc<G>(m, s, s.q, s.part);
-  int em = -1;
+  Gathered how = ROWS_IN_PART;
   if (DFG) {
     gather_pieces_df<G>(m, g.lane, reinterpret_cast<const df2*>(s.q), reinterpret_cast<df2*>(s.part));
     g.sync();
   } else if (!tc_om) {
-    if (zf) em = m.gfix ? gather_fixed<G>(m, s, qe) : gather_listed<G>(m, s);
-    if (em == -1) em = m.seg ? gather_listed_call<G>(m, s) : gather_rows<G>(m, s);
+    bool again = false;
+    how = NOT_GATHERED;
+    if (zf) how = m.gfix ? gather_fixed<G>(m, s, range, &again) : gather_listed<G>(m, s);
+    if (again) how = products_listed_call<G>(m, s, vTT, coop_tb, mp);
+    if (how == NOT_GATHERED) how = m.seg ? gather_listed_call<G>(m, s) : gather_rows<G>(m, s);
   }
   double dSh = 0.0, dcb = 0.0;
   for (int k = g.lane; k < ns; k += G) {
     const double dom = DFG ? piece_sum_df(m, reinterpret_cast<const df2*>(s.part), k)
-                           : gathered_row(m, s, k, em);
+                           : gathered_row(m, s, k, how);
     out[k] = m.W[k] * cs.invrho * fma(-s.om[k], drr, dom);
     dSh = fma(s.hRT[k], dom, dSh);
     dcb = fma(s.cp[k], v[k], dcb);

@@ -169,9 +169,11 @@ RK_FX double mul_sig(uint64_t m, int n, double D) {
 
 // ---- sums in 128-bit fixed point.  A set of doubles with largest biased
 // exponent em is put on one grid of 2^(hb + em - 1149), hb bits of headroom for
-// the sums: each value keeps every bit above 2^-(126 - hb) of the largest, so sums
-// of them are exact in any order (FP64's own 53 bits survive for values down to
-// 2^-(73 - hb) of the largest) and cost integer adds.
+// the sums: each value keeps the bits above 2^-(126 - hb) of the largest (all of its
+// 53 down to 2^-(73 - hb) of the largest, fewer below; what is cut is cut downwards,
+// at most one unit of the grid), and sums of them are exact in any order and cost
+// integer adds.  A sum of values that all lie far below the largest is the caller's to
+// form otherwise.
 struct Wide {
   uint64_t hi, lo;  // two's complement
 };

@@ -247,7 +247,7 @@ bool pack_mechanism(const void* vdesc, HostMech* out, std::string* err) {
   // point, in batches of eight entries.
   int entries = 0;
   for (auto& row : signed_rows) entries += (int)row.size();
-  const bool gfix = entries >= GFIX_MIN_ENTRIES && nr < 8191;
+  const bool gfix = entries >= GFIX_MIN_ENTRIES && nr < 8191 && nr >= ns;  // (the sums take the rates' place)
   const int step = gfix ? 8 : 1;
   int glen = 1;
   {

@@ -161,3 +161,54 @@ def test_cells_that_are_no_state_are_not_finite_and_fail(rk):
             st = stats.cpu().numpy()
             assert (st[:5, 3] != 0).all() and st[5, 3] == 0
             assert torch.equal(Y[5:], alone)
+
+
+def _terms(kin, u, v):
+    """Each entry's sum of the magnitudes of its terms: of the source term's species rows
+    and of the Jacobian-vector product's (elementary reactions only for the latter)."""
+    st = kin.state(u, P)
+    nu, W, ns = np.abs(kin.nu), kin.W, kin.ns
+    f, b = st["m"] * st["k"] * st["Pf"], st["m"] * st["kr"] * st["Pb"]
+    rhs = W / st["rho"] * (nu.T @ (f + b))
+    drr = np.sum(np.abs(v[:ns]) / W) / st["S"] + abs(v[ns]) / st["T"]
+    dC = st["rho"] / W * np.abs(v[:ns]) + st["C"] * drr
+
+    def dprod(n):  # sum over factors of |dC| times the others
+        out = np.zeros(len(n))
+        for j, row in enumerate(n):
+            ks = [k for k in np.flatnonzero(row) for _ in range(int(row[k]))]
+            for i, k in enumerate(ks):
+                out[j] += dC[k] * np.prod([st["C"][q] for q in ks[:i] + ks[i + 1:]])
+        return out
+
+    dT = np.abs(st["dlnk"]) * (f + b) + np.abs(st["dlnKc"]) * b
+    dq = st["m"] * (st["k"] * dprod(kin.nu_f) + st["kr"] * dprod(kin.nu_r)) + dT * abs(v[ns])
+    return rhs, W / st["rho"] * (nu.T @ (dq + drr * (f + b)))
+
+
+@pytest.mark.parametrize("name", ["flame1d", "batched", "adjoint"])
+@pytest.mark.parametrize("T", [200.0, 300.0, 600.0])
+def test_slow_rows_of_unburnt_mixtures_entry_by_entry(rk, name, T):
+    """Six species present, the others zero: the rows of the first radicals lie tens of
+    orders of magnitude below the fastest.  Every entry within 1e-12 of its own terms'
+    magnitudes: exponents of at most ~300 in all with about ten roundings of 2^-53 of that on
+    either side (3.4e-13), and the sums' own."""
+    from oracle.kinetics import Kinetics
+
+    mech = _mech(name)
+    kin = Kinetics(mech)
+    m = rk.mech_load(mech)
+    rng = np.random.default_rng(12)
+    U = np.zeros((24, mech.n_species + 1))
+    for u in U:
+        u[rng.permutation(mech.n_species)[:6]] = rng.dirichlet(np.full(6, 0.5))
+    U[:, -1] = T
+    V = rng.normal(size=U.shape) * (U != 0)  # along what is there
+    Ug = torch.tensor(U, device="cuda")
+    f = rk.chem_rhs(m, Ug, P).cpu().numpy()
+    jv = rk.chem_jvp(m, Ug, torch.tensor(V, device="cuda"), P).cpu().numpy()
+    for c, (u, v) in enumerate(zip(U, V)):
+        sf, sj = _terms(kin, u, v)
+        assert np.all(np.abs(f[c, :-1] - kin.rhs(u, P)[:-1]) <= 1e-12 * sf)
+        if not (mech.kind > 0).any():
+            assert np.all(np.abs(jv[c, :-1] - kin.jvp(u, P, v)[:-1]) <= 1e-12 * sj)
