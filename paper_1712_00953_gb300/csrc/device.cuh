@@ -705,7 +705,8 @@ constexpr int DEPTH_FP64 = 80;
 // reach down 2^-80 that is likely (53 species, 300 to 2000 K: 5 % of the cells at 2^-60
 // to 2^-70, 71 % at 2^-80 to 2^-90) and FP64 is taken at once: its gather costs a
 // right-hand side a tenth more, forming the rates again two thirds.
-// NOT_GATHERED, with nothing done, for these and when a rate is infinite or NaN;
+// NOT_GATHERED, with nothing done, for these, when a rate is infinite or NaN and when a
+// sum might leave FP64's range (from_grid knows no infinity);
 // *again: a row out of reach.
 template <int G>
 __device__ __forceinline__ Gathered gather_fixed(const MechView& m, const SlotPtrs& s, const RateRange& lane_range,
@@ -714,7 +715,7 @@ __device__ __forceinline__ Gathered gather_fixed(const MechView& m, const SlotPt
   const int em = g.imax((int)lane_range.top) >> 20;
   const uint32_t least = g.umin(lane_range.low);
   const int depth = least == 0xffffffffu ? 0 : em - (int)((least + 1u) >> 20);
-  if (em == 0x7ff || depth > DEPTH_FP64) return NOT_GATHERED;
+  if (em + m.ghb >= 0x7ff || depth > DEPTH_FP64) return NOT_GATHERED;
   uint64_t* qh = reinterpret_cast<uint64_t*>(s.q);
   uint64_t* ql = reinterpret_cast<uint64_t*>(s.krc);
   constexpr int U = 4;

@@ -207,7 +207,8 @@ RK_FX void sub(Wide& a, uint64_t hi, uint64_t lo) {
   a.hi -= hi + (l < lo ? 1u : 0u);
 #endif
 }
-// a 2^(hb + em - 1149) rounded to a double (zero below the normal range)
+// a 2^(hb + em - 1149) rounded to a double (zero below the normal range; it must not
+// lie above, which em + hb < 2047 ensures)
 RK_FX double from_grid(Wide a, int em, int hb) {
   const uint64_t neg = 0ull - (a.hi >> 63);  // all ones if negative
   const uint64_t lo = (a.lo ^ neg) - neg;

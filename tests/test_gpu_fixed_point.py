@@ -212,3 +212,49 @@ def test_slow_rows_of_unburnt_mixtures_entry_by_entry(rk, name, T):
         assert np.all(np.abs(f[c, :-1] - kin.rhs(u, P)[:-1]) <= 1e-12 * sf)
         if not (mech.kind > 0).any():
             assert np.all(np.abs(jv[c, :-1] - kin.jvp(u, P, v)[:-1]) <= 1e-12 * sj)
+
+
+def _extended(kin):
+    """The oracle with its arrays in numpy's long double (15-bit exponents)."""
+    import copy
+
+    ext = copy.copy(kin)
+    for name, v in vars(kin).items():
+        if isinstance(v, np.ndarray) and v.dtype == np.float64:
+            setattr(ext, name, v.astype(np.longdouble))
+    return ext
+
+
+def test_sums_past_the_largest_double(rk):
+    """Rates just below the largest double, three quarters of them of one reaction written many
+    times: a species row past the largest double is not finite, one whose terms stay below it is
+    right.  (1e-11: as the parity tests, of the magnitudes of the row's terms.)"""
+    from oracle.kinetics import Kinetics
+
+    mech = _mech("batched")
+    mech.arrh[:, 0] *= 1e34
+    U = np.concatenate([np.random.default_rng(13).dirichlet(np.full(53, 0.5), 4), np.full((4, 1), 1400.0)], 1)
+    fastest = int(np.argmax(np.abs(Kinetics(mech).rop(U[0], 1e60))))
+    for a in (mech.rxn_sp, mech.rxn_nu, mech.arrh, mech.reversible, mech.kind):
+        a[80:] = a[fastest]
+    kin = Kinetics(mech)
+    ext = _extended(kin)
+    m = rk.mech_load(mech)
+    past = 0
+    for u in U:
+        lo, hi = 90.0, 145.0  # the pressure's exponent that puts the largest rate at ~1.5e308
+        for _ in range(40):
+            mid = 0.5 * (lo + hi)
+            over = np.max(np.abs(ext.state(u.astype(np.longdouble), np.longdouble(10.0) ** mid)["q"])) > np.longdouble("1.5e308")
+            lo, hi = (lo, mid) if over else (mid, hi)
+        p = 10.0 ** lo
+        st = ext.state(u.astype(np.longdouble), np.longdouble(p))
+        terms = np.abs(kin.nu).T @ np.abs(st["q"])
+        scale = kin.W / st["rho"] * (np.abs(kin.nu).T @ (st["m"] * (st["k"] * st["Pf"] + st["kr"] * st["Pb"])))
+        f = rk.chem_rhs(m, torch.tensor(u[None], device="cuda"), p).cpu().numpy()[0, :-1]
+        ref = ext.rhs(u.astype(np.longdouble), np.longdouble(p))[:-1]
+        far, within = np.abs(st["omega"]) > np.finfo(float).max, terms < 0.5 * np.finfo(float).max
+        past += far.sum()
+        assert not np.isfinite(f[far]).any()
+        assert np.all(np.abs(f[within] - ref[within]) <= 1e-11 * scale[within])
+    assert past >= 8
