@@ -678,12 +678,13 @@ __device__ __noinline__ void gather_rows_f32(const MechView& m, const float* q, 
   }
   g.sync();
 }
-// High words without signs of a lane's rates: the largest, and the smallest that is
-// not zero, less one (a zero wraps to the top).
+// High words without signs of a lane's rates (their last bit set where the low word is
+// not zero: only a zero gives 0): the largest, and the smallest that is not zero, less
+// one (a zero wraps to the top).
 struct RateRange {
   uint32_t top = 0u, low = 0xffffffffu;
   __device__ __forceinline__ void take(double q) {
-    const uint32_t w = (uint32_t)__double2hiint(q) & 0x7fffffffu;
+    const uint32_t w = ((uint32_t)__double2hiint(q) & 0x7fffffffu) | (__double2loint(q) != 0 ? 1u : 0u);
     top = ::max(top, w);
     low = ::min(low, w - 1u);
   }
@@ -706,16 +707,17 @@ constexpr int DEPTH_FP64 = 80;
 // to 2^-70, 71 % at 2^-80 to 2^-90) and FP64 is taken at once: its gather costs a
 // right-hand side a tenth more, forming the rates again two thirds.
 // NOT_GATHERED, with nothing done, for these, when a rate is infinite or NaN and when a
-// sum might leave FP64's range (from_grid knows no infinity);
+// sum might leave FP64's normal range (from_grid knows no infinity and no subnormals:
+// a unit of 2^-1022 or more excludes the latter);
 // *again: a row out of reach.
 template <int G>
 __device__ __forceinline__ Gathered gather_fixed(const MechView& m, const SlotPtrs& s, const RateRange& lane_range,
                                                  bool* again) {
   const Grp<G> g;
-  const int em = g.imax((int)lane_range.top) >> 20;
+  const int top = g.imax((int)lane_range.top), em = top >> 20;
   const uint32_t least = g.umin(lane_range.low);
   const int depth = least == 0xffffffffu ? 0 : em - (int)((least + 1u) >> 20);
-  if (em + m.ghb >= 0x7ff || depth > DEPTH_FP64) return NOT_GATHERED;
+  if (em + m.ghb >= 0x7ff || depth > DEPTH_FP64 || (em + m.ghb < 127 && top != 0)) return NOT_GATHERED;
   uint64_t* qh = reinterpret_cast<uint64_t*>(s.q);
   uint64_t* ql = reinterpret_cast<uint64_t*>(s.krc);
   constexpr int U = 4;

@@ -22,8 +22,10 @@
 
 #ifdef __CUDACC__
 #define RK_FX __host__ __device__ __forceinline__
+#define RK_FX_RARE static __host__ __device__ __noinline__
 #else
 #define RK_FX inline
+#define RK_FX_RARE inline
 #endif
 
 namespace rk {
@@ -151,8 +153,21 @@ RK_FX uint64_t log2e_fixed(double x) {
   return (h >> 31) ? 0ull - v : v;
 }
 
-// (m 2^(n - 63)) D rounded to a double: subnormal D and results become zero,
-// infinite and NaN D are returned as they are
+// (m 2^(n - 63)) D for a subnormal D (not zero) or a result below the normal range:
+// D normalised, the result rounded once where its last place is
+RK_FX_RARE double mul_sig_small(uint64_t m, int n, double D) {
+  const uint64_t b = bits_of(D), f = b & 0x000fffffffffffffull;
+  const int ex = (int)((b >> 52) & 0x7ffu), z = ex == 0 ? clz(f) : 11;
+  const uint64_t P0 = mulhi3(m, ex == 0 ? f << z : significand(D));
+  const bool top = (P0 >> 63) != 0;
+  const uint64_t P = top ? P0 : P0 << 1;
+  const int E = n + (ex == 0 ? 12 - z : ex) + (top ? 1 : 0);  // biased exponent, 1 or more if normal
+  const int s = E >= 1 ? 11 : 12 - E;                         // bits of P below the last place
+  const uint64_t r = s > 64 ? 0ull : ((P >> (s - 1)) + 1u) >> 1;
+  const uint64_t q = E >= 2047 ? 0x7ff0000000000000ull : (E >= 1 ? ((uint64_t)(uint32_t)(E - 1) << 52) + r : r);
+  return from_bits(q | (b & 0x8000000000000000ull));
+}
+// (m 2^(n - 63)) D rounded to a double; infinite and NaN D are returned as they are
 RK_FX double mul_sig(uint64_t m, int n, double D) {
   const uint32_t h = hi32(D);
   const int eD = (int)((h >> 20) & 0x7ffu);
@@ -162,7 +177,10 @@ RK_FX double mul_sig(uint64_t m, int n, double D) {
   const int e = n + eD + (top ? 1 : 0) - 1;
   uint64_t b = ((uint64_t)(uint32_t)e << 52) + r;
   b = e >= 2046 ? 0x7ff0000000000000ull : b;
-  b = eD == 0 || e < 0 ? 0ull : b;
+  if (eD == 0 || e < 0) {
+    if (eD != 0x7ff && (bits_of(D) << 1) != 0) return mul_sig_small(m, n, D);
+    b = 0ull;
+  }
   b |= (uint64_t)(h & 0x80000000u) << 32;
   return from_bits(eD == 0x7ff ? bits_of(D) : b);
 }

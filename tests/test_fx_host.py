@@ -128,3 +128,21 @@ def test_grid_sums_are_exact(fx, spread):
             assert abs(got - exact) <= half * (1 + Fraction(1, 2 ** 10)) + cut, (n, v)
     z = np.zeros(4)
     assert fx.t_sum(z.ctypes.data, 4, hb) == 0.0
+
+
+def test_scaled_product_below_the_normal_range(fx):
+    """Subnormal factors and results: the same relative error where the result is normal
+    (test_scaled_product), else within one unit in its last place, the smallest double."""
+    rng = np.random.default_rng(5)
+    xs, Ds = rng.uniform(-700, 300, 1500), (rng.random(1500) - 0.5) * 10.0 ** rng.uniform(-323, -100, 1500)
+    xs[:4], Ds[:4] = [0.0, -0.5, 700.0, -3.0], [5e-324, 5e-324, 5e-324, 2.2250738585072014e-308]
+    subnormal = 0
+    with localcontext() as c:
+        c.prec, c.Emin = 50, -2000
+        for x, D in zip(xs, Ds):
+            y, e = fx.t_scale(float(x), float(D)), Decimal(float(x)).exp() * Decimal(float(D))
+            place = Decimal(float(np.spacing(abs(float(e)))))
+            subnormal += 0 < abs(y) < 2.3e-308
+            assert abs(Decimal(y) - e) <= (Decimal("2.5") if abs(float(e)) >= 2.3e-308 else 1) * place, (x, D)
+    assert subnormal > 30
+    assert fx.t_scale(-700.0, -1e-300) == 0.0

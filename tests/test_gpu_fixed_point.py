@@ -258,3 +258,33 @@ def test_sums_past_the_largest_double(rk):
         assert not np.isfinite(f[far]).any()
         assert np.all(np.abs(f[within] - ref[within]) <= 1e-11 * scale[within])
     assert past >= 8
+
+
+@pytest.mark.parametrize("p", [P, 1e-100])
+def test_rates_below_the_normal_range(rk, p):
+    """Irreversible reactions with rate constants near 2^-350 and a mixture of a few species with 1e-102 of the others, or
+    all of them at a pressure of 1e-100 Pa: rates of progress among the subnormal numbers, alone
+    in their rows or all a cell has.  1e-11 of the terms' magnitudes and 64 units of the
+    smallest double a row for their own rounding."""
+    from oracle.kinetics import Kinetics
+
+    mech = _mech("batched")
+    mech.arrh[:, 0] *= 1e-40
+    mech.arrh[:, 2] = 3.8e5
+    mech.reversible[:] = 0
+    kin = Kinetics(mech)
+    ext = _extended(kin)
+    rng = np.random.default_rng(14)
+    U = np.concatenate([rng.dirichlet(np.full(53, 0.5), 8), np.full((8, 1), 300.0)], 1)
+    if p == P:
+        for u in U:
+            u[rng.permutation(53)[6:]] *= 1e-102
+    got = rk.chem_rhs(rk.mech_load(mech), torch.tensor(U, device="cuda"), p).cpu().numpy()[:, :-1]
+    below = 0
+    for g, u in zip(got, U):
+        st = ext.state(u.astype(np.longdouble), np.longdouble(p))
+        ref = kin.W / st["rho"] * st["omega"]
+        terms = np.abs(kin.nu).T @ (st["k"] * st["Pf"] + st["kr"] * st["Pb"])
+        below += np.sum((np.abs(st["omega"]) < 2.2e-308) & (np.abs(st["omega"]) > 1e-315))
+        assert np.all(np.abs(g - ref) <= kin.W / st["rho"] * (1e-11 * terms + 64 * 5e-324) + 5e-324)
+    assert below >= 8
