@@ -253,6 +253,7 @@ struct MechView {
   const double *W, *invW, *Tmid, *lo, *hi, *lnA, *bexp, *EaR, *eff, *fo, *csr_nu;
   const uint64_t *fA, *fb, *fE;  // fixed-point Arrhenius coefficients (fx.cuh)
   bool fx;                       // every coefficient fits that form
+  double fx_T_lo;                // the form's lowest temperature
   bool seg;                      // the gather's list is in shared memory
   const uint32_t* slots;
   const int32_t *meta, *csr_ptr, *csr_j;
@@ -295,6 +296,7 @@ __host__ __device__ inline MechView make_view(const unsigned char* base, const u
   m.fb = reinterpret_cast<const uint64_t*>(fbase + L.off_fb);
   m.fE = reinterpret_cast<const uint64_t*>(fbase + L.off_fE);
   m.fx = fxseg && L.fx != 0;
+  m.fx_T_lo = L.fx_T_lo;
   m.seg = fxseg && L.nr < 8191;
   m.gcsr_j = reinterpret_cast<const int32_t*>(gbase + L.off_csr_j);
   m.bexp = reinterpret_cast<const double*>(gbase + L.off_b);
@@ -1081,9 +1083,22 @@ __device__ __noinline__ Gathered rates_listed_call(const MechView& m, const Slot
   g.sync();
   return gather_listed<G>(m, s);
 }
+// The biased exponents of Y and 1/W and, where E = e^lnE < 1, log2 E, summed and offset
+// by 512 (up to two below the exponent of C and of C E with rho's added); all ones for
+// Y = 0.  |lnE| by its bits in FP32, of no account from 170.
+constexpr unsigned THIN_MIN = 512 + 3 * 1023 - 480;
+__device__ __forceinline__ unsigned scaled_exponent(double Y, double invW, double lnE) {
+  const unsigned y = (unsigned)__double2hiint(Y) & 0x7fffffffu;
+  const int hi = __double2hiint(lnE);
+  const float f = ::fminf(float_bits(__hiloint2double(hi & 0x7fffffff, __double2loint(lnE))), 170.f);
+  const unsigned low = hi < 0 ? 2u + (unsigned)(f * 1.442696f) : 0u;
+  const unsigned e = (y >> 20) + ((unsigned)__double2hiint(invW) >> 20) + 512u - low;
+  return y == 0u && __double2loint(Y) == 0 ? 0xffffffffu : e;
+}
 // Every reaction with 1/Kc from one exponential of its own: the form for cells
 // the scaled one does not hold for (a Gibbs factor past e^170, T outside
-// [150, 16000) K, coefficients outside the fixed-point range, NaN).
+// [150, 16000) K or below where some rate constant passes 2^-500, coefficients outside
+// the fixed-point range, concentrations whose scaled products would not be normal, NaN).
 template <int G, bool MIXED>
 __device__ __noinline__ void reactions_direct(const MechView& m, const SlotPtrs& s, double T, double invT, double lnT,
                                               double lnRTp, bool coop_tb, bool cache, CellScalars* cs) {
@@ -1193,6 +1208,7 @@ __device__ __forceinline__ void rhs_eval(const MechView& m, const SlotPtrs& s, c
   double S = 0.0;
   double Ds = 0.0;  // sum Y_k (dcp_k/R/dT) / W_k (caching only)
   int ghi = 0;  // max over species of the high word of |g/RT + ln(RT/p_ref)| (integer compare)
+  unsigned thin = 0xffffffffu;  // min over species present of the exponents of C and C E, less rho's
   for (int k = g.lane; k < ns; k += G) {
     const double* c = below(T, m.Tmid[k]) ? m.lo : m.hi;
     const double a1 = c[k], a2 = c[ns + k], a3 = c[2 * ns + k], a4 = c[3 * ns + k], a5 = c[4 * ns + k];
@@ -1208,6 +1224,7 @@ __device__ __forceinline__ void rhs_eval(const MechView& m, const SlotPtrs& s, c
     const double a = grt + lnRTp;  // ln E
     s.gRT[k] = a;
     ghi = max(ghi, __double2hiint(a) & 0x7fffffff);
+    thin = ::min(thin, scaled_exponent(uu[k], m.invW[k], a));
     if (cache) {
       const double dcp = fma(fma(fma(a5, t43, a4), t32, a3), t21, a2);
       Ds = fma(__dmul_rn(uu[k], dcp), m.invW[k], Ds);
@@ -1224,9 +1241,7 @@ __device__ __forceinline__ void rhs_eval(const MechView& m, const SlotPtrs& s, c
   }
   S = g.sum(S);
   ghi = g.imax(ghi);
-  // the scaled form of the reactions holds while every |g/RT + ln(RT/p_ref)| < 170
-  // (false for NaN too) and T is inside the fixed-point range
-  const bool zf = m.fx && ghi < G_OVERFLOW_HI && t_fx;
+  thin = g.umin(thin);
   // auxiliary-temperature system (Eq. chemical_source_balanced): the species
   // components are rho Y_k, so C_k = u_k / W_k and d(rho Y_k)/dt = W_k w_k:
   // the constant-volume arithmetic with unit density
@@ -1236,6 +1251,11 @@ __device__ __forceinline__ void rhs_eval(const MechView& m, const SlotPtrs& s, c
   // rho = p / (R T S), 1/rho = R T S / p, with 1/p (or 1/rho) from the caller
   const double rho = aux ? 1.0 : (cv ? -p : p * invT * invS * INV_R);
   const double invrho = aux ? 1.0 : (cv ? cs->pinv : R_GAS * T * S * cs->pinv);
+  // the scaled form of the reactions holds while every |g/RT + ln(RT/p_ref)| < 170
+  // (false for NaN too), T is inside the mechanism's fixed-point range and no C or C E
+  // that is not zero lies below 2^-480, so that their products are normal numbers
+  const bool zf = m.fx && ghi < G_OVERFLOW_HI && t_fx && __double_as_longlong(T) >= __double_as_longlong(m.fx_T_lo) &&
+                  (thin == 0xffffffffu || thin + (((unsigned)__double2hiint(rho) >> 20) & 0x7ffu) >= THIN_MIN);
   // concentrations, Gibbs factors, and (for up to MAXM pressure-dependent
   // reactions) the third-body concentrations [M]_t = sum_k eff_tk C_k
   const bool coop_tb = m.ntb > 0 && m.ntb <= MAXM;

@@ -246,7 +246,8 @@ RK_FX double from_grid(Wide a, int em, int hb) {
 // Valid for |b| <= 16, Ea/R log2 e in [-2^13, 130000), |log2 A| <= 150 and T in
 // [T_LO, T_HI): a rate constant's logarithm (between -1242 and 429) and those of two
 // Gibbs factors (each below 246 in magnitude) then stay inside (-1735, 922), which
-// neither wraps nor overflows a double.
+// neither wraps nor overflows a double.  A mechanism's own lowest temperature may be
+// higher: where its slowest rate constant passes 2^-500, so that kappa stays normal.
 constexpr double T_LO = 150.0, T_HI = 16000.0;
 struct Temp {
   uint64_t lgT, iT, c;  // log2 T 2^59, 2^70 / T, and the shifts' share

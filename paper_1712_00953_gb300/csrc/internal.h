@@ -39,8 +39,10 @@ struct MechLayout {
   int64_t off_W = 0, off_invW = 0, off_Tmid = 0, off_lo = 0, off_hi = 0, off_lo17 = 0, off_hi17 = 0;
   int64_t off_lnA = 0, off_b = 0, off_EaR = 0;  // read from global memory (d ln k/dT, Troe, the direct form)
   // fixed-point Arrhenius coefficients (fx.cuh), uint64 per reaction: log2 A 2^52, (b + 32) 2^57,
-  // (Ea/R log2 e + 2^15) 2^46; fx: every reaction's fit their ranges
+  // (Ea/R log2 e + 2^15) 2^46; fx: every reaction's fit their ranges; fx_T_lo: from this
+  // temperature up every rate constant is above 2^-500
   int32_t fx = 0;
+  double fx_T_lo = 0.0;
   int64_t off_fA = 0, off_fb = 0, off_fE = 0;
   int64_t off_eff = 0;  // [ntb][ns]
   int64_t off_fo = 0;   // [ntb][FO_STRIDE]

@@ -65,6 +65,7 @@ int64_t times_log2e(double x, int bits) {
 // the given concentration order, b and Ea/R; ok: inside their ranges.
 struct FxArrhenius {
   uint64_t A = 0, b = 0, E = 0;
+  double T_lo = fx::T_LO;  // from here up the rate constant is above 2^-500 (log2 T in [7.22, 13.97])
   bool ok = false;
 };
 FxArrhenius fx_arrhenius(double A, int order, double b, double EaR) {
@@ -80,6 +81,7 @@ FxArrhenius fx_arrhenius(double A, int order, double b, double EaR) {
   f.A = (uint64_t)lg;
   f.b = (uint64_t)((int64_t)llrint(ldexp(b, 57)) + ((int64_t)32 << 57));
   f.E = (uint64_t)times_log2e(EaR, 45) * 2 + ((uint64_t)1 << 61);
+  f.T_lo = std::max(fx::T_LO, El / (500.0 + ldexp((double)lg, -52) + std::min(7.22 * b, 13.97 * b)));
   return f;
 }
 
@@ -447,6 +449,7 @@ bool pack_mechanism(const void* vdesc, HostMech* out, std::string* err) {
     D(L.off_EaR)[r] = ar[2] / R_GAS;
     const FxArrhenius f = fx_arrhenius(ar[0], order, ar[1], ar[2] / R_GAS);
     fx = fx && f.ok;
+    L.fx_T_lo = std::max(L.fx_T_lo, f.T_lo);
     X(L.off_fA)[r] = f.A;
     X(L.off_fb)[r] = f.b;
     X(L.off_fE)[r] = f.E;

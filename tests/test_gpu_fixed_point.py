@@ -174,7 +174,7 @@ def _terms(kin, u, v):
     dC = st["rho"] / W * np.abs(v[:ns]) + st["C"] * drr
 
     def dprod(n):  # sum over factors of |dC| times the others
-        out = np.zeros(len(n))
+        out = np.zeros(len(n), dtype=dC.dtype)
         for j, row in enumerate(n):
             ks = [k for k in np.flatnonzero(row) for _ in range(int(row[k]))]
             for i, k in enumerate(ks):
@@ -288,3 +288,43 @@ def test_rates_below_the_normal_range(rk, p):
         below += np.sum((np.abs(st["omega"]) < 2.2e-308) & (np.abs(st["omega"]) > 1e-315))
         assert np.all(np.abs(g - ref) <= kin.W / st["rho"] * (1e-11 * terms + 64 * 5e-324) + 5e-324)
     assert below >= 8
+
+
+@pytest.mark.parametrize("case", ["cold", "thin"])
+def test_small_rate_constants_and_fractions_with_extreme_gibbs_factors(rk, case):
+    """An element-additive enthalpy shift carries g/RT to +-160.  cold: rate constants of
+    ~2^-800, so that k / (E E) is below the normal range where k C C is not.  thin: fractions
+    of 1e-120, so that the products of C E are.  Every entry within 1e-12 of its terms'
+    magnitudes times twice the exponents of the mixtures above (E of up to 160: 2e-12 with
+    g/RT's own rounding, five operations on terms of up to ~200)."""
+    from oracle.kinetics import Kinetics
+
+    mech = _mech("batched")
+    T = 160.0 if case == "cold" else 300.0
+    atoms = mech.elem.sum(1)
+    kin0 = Kinetics(mech)
+    _, h, s, _ = kin0.thermo(T)
+    c = (1.0 if case == "cold" else -1.0) * min((160.0 - abs(x)) * T / n for x, n in zip(h - s + np.log(T / 1.2e4), atoms))
+    mech.nasa[:, 8] += c * atoms
+    mech.nasa[:, 15] += c * atoms
+    mech.reversible[:] = 0
+    rng = np.random.default_rng(15)
+    U = np.concatenate([rng.dirichlet(np.full(53, 0.5), 8), np.full((8, 1), T)], 1)
+    if case == "cold":
+        mech.arrh[:, 0] *= 1e-40
+        mech.arrh[:, 2] = 6.8e5
+    else:
+        for u in U:
+            u[rng.permutation(53)[6:]] *= 1e-120
+    assert rk.mech_validate(mech) == ""
+    kin = Kinetics(mech)
+    ext = _extended(kin)
+    V = rng.normal(size=U.shape) * U
+    m = rk.mech_load(mech)
+    Ug = torch.tensor(U, device="cuda")
+    f = rk.chem_rhs(m, Ug, P).cpu().numpy()
+    jv = rk.chem_jvp(m, Ug, torch.tensor(V, device="cuda"), P).cpu().numpy()
+    for g, j, u, v in zip(f, jv, U.astype(np.longdouble), V.astype(np.longdouble)):
+        sf, sj = _terms(ext, u, v)
+        assert np.all(np.abs(g[:-1] - ext.rhs(u, np.longdouble(P))[:-1]) <= 2e-12 * sf)
+        assert np.all(np.abs(j[:-1] - ext.jvp(u, np.longdouble(P), v)[:-1]) <= 2e-12 * sj)
