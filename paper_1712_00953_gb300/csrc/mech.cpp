@@ -50,6 +50,24 @@ bool close_rel(double x, double y, double tol) {
   return fabs(x - y) <= tol * std::max(1.0, std::max(fabs(x), fabs(y)));
 }
 
+// Items collected with a key below n each, grouped by key in the order they came.
+template <typename T>
+struct Grouped {
+  std::vector<std::pair<int, T>> in;
+  std::vector<T> item;
+  std::vector<int> ptr;
+  void add(int key, T x) { in.push_back({key, x}); }
+  void group(int n) {
+    ptr.assign(n + 1, 0);
+    for (auto& e : in) ++ptr[e.first + 1];
+    for (int k = 0; k < n; ++k) ptr[k + 1] += ptr[k];
+    item.resize(in.size());
+    std::vector<int> at(ptr.begin(), ptr.end() - 1);
+    for (auto& e : in) item[at[e.first]++] = e.second;
+  }
+  int size(int k) const { return ptr[k + 1] - ptr[k]; }
+};
+
 // x log2(e) scaled by 2^bits, rounded, from the 64-bit log2(e): x's 53-bit
 // significand times it is exact in 128 bits.  |x| log2(e) 2^bits < 2^63.
 int64_t times_log2e(double x, int bits) {
@@ -172,42 +190,41 @@ bool pack_mechanism(const void* vdesc, HostMech* out, std::string* err) {
       if (d->kind[j] == want) perm.push_back(j);
 
   // ---- species-major stoichiometry list (net coefficients, packed order)
-  std::vector<std::vector<std::pair<int, double>>> rows(ns);
+  Grouped<std::pair<int, double>> rows;
+  rows.in.reserve(4 * (size_t)nr);
   for (int r = 0; r < nr; ++r) {
     const int j = perm[r];
-    double net[RK_MAX_SPECIES + 1];
-    int touched[4];
-    int nt = 0;
+    int touched[4], net[4], nt = 0;
     for (int s = 0; s < 4; ++s) {
       const int k = d->rxn_sp[4 * (size_t)j + s];
       if (k < 0) continue;
-      bool seen = false;
-      for (int t = 0; t < nt; ++t) seen |= (touched[t] == k);
-      if (!seen) {
-        touched[nt++] = k;
-        net[k] = 0.0;
+      int t = 0;
+      while (t < nt && touched[t] != k) ++t;
+      if (t == nt) {
+        touched[nt] = k;
+        net[nt++] = 0;
       }
-      net[k] += d->rxn_nu[4 * (size_t)j + s];
+      net[t] += d->rxn_nu[4 * (size_t)j + s];
     }
     for (int t = 0; t < nt; ++t)
-      if (net[touched[t]] != 0.0) rows[touched[t]].push_back({r, net[touched[t]]});
+      if (net[t] != 0) rows.add(touched[t], {r, (double)net[t]});
   }
-  int nnz = 0;
-  for (auto& row : rows) nnz += (int)row.size();
+  rows.group(ns);
+  const int nnz = (int)rows.item.size();
 
   // ---- pieces of the list for the gather w = nu^T q: every species row is cut
   // into near-equal pieces of at most Lp entries; one lane sums one piece, so
   // a warp's loop runs ceil(npiece/32) x Lp times instead of the longest row.
   // Lp minimises that count plus the adds that join a species' pieces.
   int maxdeg = 1;
-  for (auto& row : rows) maxdeg = std::max(maxdeg, (int)row.size());
+  for (int k = 0; k < ns; ++k) maxdeg = std::max(maxdeg, rows.size(k));
   int Lp = maxdeg;
   {
     long best = -1;
     for (int cand = 1; cand <= maxdeg; ++cand) {
       int P = 0, maxp = 1;
-      for (auto& row : rows) {
-        const int pk = std::max(1, ((int)row.size() + cand - 1) / cand);
+      for (int k = 0; k < ns; ++k) {
+        const int pk = std::max(1, (rows.size(k) + cand - 1) / cand);
         P += pk;
         maxp = std::max(maxp, pk);
       }
@@ -223,7 +240,7 @@ bool pack_mechanism(const void* vdesc, HostMech* out, std::string* err) {
     int pos = 0;
     for (int k = 0; k < ns; ++k) {
       spec_piece.push_back((int32_t)piece_ptr.size());
-      const int deg = (int)rows[k].size();
+      const int deg = rows.size(k);
       const int pk = std::max(1, (deg + Lp - 1) / Lp);
       for (int i = 0; i < pk; ++i) piece_ptr.push_back(pos + (int)((long)deg * i / pk));
       pos += deg;
@@ -237,18 +254,24 @@ bool pack_mechanism(const void* vdesc, HostMech* out, std::string* err) {
   // pieces of at most glen entries; one lane sums one piece.  glen minimises the
   // group's steps (about 9 instructions an entry, 12 a piece, 10 for each piece a
   // species adds up).
-  std::vector<std::vector<int>> signed_rows(2 * (size_t)ns);
+  std::vector<int> signed_list;  // species k: its gains, then its losses
+  std::vector<int> signed_ptr(1, 0);
+  signed_list.reserve(2 * (size_t)nnz);
   int most = 1;  // largest sum of |nu| in a row
   for (int k = 0; k < ns; ++k) {
-    for (auto& e : rows[k])
-      for (int t = 0; t < (int)fabs(e.second); ++t) signed_rows[2 * k + (e.second < 0.0)].push_back(e.first);
-    most = std::max(most, (int)(signed_rows[2 * k].size() + signed_rows[2 * k + 1].size()));
+    for (int loss = 0; loss < 2; ++loss) {
+      for (int i = rows.ptr[k]; i < rows.ptr[k + 1]; ++i)
+        if ((rows.item[i].second < 0.0) == (loss == 1))
+          for (int t = (int)fabs(rows.item[i].second); t > 0; --t) signed_list.push_back(rows.item[i].first);
+      signed_ptr.push_back((int)signed_list.size());
+    }
+    most = std::max(most, signed_ptr[2 * k + 2] - signed_ptr[2 * k]);
   }
-  auto pieces_of = [](size_t n, int len) { return (int)((n + len - 1) / len); };
+  auto row_size = [&](int r) { return signed_ptr[r + 1] - signed_ptr[r]; };
+  auto pieces_of = [](int n, int len) { return (n + len - 1) / len; };
   // Few entries: in FP64, 64 cycles for each that a lane adds; otherwise in fixed
   // point, in batches of eight entries.
-  int entries = 0;
-  for (auto& row : signed_rows) entries += (int)row.size();
+  const int entries = (int)signed_list.size();
   const bool gfix = entries >= GFIX_MIN_ENTRIES && nr < 8191 && nr >= ns;  // (the sums take the rates' place)
   const int step = gfix ? 8 : 1;
   int glen = 1;
@@ -257,7 +280,7 @@ bool pack_mechanism(const void* vdesc, HostMech* out, std::string* err) {
     for (int cand = step; cand < most + step; cand += step) {
       int P = 0, maxp = 0;
       for (int k = 0; k < ns; ++k) {
-        const int pk = pieces_of(signed_rows[2 * k].size(), cand) + pieces_of(signed_rows[2 * k + 1].size(), cand);
+        const int pk = pieces_of(row_size(2 * k), cand) + pieces_of(row_size(2 * k + 1), cand);
         P += pk;
         maxp = std::max(maxp, pk);
       }
@@ -268,19 +291,25 @@ bool pack_mechanism(const void* vdesc, HostMech* out, std::string* err) {
       }
     }
   }
-  std::vector<std::vector<int>> gpieces;
+  struct Piece {
+    int* at;
+    int n;
+  };
+  std::vector<Piece> gpieces;
   std::vector<int32_t> gspec;
   for (int r = 0; r < 2 * ns; ++r) {
     gspec.push_back((int32_t)gpieces.size());
-    const auto& row = signed_rows[r];
-    const int pk = pieces_of(row.size(), glen);
-    for (int i = 0; i < pk; ++i)
-      gpieces.emplace_back(row.begin() + row.size() * i / pk, row.begin() + row.size() * (i + 1) / pk);
+    const int64_t n = row_size(r);
+    const int pk = pieces_of((int)n, glen);
+    for (int i = 0; i < pk; ++i) {
+      const int a = (int)(n * i / pk), b = (int)(n * (i + 1) / pk);
+      gpieces.push_back({signed_list.data() + signed_ptr[r] + a, b - a});
+    }
   }
   gspec.push_back((int32_t)gpieces.size());
   const int gnpp = std::max(32, ((int)gpieces.size() + 31) / 32 * 32);
-  gpieces.resize(gnpp);
-  // The sums are exact, so a piece's entries may come in any order: at each step the
+  gpieces.resize(gnpp, {nullptr, 0});
+  // A piece's sum does not depend on the order of its entries: at each step the
   // 16 lanes of a half-warp take entries of different 8-byte shared-memory banks
   // (index mod 16) where they can.
   const int gbat = (glen + 7) / 8;
@@ -293,8 +322,8 @@ bool pack_mechanism(const void* vdesc, HostMech* out, std::string* err) {
         for (int& b : bank) b = -1;
         for (int u = 0; u < 16; ++u) {
           const int p = p0 + (u + i) % 16;  // the lane that chooses first goes round
-          auto& l = gpieces[p];
-          const int n = (int)l.size();
+          int* const l = gpieces[p].at;
+          const int n = gpieces[p].n;
           int at = n;
           for (int t = done[p]; t < n; ++t)
             if (bank[l[t] & 15] < 0 || bank[l[t] & 15] == l[t]) {
@@ -366,7 +395,8 @@ bool pack_mechanism(const void* vdesc, HostMech* out, std::string* err) {
   L.off_csr_ptr = take(4 * (int64_t)(ns + 1));
   L.off_perm = take(4 * (int64_t)nr);
   // reaction slots per species (filled below from the packed slots)
-  std::vector<std::vector<int32_t>> roles(ns);
+  Grouped<int32_t> roles;
+  roles.in.reserve(4 * (size_t)nr);
   for (int r = 0; r < nr; ++r) {
     const int j = perm[r];
     // the same expansion as the packed slots below: entries 0, 1 reactants, 2, 3 products
@@ -380,9 +410,10 @@ bool pack_mechanism(const void* vdesc, HostMech* out, std::string* err) {
       }
     }
     for (int role = 0; role < 4; ++role)
-      if (sl[role] < ns) roles[sl[role]].push_back(r << 2 | role);
+      if (sl[role] < ns) roles.add(sl[role], r << 2 | role);
   }
-  for (auto& v : roles) L.nrole += (int32_t)v.size();
+  roles.group(ns);
+  L.nrole = (int32_t)roles.item.size();
   L.off_role_ptr = take(4 * (int64_t)(ns + 1));
   L.off_role = take(4 * (int64_t)(L.nrole > 0 ? L.nrole : 1));
   L.off_lo = take(8 * 7 * (int64_t)ns);
@@ -475,16 +506,11 @@ bool pack_mechanism(const void* vdesc, HostMech* out, std::string* err) {
     I(L.off_meta)[r] = kind | (rev << 2) | ((dnu + 4) << 4) | (slot << 8);
   }
   L.fx = fx && nr < 8191 ? 1 : 0;
-  int pos = 0;
-  for (int k = 0; k < ns; ++k) {
-    I(L.off_csr_ptr)[k] = pos;
-    for (auto& e : rows[k]) {
-      I(L.off_csr_j)[pos] = e.first;
-      D(L.off_csr_nu)[pos] = e.second;
-      ++pos;
-    }
+  for (int k = 0; k <= ns; ++k) I(L.off_csr_ptr)[k] = rows.ptr[k];
+  for (int i = 0; i < nnz; ++i) {
+    I(L.off_csr_j)[i] = rows.item[i].first;
+    D(L.off_csr_nu)[i] = rows.item[i].second;
   }
-  I(L.off_csr_ptr)[ns] = pos;
   if (!gidx.empty()) memcpy(buf.data() + L.off_gidx, gidx.data(), 2 * gidx.size());
   for (size_t i = 0; i < gspec.size(); ++i) I(L.off_gspec)[i] = gspec[i];
   for (int p = 0; p <= npiece; ++p) I(L.off_piece_ptr)[p] = piece_ptr[p];
@@ -501,42 +527,24 @@ bool pack_mechanism(const void* vdesc, HostMech* out, std::string* err) {
   for (int i = 0; i < L.ntb * ns; ++i) F(L.off_efff)[i] = (float)D(L.off_eff)[i];
   for (int i = 0; i < nnz; ++i) F(L.off_csr_nuf)[i] = (float)D(L.off_csr_nu)[i];
   for (int r = 0; r < nr; ++r) I(L.off_perm)[r] = perm[r];
-  {
-    int pos = 0;
-    for (int k = 0; k < ns; ++k) {
-      I(L.off_role_ptr)[k] = pos;
-      for (int32_t e : roles[k]) I(L.off_role)[pos++] = e;
-    }
-    I(L.off_role_ptr)[ns] = pos;
-  }
+  for (int k = 0; k <= ns; ++k) I(L.off_role_ptr)[k] = roles.ptr[k];
+  for (int i = 0; i < L.nrole; ++i) I(L.off_role)[i] = roles.item[i];
   // nu^T tiles for the tensor-core gather: net coefficients (small integers,
   // exact in BF16) placed in each lane's A-operand registers of mma.m16n8k16
   // (register 0: row g, columns 2t, 2t+1; 1: row g+8; 2: row g, columns
   // 2t+8, 2t+9; 3: row g+8; g = lane / 4, t = lane % 4; the lower column in
   // the lower 16 bits)
   {
-    std::vector<double> A((size_t)ns * nr, 0.0);
+    uint16_t* T = reinterpret_cast<uint16_t*>(buf.data() + L.off_nuT);
     for (int k = 0; k < ns; ++k)
-      for (auto& e : rows[k]) A[(size_t)k * nr + e.first] = e.second;
-    auto a = [&](int k, int r) { return (k < ns && r < nr) ? A[(size_t)k * nr + r] : 0.0; };
-    auto bf16 = [](double x) {
-      const float f = (float)x;  // a small integer: its BF16 is the float's upper half, exactly
-      uint32_t u;
-      memcpy(&u, &f, 4);
-      return u >> 16;
-    };
-    auto pack = [&](int k, int r) { return bf16(a(k, r)) | (bf16(a(k, r + 1)) << 16); };
-    uint32_t* T = U(L.off_nuT);
-    for (int st = 0; st < L.nst; ++st)
-      for (int rt = 0; rt < L.nrt; ++rt)
-        for (int l = 0; l < 32; ++l) {
-          const int g = l >> 2, t = l & 3, k0 = 16 * st + g, r0 = 16 * rt + 2 * t;
-          uint32_t* R = T + 4 * ((size_t)(st * L.nrt + rt) * 32 + l);
-          R[0] = pack(k0, r0);
-          R[1] = pack(k0 + 8, r0);
-          R[2] = pack(k0, r0 + 8);
-          R[3] = pack(k0 + 8, r0 + 8);
-        }
+      for (int i = rows.ptr[k]; i < rows.ptr[k + 1]; ++i) {
+        const auto& e = rows.item[i];
+        const int g = k & 7, c = e.first & 15, t = (c & 7) >> 1, reg = ((k >> 3) & 1) + 2 * (c >> 3);
+        const float f = (float)e.second;  // a small integer: its BF16 is the float's upper half, exactly
+        uint32_t u;
+        memcpy(&u, &f, 4);
+        T[8 * ((size_t)((k >> 4) * L.nrt + (e.first >> 4)) * 32 + 4 * g + t) + 2 * reg + (c & 1)] = (uint16_t)(u >> 16);
+      }
   }
 
   out->L = L;
