@@ -1951,11 +1951,11 @@ __device__ __forceinline__ void jvp_eval_f32x(const MechView& m, const SlotPtrs&
   float* fpart = reinterpret_cast<float*>(s.part);
   auto f = [](double x) { return __double2float_rn(x); };
   const float vT = f(v[ns]);
-  const float T = f(cs.T), invT = f(cs.invT);
+  const float T = f(cs.T), vTT = f(v[ns] * cs.invT);  // vT / T, rounded once
   float a = 0.f;
   for (int k = g.lane; k < ns; k += G) a = fmaf(f(v[k]), f(m.invW[k]), a);
   a = g.sum(a);
-  const float drr = cs.cv ? 0.f : -fmaf(a, f(cs.invS), vT * invT);
+  const float drr = cs.cv ? 0.f : -fmaf(a, f(cs.invS), vTT);
   const bool coop_tb = m.ntb > 0 && m.ntb <= MAXM;
   float mp[MAXM];
 #pragma unroll
@@ -1984,7 +1984,7 @@ __device__ __forceinline__ void jvp_eval_f32x(const MechView& m, const SlotPtrs&
     const float dPf = fmaf(fdC[ra], Crb, Cra * fdC[rb]);
     const float dPb = fmaf(fdC[pa], Cpb, Cpa * fdC[pb]);
     const float k = s.xk[j], kr = s.xkr[j];
-    float dq = fmaf(s.xqT[j], vT * invT, fmaf(k, dPf, -kr * dPb));  // xqT: T d q/dT
+    float dq = fmaf(s.xqT[j], vTT, fmaf(k, dPf, -kr * dPb));  // xqT: T d q/dT
     if (kind != 0) {
       const int slot = meta >> 8;
       const double* t = s.tb + 4 * slot;

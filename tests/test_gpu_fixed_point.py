@@ -328,3 +328,21 @@ def test_small_rate_constants_and_fractions_with_extreme_gibbs_factors(rk, case)
         sf, sj = _terms(ext, u, v)
         assert np.all(np.abs(g[:-1] - ext.rhs(u, np.longdouble(P))[:-1]) <= 2e-12 * sf)
         assert np.all(np.abs(j[:-1] - ext.jvp(u, np.longdouble(P), v)[:-1]) <= 2e-12 * sj)
+
+
+def test_temperature_direction_of_the_fp32_product(rk):
+    """J v of precision 6 along T: every reaction and the density take the same FP32 factor
+    vT / T, so its rounding scales the whole row, the median over the species being hardly
+    touched by their own.  Rounded once it is off by 0.36 x 2^-24 on average, as a product of
+    rounded factors by 0.58; the line is between the two."""
+    mech = _mech("batched")
+    m = rk.mech_load(mech)
+    n = 4000
+    rng = np.random.default_rng(16)
+    U = np.concatenate([rng.dirichlet(np.full(53, 0.5), n), rng.uniform(900.0, 2500.0, (n, 1))], 1)
+    V = np.zeros_like(U)
+    V[:, -1] = rng.uniform(0.5, 1.0, n)
+    Ug, Vg = torch.tensor(U, device="cuda"), torch.tensor(V, device="cuda")
+    a, b = (rk.chem_jvp(m, Ug, Vg, P, mode=k).cpu().numpy()[:, :-1] for k in (0, 5))
+    factor = np.median(b / a - 1.0, axis=1)
+    assert np.mean(np.abs(factor)) < 0.47 * 2.0 ** -24
