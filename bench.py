@@ -226,6 +226,43 @@ class ClockSampler:
         return {"sm_mhz": statistics.median(sm), "sm_max_mhz": mx, "reasons": sorted(reasons), "samples": len(sm)}
 
 
+# ---------------------------------------------------------------- the printed line
+LINE_LIMIT = 2400  # characters: readers that keep the end of the output see the whole line
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+             "vs_baseline", "dtype", "data", "gpu_launches", "cells_failed", "attempts_per_cell_step", "attempts_per_s",
+             "e2e", "clocks")
+LINE_PARTS = {
+    "config": ("workload", "cells_per_gpu", "krylov_dim", "precision", "lanes_per_cell", "l2", "parallelism"),
+    "roofline": ("bound", "achieved", "peak", "unit", "frac", "traffic", "kernel"),
+    "accuracy": ("cells", "max_abs_dY", "max_abs_dT_K", "within_1e-8_plus_1e-6Y_and_1e-6K"),
+    "cpu_baseline": ("value", "cores"),
+}
+
+
+def compact_line(line, details):
+    """The one printed line of a full record: every key that names the measurement, and of the
+    other workloads' blocks their values; `details` is the file that holds the rest."""
+    def short(x):
+        if isinstance(x, dict):
+            return {k: short(v) for k, v in x.items()}
+        return float(f"{x:.7g}") if isinstance(x, float) else x
+
+    def values(block):
+        if "value" in block:
+            return short(block["value"])
+        return {k: values(v) for k, v in block.items() if isinstance(v, dict)}
+
+    out = {k: line[k] for k in LINE_KEYS if k in line}
+    for part, keys in LINE_PARTS.items():
+        if part in line:
+            out[part] = {k: line[part][k] for k in keys if k in line[part]}
+    out = short(out)
+    if "configs" in line:
+        out["configs"] = values(line["configs"])
+    out["details"] = details
+    return out
+
+
 # ---------------------------------------------------------------- oracle legs
 def golden_cells(n, count, offset=1):
     """count distinct cell indices spread over [0, n) (golden-ratio sequence)."""
@@ -1207,7 +1244,9 @@ def run_ours(args, rank, world, local_rank):
         line["configs"] = configs
         line["gpu_launches"] += (configs["small"]["gpu_launches"] + configs["flame1d"]["gpu_launches"]
                                  + sum(v["gpu_launches"] for k, v in mixed.items() if k != "note"))
-    print(json.dumps(line))
+    with open(args.details, "w") as f:
+        json.dump(line, f, indent=1)
+    print(json.dumps(compact_line(line, args.details)))
     return 0
 
 
@@ -1218,6 +1257,7 @@ def main():
     ap.add_argument("--warmup", type=int, default=3)
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--headline-only", action="store_true", help="skip the other workloads' blocks")
+    ap.add_argument("--details", default="bench_details.json", help="file for the full record; the line keeps its values")
     ap.add_argument("--cpu-cells", type=int, default=64, help="C-oracle cells per host thread for the CPU baselines")
     ap.add_argument("--ref-cells", type=int, default=32, help="C-oracle cells per host thread per reference step")
     ap.add_argument("--e2e-steps", type=int, default=2, help="steps of the end-to-end measurement (headline)")

@@ -107,3 +107,29 @@ def test_adjoint_flop_model_is_linear_in_its_passes():
     one_rhs = f4["rhs"] + bench.EXP_FLOPS * f4["rhs_exp"]
     assert 2.5 * f4["rhs"] < dual_pair < 10 * one_rhs
     assert a4 == pytest.approx(753398.0, rel=1e-12)  # 0.75 MFLOP per cell-step, as quoted
+
+
+def test_printed_line_is_short_and_names_the_measurement():
+    """The full record (per-cell lists, notes, a block per workload and level) runs to tens of
+    thousands of characters; the line keeps the keys that name the measurement and fits."""
+    import json
+
+    v = 123456.78901234567
+    block = {"value": v, "unit": "cell-steps/s", "note": "x" * 300, "roofline": {"frac": 0.5}, "cells": [v] * 100}
+    levels = {k: block for k in ("fp64", "mixed", "mixed-fp32jv", "mixed-df", "tensor", "exp32", "fp32jv")}
+    line = {k: v for k in bench.LINE_KEYS}
+    line.update({"metric": "cell-steps/s", "unit": "cell-steps/s", "data": "synthetic (seeded)", "dtype": "f64",
+                 "e2e": {"value": v, "unit": "cell-steps/s", "h2d_bytes_per_step": 461373440, "d2h_bytes_per_step": 461373440,
+                         "steps": 2, "result_matches_device_run_bitwise": True},
+                 "clocks": {"sm_mhz": 2070.0, "sm_max_mhz": 2070.0, "reasons": ["sw_power_cap"], "samples": 100}})
+    for part, keys in bench.LINE_PARTS.items():
+        line[part] = {**{k: v for k in keys}, "per_species": [v] * 500}
+    line["config"]["workload"] = "w" * 220
+    line["config"]["l2"] = "l" * 90
+    line["configs"] = {"small": block, "flame1d": block, "mixed": {**levels, "note": "y" * 200}, "mixed_batched": levels,
+                       "adjoint": block}
+    assert len(json.dumps(line)) > 20000
+    out = bench.compact_line(line, "bench_details.json")
+    assert len(json.dumps(out)) <= bench.LINE_LIMIT
+    assert set(bench.LINE_KEYS) | set(bench.LINE_PARTS) <= set(out)
+    assert out["configs"]["mixed"]["tensor"] == pytest.approx(v, rel=1e-6) and out["e2e"]["d2h_bytes_per_step"] == 461373440
