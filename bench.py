@@ -1244,9 +1244,13 @@ def run_ours(args, rank, world, local_rank):
         line["configs"] = configs
         line["gpu_launches"] += (configs["small"]["gpu_launches"] + configs["flame1d"]["gpu_launches"]
                                  + sum(v["gpu_launches"] for k, v in mixed.items() if k != "note"))
-    with open(args.details, "w") as f:
-        json.dump(line, f, indent=1)
-    print(json.dumps(compact_line(line, args.details)))
+    details = args.details
+    try:
+        with open(details, "w") as f:
+            json.dump(line, f, indent=1)
+    except OSError as e:
+        details = f"not written: {e.strerror}"
+    print(json.dumps(compact_line(line, details)))
     return 0
 
 

@@ -123,7 +123,10 @@ int rk_mech_info(const rk_mech* mech, int32_t* n_species, int32_t* n_reactions,
  * reactor source: dY_k/dt = W_k w_k / rho, dT/dt = -sum_k h_k w_k / (rho c_p),
  * w = nu^T q the net molar production rates (Eq. cv_reactor read at constant
  * pressure).  Y, src, dYdt: device [ncell x N]; src may be NULL (zero source).
- * dYdt must not alias Y. */
+ * dYdt must not alias Y.  Every entry has FP64's accuracy in its own terms, those of
+ * slow species in cold mixtures too; a cell that is no state (all mass fractions zero,
+ * T = 0, NaN) gives NaN.  For mechanisms of some 2000 reactions, whose coefficients fit
+ * in shared memory here and not in the integrator, the two agree to rounding, not bitwise. */
 int rk_chem_rhs(const rk_mech* mech, const double* Y, const double* src, double p,
                 double* dYdt, int64_t ncell, void* stream);
 
@@ -138,7 +141,8 @@ int rk_chem_rhs(const rk_mech* mech, const double* Y, const double* src, double 
  * arithmetic on the FP32 copies of its caches that the caching right-hand
  * side writes at precision level 6 (that level's J v).  Each mode computes
  * exactly what the integrator's J v at that level computes.  All arrays
- * device [ncell x N]; RK_E_INVALID_ARGUMENT for a mode outside 0..5. */
+ * device [ncell x N]; RK_E_INVALID_ARGUMENT for a mode outside 0..5.  V is multiplied
+ * by Gibbs factors between e^-170 and e^170: magnitudes within 1e-200 .. 1e200. */
 int rk_chem_jvp(const rk_mech* mech, const double* Y, const double* V, double p, double* JV,
                 int64_t ncell, int32_t mode, void* stream);
 

@@ -483,11 +483,6 @@ struct Grp {
     for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o, G);
     return v;
   }
-  __device__ __forceinline__ double max(double v) const {
-#pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(mask, v, o, G));
-    return v;
-  }
   __device__ __forceinline__ unsigned umin(unsigned v) const {
     if constexpr (G == 32) return __reduce_min_sync(0xffffffffu, v);
 #pragma unroll
@@ -3153,7 +3148,7 @@ inline int64_t segment_bytes(const MechLayout& L, int64_t rest) {
 // Shared memory that precision 4 counts beside its tiles when it decides whether
 // it can run: the mechanism arrays and one cell's slot of its first layout.  The
 // present layout needs less; the limit on the mechanism's size stays where callers
-// know it.
+// know it, and what was refused stays refused.
 inline int64_t tensor_core_bytes(const MechLayout& L, int M, int nx) {
   auto even = [](int64_t n) { return (n + 1) & ~int64_t(1); };
   auto al = [](int64_t b) { return (b + 15) & ~int64_t(15); };

@@ -27,6 +27,8 @@ def main():
     ln2 = Decimal(2).ln()
     lines = ["// Generated by gen_exp_table.py: RK_EXP2_TABLE_VALUES[j] = 2^(j/256) rounded to binary64;",
              "// RK_LOG_INV_C_VALUES[j] = 1/(1 + (j + 1/2)/128) rounded, RK_LOG_LN_C_VALUES[j] = -ln of it.",
+             "// The kernels read the logarithm's tables; their exponential is on 64-bit integers (fx_table.h),",
+             "// the binary64 one here serves the host check of the method.",
              "#pragma once", f"#define RK_EXP2_TABLE_N {N}", f"#define RK_LOG_TABLE_N {NL}",
              "#define RK_EXP2_TABLE_VALUES \\"]
     for j in range(N):

@@ -388,7 +388,7 @@ int integrate_impl(const rk_mech* mech, double* Y, const double* src, double* h_
     size_t smem_max = 0;
     if (tc && (rc = device_props(&n_sm, &smem_max))) return rc;
     if (tc && tensor_core_bytes(L, Meff, nx) + 64 > (int64_t)smem_max)
-      return set_error(RK_E_UNSUPPORTED, "mechanism, nu^T tiles and one cell's work arrays exceed shared memory");
+      return set_error(RK_E_UNSUPPORTED, "precision 4: mechanism and nu^T tiles beyond its limit on shared memory");
   }
   P.qstride = queue_stride(ncell);
   P.order = nullptr;
