@@ -23,7 +23,7 @@
 //
 // Arithmetic.  FP64 accuracy throughout, on two kinds of pipe: a warp's FP64
 // instruction holds its sub-partition's FP64 unit for 64 cycles, an integer one
-// its pipe for 2 to 4, so what can be formed from 64-bit integers without loss is
+// its pipe for 2 to 4, so what 64-bit integers carry to the last FP64 bit is
 // (fx.cuh), and FP64 instructions are kept for the rest.  Restatements that differ
 // from a literal transcription of the kinetics while computing the same quantities:
 //  * with E_k = exp(g_k/RT) (RT/p_ref) and z_k = C_k E_k, 1/Kc is a product of E
